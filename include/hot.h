@@ -50,27 +50,26 @@ typedef enum {
  * |V_m| within 1e-4 relative after one GSW iteration, e and u within 1e-3 after a run, 8-bit
  * output equal except within 1e-4 rad of a level boundary.  HOT_PREC_ACCURATE and
  * HOT_PREC_SEPARABLE meet these bounds on every tested case, up to HOT_MAX_TRAPS traps.
- * HOT_PREC_FAST and HOT_PREC_TENSOR meet them on every tested case except strongly cancelling
- * back-projections: 4096 traps on a 160 x 120 SLM, whose first weight update spreads the weights
- * over a factor ~400, so that the superposition cancels at some pixels and amplifies each term's
- * error.  There the |V_m| error after one iteration is bounded by 2e-4 in the fast mode (1.2e-4
- * measured; accurate 7.6e-5) and by 5e-4 in the tensor mode (3.3e-4 measured).  Measured
- * elsewhere: 512 x 512 px with 100 traps, 2.5e-6 fast, 2.4e-6 accurate (the one-exponential step,
- * hot_set_once; the direct kernels: 4.1e-6, 6.0e-6); 1920 x 1152 px with 1000 traps, 8.8e-6 fast. */
+ * The direct kernels of HOT_PREC_FAST (hot_set_once) and HOT_PREC_TENSOR meet them on every tested
+ * case except strongly cancelling back-projections: 4096 traps on a 160 x 120 SLM, whose first
+ * weight update spreads the weights over a factor ~400, so that the superposition cancels at some
+ * pixels and amplifies each term's error.  There the |V_m| error after one iteration is bounded by
+ * 2e-4 in the fast mode's direct kernels (1.2e-4 measured; accurate 7.6e-5) and by 5e-4 in the
+ * tensor mode (3.3e-4 measured). */
 typedef enum {
-  HOT_PREC_ACCURATE = 0, /* sincospif on the exactly reduced phase (FP32, ~1 ulp) */
-  HOT_PREC_FAST = 1,     /* the direct evaluation on the special-function unit: sin.approx /
-                             cos.approx of the reduced phase (arguments pre-scaled by 1 + 8.17e-8
-                             against the unit's mean argument shrink); the direct step's forward
-                             field rotates the phases of each pixel sub-tile by a fixed
-                             pseudo-random angle and its sums back, so that the unit's systematic
-                             error does not add up over the pixels (the one-exponential step,
-                             M <= 128, forms the forward terms as e^{i phi_j} conj(e^{i Delta}),
-                             where a constant error of the unit only meets the small zero-order
-                             sum of e^{i phi_j}) */
+  HOT_PREC_ACCURATE = 0, /* each pair's e^{i Delta} as the product of its column and row phasors (as
+                             HOT_PREC_SEPARABLE), to FP32 rounding; with hot_set_once(c, 0):
+                             sincospif on the exactly reduced phase (~1 ulp) */
+  HOT_PREC_FAST = 1,     /* the same product; with hot_set_once(c, 0) the direct evaluation on the
+                             special-function unit: sin.approx / cos.approx of the reduced phase
+                             (arguments pre-scaled by 1 + 8.17e-8 against the unit's mean argument
+                             shrink), the forward field's phases of each pixel sub-tile rotated by a
+                             fixed pseudo-random angle and its sums back, so that the unit's
+                             systematic error does not add up over the pixels */
   HOT_PREC_SEPARABLE = 2, /* Eq. 2 factorised: e^{i Delta} = e^{i X_m(ix)} e^{i Y_m(iy)} from FP32
                              complex tables (FP64 cos/sin once per entry); per pair one complex
-                             multiply-add in each step, no transcendental function */
+                             multiply-add in each step, no transcendental function; the state is
+                             the phases at every trap count (hot_get_phasors) */
   HOT_PREC_TENSOR = 3      /* EXPERIMENTAL, outside the direct method: the separable form on the
                              tensor cores; each step of a GSW iteration is a complex matrix product
                              (S = P X, T = U X^H) run as tcgen05 FP16 MMAs with every operand split
@@ -146,7 +145,7 @@ int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out);
 int hot_get_state(hot_ctx *c, float *phi, float *w);
 int hot_set_state(hot_ctx *c, const float *phi, const float *w);
 
-/* The one-exponential step (hot_set_once) takes u_j = S_j/|S_j| for the forward field of each
+/* With up to 128 traps the accurate and fast modes (hot_set_once) take u_j = S_j/|S_j| for the forward field of each
  * iteration and evaluates phi_j = arg S_j only in the last launch of a hot_gsw, where it also
  * keeps u_j; the next hot_gsw of the context starts from those u_j, so that hot_gsw(a) followed by
  * hot_gsw(b) equals hot_gsw(a + b) bit for bit.  They belong to the state of that form:
@@ -155,7 +154,7 @@ int hot_set_state(hot_ctx *c, const float *phi, const float *w);
  * they belong to, restores them, and the resumed run continues bit for bit (without them it
  * starts from e^{i phi_j}, equal to within the phasors' rounding, ~1e-7).  u: HOST float32
  * [H*W][2] (re, im); every value finite with magnitude <= 2, else HOT_EINVAL; HOT_ESTATE when the
- * one-exponential step is not in effect.  Both synchronise.  (No counterpart in the paper.) */
+ * unit phasors are not in effect.  Both synchronise.  (No counterpart in the paper.) */
 int hot_get_phasors(hot_ctx *c, float *u);
 int hot_set_phasors(hot_ctx *c, const float *u);
 
@@ -299,32 +298,30 @@ int hot_get_tiling(const hot_ctx *c, int *rows, int *blocks_per_sm, int *chunk);
 int hot_set_block_merge(hot_ctx *c, int merge);
 int hot_get_block_merge(const hot_ctx *c, int *requested, int *in_effect);
 
-/* One-exponential step of the accurate and fast modes (no counterpart in the paper's kernel;
- * the same sums, Eq. 1 and Sec. 3): with M <= 128 traps the GSW step evaluates each pixel-trap
- * exponential E = e^{i Delta_j^m} (Eq. 2) once per iteration and keeps it in registers between
- * the back-projection S_j = sum_m c_m E and the forward field N V_m = sum_j u_j conj(E), with
- * u_j = S_j/|S_j| = e^{i phi_j} (phi_j = atan2 S_j is evaluated only in the last launch of a
- * call), which halves the cos/sin work of an iteration.  Its blocks split the M traps among their
- * warps (at most 16 traps per warp, so at most 128 traps) and walk sub-tiles of 2 to 8 rows (fixed
- * by M); its schedule is its own, so the tiling above does not apply to it (it still applies to
- * the adjoint and the superposition, which keep the direct kernels).  A call that continues from
- * the phases of the previous one starts with the forward field of the unit phasors that call's
- * last step kept (hot_get_phasors), in the step's arithmetic, so resumed sequences, CUDA graphs
- * and the persistent form give the same bits; a call that starts from phases the caller set
- * takes their forward field from the separable kernel (complex tables).  Its results differ from
- * the direct kernels' by FP32 rounding.  on: 1 (default) or 0, else HOT_EINVAL; it is in effect
- * where M <= 128 and the mode is HOT_PREC_ACCURATE or HOT_PREC_FAST.  Rebuilds the schedule;
- * synchronises the context's stream.  hot_get_once reports the setting and whether it is in
- * effect. */
+/* The kernels of the accurate and fast modes (no counterpart in the paper).  on = 1 (default): the
+ * register-tiled kernels, which take each pixel-trap exponential e^{i Delta_j^m} (Eq. 2) as the
+ * product of a tabulated column and a tabulated row phasor, for every call (GSW, fields, adjoint,
+ * superposition); on = 0: the direct step kernels, which evaluate cos and sin of every pair's
+ * phase in each sum (the tilings and the block merging above are theirs).  Both compute Eq. 1 and
+ * the back-projection of Sec. 3-4; their results differ by FP32 rounding.
+ * With on = 1 and M <= 128 traps the state keeps unit phasors ("in effect"): the forward field of an
+ * iteration takes u_j = S_j/|S_j| = e^{i phi_j}, and phi_j = atan2 S_j is evaluated only in the last
+ * launch of a call, which keeps u_j; a call that continues from the phases of the previous one
+ * starts from them (hot_get_phasors), so that resumed sequences, CUDA graphs and the persistent
+ * form give the same bits.  With more traps u_j is e^{i phi_j} of the stored phases.
+ * on: 1 or 0, else HOT_EINVAL.  Rebuilds the schedule; synchronises the context's stream.
+ * hot_get_once reports the setting and whether the unit phasors are in effect (M <= 128, mode
+ * HOT_PREC_ACCURATE or HOT_PREC_FAST). */
 int hot_set_once(hot_ctx *c, int on);
 int hot_get_once(const hot_ctx *c, int *requested, int *in_effect);
 
 /* Autotuner: times hot_gsw(iters) (CUDA events, best of 3 graph replays) for candidate tilings
  * by coordinate search over rows, blocks_per_sm (with block merging, hot_set_block_merge, as a
  * candidate in the accurate and fast modes) and chunk, keeps the fastest, and reports it
- * with its time per iteration in microseconds (outputs may be NULL).  Where the one-exponential
- * step is requested and applies (hot_set_once), it is timed too and kept if it is faster than
- * the best tiling of the direct kernels; otherwise the setting is turned off (hot_get_once).  The phases and weights
+ * with its time per iteration in microseconds (outputs may be NULL).  The search is over the
+ * direct kernels of the accurate and fast modes; the register-tiled kernels (hot_set_once), where
+ * requested, are timed too and kept if they are faster, otherwise the setting is turned off
+ * (hot_get_once).  The separable mode has no other kernels: its time is reported.  The phases and weights
  * are restored afterwards; the fields are stale until the next forward evaluation (HOT_ESTATE
  * from hot_get_fields).  Synchronises.  HOT_ESTATE before hot_set_traps; iters >= 1. */
 int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chunk, double *us_per_iter);

@@ -10,7 +10,9 @@
 // another and no reduction tail sits between iterations.  Accumulators rotate over three
 // buffers (read, written, cleared) and weights over two.  No FP64 runs per iteration.
 //
-// Per pair the kernels take exactly one complex exponential and accumulate it without a
+// This file holds the direct step kernels (hot_set_once(c, 0)) and what every mode shares; the
+// register-tiled kernels of the accurate, fast and separable modes are in tile_kernels.cuh.
+// Per pair the direct kernels take exactly one complex exponential and accumulate it without a
 // complex multiply: the back-projection folds the phase of its coefficient into the argument,
 // S_j += w_m e^{i (Delta_j^m + arg V_m)}, and the forward field evaluates Eq. 1 as written,
 // V_m += e^{i (phi_j - Delta_j^m)} (the fast mode with a per-sub-tile rotation of the phases
@@ -38,7 +40,6 @@ constexpr int kYStride = (kRowsMax + 3) & ~3;  // floats per trap in the staged 
 static_assert(kTileW == 32 && kYStride == 16, "16-byte staging of 32 columns and 16 rows per trap");
 constexpr int kChunk = 128;     // traps whose tables are staged in shared memory at once
 constexpr float kTwoPi = 6.283185307179586f;
-constexpr int kModeAccurate = 0, kModeFast = 1, kModeSeparable = 2;  // kernel variants
 
 // Work decomposition: the image is cut into 32-pixel-wide column strips; each strip's rows
 // are dealt out as contiguous runs to a fixed number of resident blocks (one wave), so that
@@ -52,7 +53,7 @@ struct StepArgs {
   int W, H, M;
   int chunk;              // traps staged in shared memory at once (1..kChunk)
   int copies;             // copies of each fixed-point accumulator buffer (a power of two; more than
-                          // one in the separable mode only): block b adds into copy b % copies,
+                          // one with the tile kernels only): block b adds into copy b % copies,
                           // spreading the atomics over more addresses
   int ldy4;               // row stride of Y4 (below)
   const SubTile *sub;     // work schedule: sub-tiles
@@ -62,10 +63,6 @@ struct StepArgs {
   const float *Y4;        // NULL, or [4][M][ldy4]: copy s holds Y shifted by s rows (Y4[s][m][i + s] =
                           // Y[m][i], zero elsewhere), so that every sub-tile's rows start 16-byte aligned
                           // in one of the copies
-  const float2 *Xc;       // [M][W] e^{i 2pi X} (separable variant)
-  const float2 *Yc;       // [2][M][ldy4] e^{i 2pi Y} (separable variant), in two copies: copy s holds the
-                          // rows shifted by s (Yc[s][m][i + s] = e^{i 2pi Y_m(i)}, zero elsewhere), so
-                          // that every sub-tile's rows start 16-byte aligned in one of them
   float *phi;             // [H*W] pixel phases, radians
   // BACK: weight update and coefficients from the previous launch's forward field
   const unsigned long long *acc_in;  // [copies][2][M] fixed-point sums of the previous forward: Re, Im
@@ -79,13 +76,13 @@ struct StepArgs {
   const float2 *G;                   // [M] or NULL: coefficients of the back-projection
   union {
     float *grad;  // [H*W] out: dL/dphi_j (ADJ)
-    float2 *u;    // NULL, or [H*W]: unit phasors u_j of phi (gsw_once_kernel, see once_flags)
+    float2 *u;    // NULL, or [H*W]: unit phasors u_j of phi (tile kernels, see once_flags)
   };
   float inv_n;                       // 1 / N
-  // gsw_once_kernel: its step takes u_j = S_j/|S_j| for the forward field and writes phi_j = arg S_j
-  // only in the last launch of a call (kOnceLast), with u_j into u when set; its forward field of
-  // the phases in phi reads u_j from u under kOnceReadU (the phasors the last step wrote for them)
-  // instead of evaluating e^{i phi_j}.
+  // Tile kernels, where the state keeps unit phasors (kOnceState): the step takes u_j = S_j/|S_j|
+  // for the forward field and writes phi_j = arg S_j only in the last launch of a call (kOnceLast),
+  // with u_j into u when set; the forward field of the phases in phi reads u_j from u under
+  // kOnceReadU (the phasors the last step wrote for them) instead of evaluating e^{i phi_j}.
   int once_flags;
   float *trace;                      // NULL, or out: e, u (Eq. 4) of the field this launch reads
   float fx_scale;           // 2^fx_shift: fixed-point scale of the sums
@@ -497,14 +494,12 @@ struct LateWeight {
 };
 
 // Start of a GSW step: the previous forward's fields are read once, every load issued before
-// any is used.  Writes the coefficients of traps [0, mc) into C0 (polar, or complex when
-// COMPLEX) without the factor <|V|> of the weight update: a factor common to all coefficients
+// any is used.  Writes the coefficients of traps [0, mc) into C0 (polar) without the factor <|V|> of the weight update: a factor common to all coefficients
 // scales S_j and leaves arg S_j unchanged (the weights' global scale is free, reading R6), so
 // no block-wide reduction stands between the sums and the back-projection.  Keeps in lw the
 // thread's share of sum |V_m| and the prefetched weight of trap own + stride * gthread(),
 // which write_weights completes after the block's work.
 // trace: NULL, or where block 0 writes e and u (Eq. 4) of the fields it read (convergence trace).
-template <bool COMPLEX>
 __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *C0, int own, int stride,
                                              LateWeight &lw, float *trace = nullptr) {
   const int t = gthread();
@@ -513,7 +508,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
   lw.v = make_float2(0.f, 0.f);
   lw.w = 0.f;
   if (lw.m < a.M) {
-    lw.v = field_from_sums<COMPLEX>(a, lw.m);
+    lw.v = field_from_sums(a, lw.m);
     lw.w = __ldcg(a.w_in + lw.m);
   }
   const float w0 = t < mc ? __ldcg(a.w_in + t) : 0.f;
@@ -523,7 +518,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
   ff si = {0.f, 0.f};
   float mx = -1.f, mn = 3.0e38f;
   for (int m = t; m < a.M; m += kThreads) {
-    const float2 v = field_from_sums<COMPLEX>(a, m);
+    const float2 v = field_from_sums(a, m);
     if (m == t) v0 = v;
     s = ff_add(s, {sqrtf(abs2(v)), 0.f});
     if (tr) {
@@ -534,7 +529,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
     }
   }
   lw.part = s;
-  if (t < mc) C0[t] = update_from<COMPLEX>(v0, w0, 1.f, a.angle_units, a.angle_eta);
+  if (t < mc) C0[t] = update_from<false>(v0, w0, 1.f, a.angle_units, a.angle_eta);
   if (tr) {  // virtual block 0 only: e = sum I_m, u = 1 - (max - min)/(max + min) of the fields read
     __shared__ ff tpart[kWarps];
     __shared__ float ext[2][kWarps];  // (group 0 of block 0 alone uses these)
@@ -568,7 +563,6 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
 // of |V_m| over the traps, Sec. 3) from the threads' shares in one fixed order (warp
 // shuffles, warps in order), so every such block obtains the same bits, and the block's
 // weight updates w_m <- w_m <|V|>/|V_m| (traps lw.m, lw.m + stride * kThreads, ...).
-template <bool MULTI = false>
 __device__ __forceinline__ void write_weights(const StepArgs &a, const LateWeight &lw, int stride) {
   if (lw.own >= a.M) return;
   __shared__ ff parts[kMaxGroups][kWarps];
@@ -586,7 +580,7 @@ __device__ __forceinline__ void write_weights(const StepArgs &a, const LateWeigh
   const float mean = (q.hi + q.lo) / (float)a.M;
   if (lw.m < a.M) a.w_out[lw.m] = update_from<false>(lw.v, lw.w, mean, 1.f).x;
   for (int m = lw.m + stride * kThreads; m < a.M; m += stride * kThreads)
-    a.w_out[m] = update_from<false>(field_from_sums<MULTI>(a, m), __ldcg(a.w_in + m), mean, 1.f).x;
+    a.w_out[m] = update_from<false>(field_from_sums(a, m), __ldcg(a.w_in + m), mean, 1.f).x;
 }
 
 struct FinalizeArgs {
@@ -835,7 +829,7 @@ __global__ void __launch_bounds__(kThreads * GROUPS, kMaxGroups / GROUPS) gsw_st
     for (int i = vb * kThreads + gthread(); i < 2 * a.M * a.copies; i += vg * kThreads) a.acc_clear[i] = 0ull;
   LateWeight lw;
   const bool gsw = BACK && !ADJ && !a.G;
-  if (gsw) gsw_prologue<false>(a, mc, sm.C0, vb, vg, lw, a.trace);
+  if (gsw) gsw_prologue(a, mc, sm.C0, vb, vg, lw, a.trace);
   for (int t = t_begin; t < t_end; t++)
     process_subtile<FAST, BACK, FWD, ADJ>(a, a.sub[t], 1.f, prestaged, sm, gsw ? sm.C0 : nullptr);
   if (gsw) write_weights(a, lw, vg);
@@ -934,99 +928,10 @@ static __global__ void __launch_bounds__(kLossThreads) intensity_loss_kernel(Los
 }
 
 // ---------------------------------------------------------------------------------------------
-// One-exponential step (direct modes, M <= kOnceMaxM traps).  The back-projection and the
-// forward field of an iteration use the same pair exponentials E_j^m = e^{i Delta_j^m}:
-//   S_j = sum_m c_m E_j^m,  c_m = w_m V_m/|V_m|      (back-projection, Sec. 3)
-//   u_j = e^{i arg S_j}                              (the new phase, phi_j = arg S_j)
-//   N V_m = sum_j u_j conj(E_j^m)                    (forward field, Eq. 1).
-// A thread keeps the exponentials of its pixels and traps in registers between the two sums,
-// so each pair costs one cos/sin per iteration instead of two.  The 8 warps of a block split
-// the traps (warp_traps over all M, at most TMAX each, fixed for the launch); lane l holds
-// column x0 + l of a sub-tile of at most R rows.  All M traps' tables of a sub-tile are staged
-// in shared memory at once (the column parts once per 32-pixel strip), one sub-tile ahead.  A
-// thread's forward sums stay in registers over all of the block's sub-tiles; they are summed
-// over the warp and added, in fixed point, once at the end.  The forward-only variant (the
-// field of given phases) evaluates the same expressions in the same order, so a sequence
-// resumed from stored phases gives the same bits.
+// Helpers of the register-tiled kernels (tile_kernels.cuh).
+
+// Largest trap count whose state keeps unit phasors (hot_set_once).
 constexpr int kOnceMaxM = 128;
-constexpr int kOnceTMax = 16;  // traps per warp at most (8 warps x 16 = kOnceMaxM)
-// Rows per sub-tile of the forward field of given phases (no exponentials kept between sub-tiles,
-// so taller sub-tiles: fewer barriers).  Its block runs are the step's, cut into sub-tiles of
-// these rows: per trap the same rows are added in the same order, so the sums are the bits of
-// the step's forward field.
-constexpr int kOnceFwdRows = 8;
-
-// Floats per trap in a staged block of row parts (R rows, in 16-byte pieces).
-__host__ __device__ constexpr int once_yw(int R) { return (R + 3) & ~3; }
-
-// Shared memory of a block: the coefficients, the row parts of two sub-tiles and the column
-// parts of two strips (the next ones are staged during the current sub-tile), the warps'
-// partial superpositions and the unit phasors u_j.
-__host__ __device__ constexpr int once_smem_bytes(int R) {
-  return kOnceMaxM * 8 + kWarps * kOnceTMax * 8 + 2 * kOnceMaxM * once_yw(R) * 4 + 2 * kOnceMaxM * kTileW * 4 +
-         kWarps * R * kTileW * 8 + R * kTileW * 8;
-}
-
-struct OnceSmem {
-  float2 *C;   // [kOnceMaxM] complex coefficients (gsw_prologue<true>)
-  float2 *Cw;  // [kWarps][kOnceTMax] each warp's coefficients, zero past its traps
-  float *Yb;   // [2][kOnceMaxM][once_yw(R)] row parts of a sub-tile's rows, by trap
-  float *Xb;   // [2][kOnceMaxM][kTileW] column parts of a strip, by trap
-  float2 *Sp;  // [kWarps][R][kTileW] per-warp superpositions
-  float2 *Ps;  // [R][kTileW] unit phasors of the sub-tile's pixels (0 outside the image)
-  int yw;
-  __device__ __forceinline__ OnceSmem(unsigned char *raw, int R) {
-    yw = once_yw(R);
-    C = reinterpret_cast<float2 *>(raw);
-    Cw = C + kOnceMaxM;
-    Yb = reinterpret_cast<float *>(Cw + kWarps * kOnceTMax);
-    Xb = Yb + 2 * kOnceMaxM * yw;
-    Sp = reinterpret_cast<float2 *>(Xb + 2 * kOnceMaxM * kTileW);
-    Ps = Sp + kWarps * R * kTileW;
-  }
-  __device__ __forceinline__ float *rows(int buf) const { return Yb + buf * kOnceMaxM * yw; }
-  __device__ __forceinline__ float *cols(int buf) const { return Xb + buf * kOnceMaxM * kTileW; }
-};
-
-// Issues the asynchronous copies of the column parts X_m(x0 .. x0 + 31) of every trap into Xb
-// (16-byte pieces when the strip lies inside the image and W is a multiple of 4; zero past the
-// right edge otherwise).  Not committed.
-__device__ __forceinline__ void once_stage_columns(const StepArgs &a, int x0, float *Xb) {
-  if ((a.W & 3) == 0 && x0 + kTileW <= a.W) {
-    for (int i = gthread(); i < a.M * (kTileW / 4); i += kThreads) {
-      const int k = i >> 3, q = i & 7;
-      cp_async16(Xb + k * kTileW + 4 * q, a.X + (size_t)k * a.W + x0 + 4 * q);
-    }
-  } else {
-    for (int i = gthread(); i < a.M * kTileW; i += kThreads) {
-      const int k = i / kTileW, col = x0 + (i % kTileW);
-      const bool ok = col < a.W;
-      cp_async4(Xb + i, a.X + (ok ? (size_t)k * a.W + col : 0), ok);
-    }
-  }
-}
-
-// Issues the asynchronous copies of the row parts Y_m(y0 .. y0 + R - 1) of every trap into Yb
-// (once_yw(R) floats per trap, 16-byte pieces of the aligned shifted copy when there is one).
-// Not committed.
-template <int R>
-__device__ __forceinline__ void once_stage_rows(const StepArgs &a, const SubTile &st, float *Yb) {
-  constexpr int YW = once_yw(R), Q = YW / 4;
-  if (a.Y4) {
-    const int s = (4 - (st.y0 & 3)) & 3;
-    const float *src = a.Y4 + (size_t)s * a.M * a.ldy4 + st.y0 + s;
-    for (int i = gthread(); i < a.M * Q; i += kThreads) {
-      const int k = i / Q, q = i % Q;
-      cp_async16(Yb + k * YW + 4 * q, src + (size_t)k * a.ldy4 + 4 * q);
-    }
-  } else {
-    for (int i = gthread(); i < a.M * YW; i += kThreads) {
-      const int k = i / YW, r = i % YW;
-      const bool ok = r < st.rows;
-      cp_async4(Yb + i, a.Y + (ok ? (size_t)k * a.H + st.y0 + r : 0), ok);
-    }
-  }
-}
 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 
@@ -1047,28 +952,13 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
   unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 
-// u = e^{i phi} of a phase reduced to one turn in table units: radians in [-pi, pi] (fast,
-// scaled by 1 + kFastEta here like the tables) or turns in [-1/2, 1/2] (accurate).
-template <bool FAST>
-__device__ __forceinline__ float2 unit_phasor(float ph) {
-  float s, c;
-  if (FAST) {
-    const float x = fmaf(ph, kFastEta, ph);
-    s = sin_approx(x);
-    c = cos_approx(x);
-  } else {
-    sincospif(2.0f * ph, &s, &c);
-  }
-  return make_float2(c, s);
-}
-
-constexpr int kOnceLast = 1, kOnceReadU = 2;  // StepArgs::once_flags
+constexpr int kOnceLast = 1, kOnceReadU = 2, kOnceState = 4;  // StepArgs::once_flags
 
 // u = S/|S|, the unit phasor e^{i arg S} without the angle; 1 for S = 0 (atan2(0, 0) = 0).
 __device__ __forceinline__ float2 unit_of(float2 s) {
@@ -1081,613 +971,6 @@ __device__ __forceinline__ float2 unit_of(float2 s) {
   if (q == 0.f) return make_float2(1.f, 0.f);
   const float r = rsqrtf(q);
   return make_float2(s.x * r, s.y * r);
-}
-
-// Back-projection of a warp's TV traps (tables and coefficients from Xs, Yb, Cw, trap by trap)
-// onto the lane's R rows: E[k][r] = e^{i (X + Y)} (kept), S[r] = sum_k c_k E[k][r], accumulated
-// as U[r] = sum_k Re(c_k) E[k][r] and W[r] = sum_k Im(c_k) E[k][r] (S = U + i W) with packed FP32
-// multiply-adds on E's (cos, sin) pair; the arguments X + Y of two rows are one packed add.  All
-// R rows are evaluated (no per-row branches): the rows past a short sub-tile's end are staged
-// rows of the next sub-tile or zero padding, and their results are discarded.
-// PIPE: the forward field of the previous sub-tile is fused in -- each of its exponentials is
-// used for acc[k] += Pp[r] conj(E[k][r]) just before it is replaced -- so that its FP32 work
-// overlaps this sub-tile's cos/sin (per trap the rows and sub-tiles are added in the same order
-// as by once_accumulate, so the sums are the same bits).
-template <bool FAST, int TV, int R, bool PIPE>
-__device__ __forceinline__ void once_back(const float *Xs, const float *Yb, const float2 *Cw, int lane,
-                                          float2 (&E)[TV][R], float2 (&S)[R], const float2 (&Pp)[R],
-                                          float2 (&acc)[TV]) {
-  constexpr int YW = once_yw(R);
-  unsigned long long U[R], Wp[R];
-#pragma unroll
-  for (int r = 0; r < R; r++) U[r] = Wp[r] = 0ull;  // (+0, +0)
-#pragma unroll
-  for (int k = 0; k < TV; k++) {
-    const float2 c = Cw[k];
-    const unsigned long long cx = pack2(c.x, c.x), cy = pack2(c.y, c.y);
-    const float xk = Xs[k * kTileW + lane];
-    const unsigned long long xx = pack2(xk, xk);
-    const ulonglong2 *yq = reinterpret_cast<const ulonglong2 *>(Yb + k * YW);
-#pragma unroll
-    for (int h = 0; h < (R + 1) / 2; h++) {
-      const ulonglong2 y4 = yq[h / 2];  // rows 4 (h / 2) .. + 3, one 16-byte load
-      const float2 arg = unpack2(add2(xx, (h & 1) ? y4.y : y4.x));  // rows 2h and 2h + 1
-      const float a2[2] = {arg.x, arg.y};
-#pragma unroll
-      for (int j = 0; j < 2; j++) {
-        const int r = 2 * h + j;
-        if (r < R) {
-          if (PIPE) {
-            acc[k].x = fmaf(Pp[r].x, E[k][r].x, fmaf(Pp[r].y, E[k][r].y, acc[k].x));
-            acc[k].y = fmaf(Pp[r].y, E[k][r].x, fmaf(-Pp[r].x, E[k][r].y, acc[k].y));
-          }
-          float co, si;
-          cis<FAST>(a2[j], co, si);
-          E[k][r] = make_float2(co, si);
-          const unsigned long long e = pack2(co, si);
-          U[r] = fma2(cx, e, U[r]);
-          Wp[r] = fma2(cy, e, Wp[r]);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < R; r++) {
-    const float2 u = unpack2(U[r]), w = unpack2(Wp[r]);
-    S[r] = make_float2(u.x - w.y, u.y + w.x);
-  }
-}
-
-// acc[k] += u_r conj(E[k][r]) over the lane's R rows (u_r = 0 past the sub-tile's end).
-template <int TV, int R>
-__device__ __forceinline__ void once_accumulate(const float2 (&P)[R], const float2 (&E)[TV][R], float2 (&acc)[TV]) {
-#pragma unroll
-  for (int k = 0; k < TV; k++) {
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-      acc[k].x = fmaf(P[r].x, E[k][r].x, fmaf(P[r].y, E[k][r].y, acc[k].x));
-      acc[k].y = fmaf(P[r].y, E[k][r].x, fmaf(-P[r].x, E[k][r].y, acc[k].y));
-    }
-  }
-}
-
-// Forward field of given phases: the exponentials of the back-projection's expression, then the
-// same accumulation (trap by trap, one trap's rows at a time).
-template <bool FAST, int TV, int R>
-__device__ __forceinline__ void once_forward_only(const float *Xs, const float *Yb, const float2 (&P)[R], int lane,
-                                                  float2 (&acc)[TV]) {
-  constexpr int YW = once_yw(R);
-#pragma unroll
-  for (int k = 0; k < TV; k++) {
-    float2 E[1][R];
-    const float xk = Xs[k * kTileW + lane];
-    const float4 *yq = reinterpret_cast<const float4 *>(Yb + k * YW);
-#pragma unroll
-    for (int q = 0; q < YW / 4; q++) {
-      const float4 y4 = yq[q];
-      const float yy[4] = {y4.x, y4.y, y4.z, y4.w};
-#pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const int r = 4 * q + j;
-        if (r < R) cis<FAST>(xk + yy[j], E[0][r].x, E[0][r].y);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-      acc[k].x = fmaf(P[r].x, E[0][r].x, fmaf(P[r].y, E[0][r].y, acc[k].x));
-      acc[k].y = fmaf(P[r].y, E[0][r].x, fmaf(-P[r].x, E[0][r].y, acc[k].y));
-    }
-  }
-}
-
-// The sub-tiles of a block, for a warp whose traps lo .. lo + T - 1 are evaluated as TV traps
-// (T <= TV; the rest are padding: zero coefficients, their sums dropped), then the warp's
-// forward sums, totalled over its lanes in a fixed order and added in fixed point.
-// PIPE: the forward field of each sub-tile runs inside the next sub-tile's back-projection
-// (once_back), the last one's after the loop.
-// BACK: the forward field takes u_j = S_j/|S_j|; last: phi_j = atan2(S_j) is written (and u_j to
-// a.u when set).  Otherwise u_j is read from a.u under kOnceReadU, else e^{i phi_j} from a.phi.
-template <bool FAST, bool BACK, int TV, int R, bool PIPE>
-__device__ __forceinline__ void once_loop(const StepArgs &a, const OnceSmem &sm, int t_begin, int t_end, int lo,
-                                          int T, bool last) {
-  const int lane = threadIdx.x & 31, warp = gthread() >> 5, t = gthread();
-  constexpr int YW = once_yw(R);
-  float2 acc[TV];
-#pragma unroll
-  for (int k = 0; k < TV; k++) acc[k] = make_float2(0.f, 0.f);
-  // the sub-tile's exponentials and unit phasors (PIPE: the previous sub-tile's until replaced;
-  // zero before the first, which adds nothing)
-  float2 E[TV][R], P[R];
-#pragma unroll
-  for (int r = 0; r < R; r++) {
-    P[r] = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < TV; k++) E[k][r] = make_float2(0.f, 0.f);
-  }
-  int xb = 0;  // the buffer of the current strip's column parts
-  for (int i = t_begin; i < t_end; i++) {
-    const SubTile st = a.sub[i];
-    const int buf = (i - t_begin) & 1;
-    if (!BACK) group_sync();  // the previous sub-tile's readers of Ps and of the other buffers are done
-    bool next_strip = false;
-    if (i + 1 < t_end) {  // stage the next sub-tile's tables
-      const SubTile nx = a.sub[i + 1];
-      once_stage_rows<R>(a, nx, sm.rows(buf ^ 1));
-      next_strip = nx.x0 != st.x0;
-      if (next_strip) once_stage_columns(a, nx.x0, sm.cols(xb ^ 1));
-    }
-    cp_async_commit();  // (an empty group after the last sub-tile: uniform waits)
-    const float *Xs = sm.cols(xb) + lo * kTileW, *Yb = sm.rows(buf) + lo * YW;
-    if (BACK) {
-      float2 S[R];
-#pragma unroll
-      for (int r = 0; r < R; r++) S[r] = make_float2(0.f, 0.f);
-      once_back<FAST, TV, R, PIPE>(Xs, Yb, sm.Cw + warp * kOnceTMax, lane, E, S, P, acc);
-#pragma unroll
-      for (int r = 0; r < R; r++)
-        if (r < st.rows) sm.Sp[(warp * R + r) * kTileW + lane] = S[r];
-      group_sync();
-      if (t < st.rows * kTileW) {  // one pixel per thread: the 8 warps' sums in warp order
-        const int r = t >> 5, l = t & 31, ix = st.x0 + l;
-        float2 s = sm.Sp[r * kTileW + l];
-#pragma unroll
-        for (int w = 1; w < kWarps; w++) {
-          const float2 q = sm.Sp[(w * R + r) * kTileW + l];
-          s.x += q.x;
-          s.y += q.y;
-        }
-        const float2 u = unit_of(s);
-        if (last && ix < a.W) {
-          const size_t j = (size_t)(st.y0 + r) * a.W + ix;
-          a.phi[j] = atan2f(s.y, s.x);
-          if (a.u) a.u[j] = u;
-        }
-        sm.Ps[r * kTileW + l] = ix < a.W ? u : make_float2(0.f, 0.f);
-      }
-      asm volatile("cp.async.wait_group 0;\n" ::: "memory");  // the next sub-tile's tables
-    } else {
-      if (t < st.rows * kTileW) {
-        const int r = t >> 5, l = t & 31, ix = st.x0 + l;
-        const size_t j = (size_t)(st.y0 + r) * a.W + ix;
-        float2 u = make_float2(0.f, 0.f);
-        if (ix < a.W)
-          u = (a.once_flags & kOnceReadU) ? a.u[j]
-                                          : unit_phasor<FAST>(FAST ? reduced_radians(a.phi[j]) : reduced_phase_turns(a.phi[j]));
-        sm.Ps[r * kTileW + l] = u;
-      }
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // this sub-tile's tables
-    }
-    group_sync();
-#pragma unroll
-    for (int r = 0; r < R; r++) P[r] = r < st.rows ? sm.Ps[r * kTileW + lane] : make_float2(0.f, 0.f);
-    if (!BACK)
-      once_forward_only<FAST, TV, R>(Xs, Yb, P, lane, acc);
-    else if (!PIPE)
-      once_accumulate<TV, R>(P, E, acc);
-    if (next_strip) xb ^= 1;
-  }
-  if (BACK && PIPE) once_accumulate<TV, R>(P, E, acc);  // the forward field of the last sub-tile
-  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-  unsigned long long *const out = block_acc(a);
-#pragma unroll
-  for (int g = 0; g < TV; g += kGroup) {
-    float2 v8[kGroup];
-#pragma unroll
-    for (int i = 0; i < kGroup; i++) v8[i] = g + i < TV ? acc[g + i] : make_float2(0.f, 0.f);
-    const float2 v = warp_reduce8(v8, lane);
-    const int k = g + ((lane >> 2) & 7);
-    if ((lane & 3) == 0 && k < T) {
-      // |v| <= the block's pixel count <= N, so v * 2^fx_shift is an exact integer below 2^62
-      atomicAdd(out + lo + k, (unsigned long long)__float2ll_rn(v.x * a.fx_scale));
-      atomicAdd(out + a.M + lo + k, (unsigned long long)__float2ll_rn(v.y * a.fx_scale));
-    }
-  }
-}
-
-// The work of one block on its sub-tiles [t_begin, t_end) after the dependency wait and the
-// clearing of the next accumulator.  On entry the first sub-tile's row and column parts are
-// being staged into rows(0) and cols(0) (one committed group).
-// BACK: weight update, back-projection -> a.phi, forward field of the new phases; otherwise
-// the forward field of the phases in a.phi.
-// A warp's trap count T is TMAX, TMAX - 1 or TMAX - 2 (warp_traps); every warp runs the loop
-// compiled for TMAX traps, the ones past T as padding, so that no per-trap branch remains and
-// one copy of the unrolled loop serves the block (with the fused forward field, copies for T
-// and T - 1 ran slower).  From 4 traps per warp, with at most 32 exponentials per thread, each
-// sub-tile's forward field is fused into the next sub-tile's back-projection (with more the
-// registers spill; with 2 traps per warp it does not pay).
-template <bool FAST, bool BACK, int TMAX, int R>
-__device__ __forceinline__ void once_block(const StepArgs &a, const OnceSmem &sm, int t_begin, int t_end,
-                                           float *trace, bool last) {
-  static_assert(TMAX >= 1 && TMAX <= kOnceTMax, "traps per warp");
-  const int lane = threadIdx.x & 31, warp = gthread() >> 5;
-  int lo, hi;
-  warp_traps(a.M, warp, lo, hi);
-  const int T = hi - lo;
-  if (BACK) {  // the weights are written here, before the sub-tiles: nothing stays live across them
-    LateWeight lw;
-    gsw_prologue<true>(a, a.M, sm.C, vblock(), vgrid(), lw, trace);
-    write_weights<true>(a, lw, vgrid());
-  }
-  // Padding traps read table rows from M on (never staged): zero, in both buffers.
-  for (int i = gthread(); i < 2 * kOnceTMax * (kTileW + sm.yw); i += kThreads) {
-    const int b = i / (kOnceTMax * (kTileW + sm.yw)), j = i % (kOnceTMax * (kTileW + sm.yw));
-    if (j < kOnceTMax * kTileW) {
-      if (a.M * kTileW + j < kOnceMaxM * kTileW) sm.cols(b)[a.M * kTileW + j] = 0.f;
-    } else if (a.M * sm.yw + (j - kOnceTMax * kTileW) < kOnceMaxM * sm.yw) {
-      sm.rows(b)[a.M * sm.yw + (j - kOnceTMax * kTileW)] = 0.f;
-    }
-  }
-  if (BACK) {
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    group_sync();  // coefficients, padding and the first tables are in place
-    if (lane < kOnceTMax) sm.Cw[warp * kOnceTMax + lane] = lane < T ? sm.C[lo + lane] : make_float2(0.f, 0.f);
-    __syncwarp();
-  }
-  constexpr bool PIPE = TMAX >= 4 && TMAX * R <= 32;
-  once_loop<FAST, BACK, TMAX, R, PIPE>(a, sm, t_begin, t_end, lo, T, last);
-}
-
-// Stages the first sub-tile's tables of a block (one committed group; empty without work).
-template <int R>
-__device__ __forceinline__ void once_stage_first(const StepArgs &a, const OnceSmem &sm, int t_begin, int t_end) {
-  if (t_begin < t_end) {
-    const SubTile st0 = a.sub[t_begin];
-    once_stage_rows<R>(a, st0, sm.rows(0));
-    once_stage_columns(a, st0.x0, sm.cols(0));
-  }
-  cp_async_commit();
-}
-
-// The shape of M traps (0: none, M > kOnceMaxM): TMAX = ceil(M / 8) traps per warp at most.
-__host__ __device__ constexpr int once_shape(int M) { return M <= 0 || M > kOnceMaxM ? 0 : (M + kWarps - 1) / kWarps; }
-// R, the rows per sub-tile of a shape: 8 up to 4 traps per warp, 3 for 11 (faster there than 2),
-// otherwise the largest R with TMAX R <= 32 (the fused forward field, once_block).
-__host__ __device__ constexpr int once_rows(int shape) {
-  return shape <= 4 ? 8 : shape == 11 ? 3 : 32 / shape < 8 ? 32 / shape : 8;
-}
-
-// Calls BODY (parenthesised) with compile-time TMAX and R of a shape (once_shape).
-#define HOT_ONCE_CASE(k, BODY) \
-  case k: { constexpr int TMAX = k, R = ::hot::once_rows(k); BODY; } break;
-#define HOT_WITH_ONCE_SHAPE(shape, BODY)                                                        \
-  switch (shape) {                                                                              \
-    HOT_ONCE_CASE(1, BODY) HOT_ONCE_CASE(2, BODY) HOT_ONCE_CASE(3, BODY) HOT_ONCE_CASE(4, BODY)   \
-    HOT_ONCE_CASE(5, BODY) HOT_ONCE_CASE(6, BODY) HOT_ONCE_CASE(7, BODY) HOT_ONCE_CASE(8, BODY)   \
-    HOT_ONCE_CASE(9, BODY) HOT_ONCE_CASE(10, BODY) HOT_ONCE_CASE(11, BODY) HOT_ONCE_CASE(12, BODY) \
-    HOT_ONCE_CASE(13, BODY) HOT_ONCE_CASE(14, BODY) HOT_ONCE_CASE(15, BODY)                      \
-    default: HOT_ONCE_CASE(16, BODY)                                                            \
-  }
-
-// The per-launch form.  The tables are constant during hot_gsw: the first sub-tile's are
-// staged before waiting for the previous launch.
-template <bool FAST, bool BACK, int TMAX, int R>
-__global__ void __launch_bounds__(kThreads, 2) gsw_once_kernel(StepArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const OnceSmem sm(smem_raw, R);
-  const int vb = vblock(), vg = vgrid();
-  const int t_begin = a.first[vb], t_end = a.first[vb + 1];
-  allow_dependents();
-  once_stage_first<R>(a, sm, t_begin, t_end);
-  grid_dependency_wait();
-  for (int i = vb * kThreads + gthread(); i < 2 * a.M * a.copies; i += vg * kThreads) a.acc_clear[i] = 0ull;
-  once_block<FAST, BACK, TMAX, R>(a, sm, t_begin, t_end, a.trace, (a.once_flags & kOnceLast) != 0);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Separable variant.  Eq. 2 is a sum of a column part and a row part, so every pair's
-// exponential factorises: e^{i Delta_j^m} = Xc_m(ix) Yc_m(iy), with both factors tabulated once
-// per trap (FP64 cos/sin of the exactly reduced turns, stored as FP32 complex).  Per pair the
-// back-projection then takes one complex multiply-add,
-//   S_j += Yc_m(iy) [c_m Xc_m(ix)]           (the bracket once per trap and lane),
-// and the forward field another,
-//   V_m += conj(Xc_m(ix)) sum_iy u_j conj(Yc_m(iy))   with u_j = e^{i phi_j},
-// i.e. 8 FP32 FMA per pixel-trap update and no per-pair transcendental function (one sincos
-// per pixel and iteration gives u_j from the stored phase).  The coefficients are kept
-// complex, c_m = w_m V_m/|V_m| (Sec. 3).
-// The work decomposition, staging, reductions and fixed-point sums are the direct kernel's.
-constexpr int kSepUsFloats = kRowsMax * kTileW * 2;
-
-__host__ __device__ constexpr int sep_smem_bytes(int chunk) {
-  return chunk * (kTileW + kYStride) * 8 + 2 * chunk * 8 + kWarps * kHalfRows * kTileW * 8 + kSepUsFloats * 4;
-}
-
-struct SepSmem {
-  float2 *Xs, *Ys, *Cs, *Sp, *Us, *C0;
-  __device__ __forceinline__ SepSmem(unsigned char *raw, int chunk) {
-    Xs = reinterpret_cast<float2 *>(raw);  // [chunk][kTileW]
-    Ys = Xs + chunk * kTileW;              // [chunk][kYStride]
-    Cs = Ys + chunk * kYStride;            // [chunk]
-    Sp = Cs + chunk;                       // [kWarps][kHalfRows][kTileW]
-    Us = Sp + kWarps * kHalfRows * kTileW; // [kRowsMax][kTileW] unit phasors of the sub-tile
-    C0 = Us + kRowsMax * kTileW;           // [chunk] coefficients of the first chunk (prologue)
-  }
-};
-
-// Sec. 3 coefficient of trap m in complex form: w_m' V_m/|V_m| with w_m' = w_m <|V|>/|V_m|
-// (R4: |V_m| = 0 keeps w_m and takes the unit field 1).
-__device__ __forceinline__ float2 complex_coefficient(const StepArgs &a, int m, float mean) {
-  return update_from<true>(field_from_sums<true>(a, m), __ldcg(a.w_in + m), mean, 1.f);
-}
-
-template <bool BACK, bool ADJ = false>
-__device__ __forceinline__ void stage_sep(const StepArgs &a, int m0, int n, const SubTile &st, const SepSmem &sm,
-                                          bool xy = true, float mean = 0.f, bool coef = true) {
-  if (xy) {
-    if ((a.W & 1) == 0 && st.x0 + kTileW <= a.W) {
-      // thread t copies columns 2 (t % 16), +1 of traps t / 16, t / 16 + 16, ... (16 bytes:
-      // rows start 16-byte aligned for even W)
-      const int q = gthread() % (kTileW / 2), kx = gthread() / (kTileW / 2);
-      const float2 *src = a.Xc + (size_t)(m0 + kx) * a.W + st.x0 + 2 * q;
-      const size_t sx = (size_t)(kThreads / (kTileW / 2)) * a.W;
-      for (int k = kx; k < n; k += kThreads / (kTileW / 2), src += sx) cp_async16(sm.Xs + k * kTileW + 2 * q, src);
-    } else {
-      // thread t copies column t % 32 of traps t / 32, t / 32 + 8, ...: fixed column, pointers
-      // advanced by whole trap strides
-      const int col = gthread() % kTileW, kx = gthread() / kTileW;
-      const bool okx = st.x0 + col < a.W;
-      const float2 *src = a.Xc + (okx ? (size_t)(m0 + kx) * a.W + st.x0 + col : 0);
-      const size_t sx = okx ? (size_t)(kThreads / kTileW) * a.W : 0;
-      for (int k = kx; k < n; k += kThreads / kTileW, src += sx) cp_async8(sm.Xs + k * kTileW + col, src, okx);
-    }
-    // rows y0 .. y0 + 15 of copy y0 % 2 (16-byte aligned): thread t copies rows 2 (t % 8), +1 of
-    // traps t / 8, t / 8 + 32, ...
-    const int s = st.y0 & 1, q = gthread() % (kYStride / 2), ky = gthread() / (kYStride / 2);
-    const float2 *srcy = a.Yc + ((size_t)s * a.M + m0 + ky) * a.ldy4 + st.y0 + s + 2 * q;
-    const size_t sy = (size_t)(kThreads / (kYStride / 2)) * a.ldy4;
-    for (int k = ky; k < n; k += kThreads / (kYStride / 2), srcy += sy) cp_async16(sm.Ys + k * kYStride + 2 * q, srcy);
-  }
-  if (BACK && coef)
-    for (int i = gthread(); i < n; i += kThreads)
-      sm.Cs[i] = (ADJ || a.G) ? a.G[m0 + i] : complex_coefficient(a, m0 + i, mean);
-  cp_async_wait_all();
-}
-
-// S_r += Yc_m(r) (c_m Xc_m(lane)) for traps [lo, hi) of the staged chunk (coefficients C).
-template <int R>
-__device__ __forceinline__ void back_traps_sep(const SepSmem &sm, const float2 *C, int lo, int hi, int lane,
-                                               float2 (&S)[kRowsMax]) {
-  for (int k = lo; k < hi; k++) {
-    const float2 x = sm.Xs[k * kTileW + lane], c = C[k];
-    const float2 b = make_float2(c.x * x.x - c.y * x.y, c.x * x.y + c.y * x.x);
-    const float4 *yq = reinterpret_cast<const float4 *>(sm.Ys + k * kYStride);
-#pragma unroll
-    for (int q = 0; q < (R + 1) / 2; q++) {
-      const float4 y2 = yq[q];
-      const float2 yy[2] = {make_float2(y2.x, y2.y), make_float2(y2.z, y2.w)};
-#pragma unroll
-      for (int j = 0; j < 2; j++) {
-        const int r = 2 * q + j;
-        if (r < R) {
-          S[r].x = fmaf(yy[j].x, b.x, fmaf(-yy[j].y, b.y, S[r].x));
-          S[r].y = fmaf(yy[j].x, b.y, fmaf(yy[j].y, b.x, S[r].y));
-        }
-      }
-    }
-  }
-}
-
-// Forward field of traps [lo, hi): conj(Xc_m(lane)) sum_r u_r conj(Yc_m(r)), summed over the
-// warp 8 traps at a time and added in fixed point (as forward_traps).  u is zero outside the
-// image, so no mask is needed.
-template <int R>
-__device__ __forceinline__ void forward_traps_sep(const SepSmem &sm, int lo, int hi, int lane,
-                                                  const float2 (&u)[kRowsMax], const StepArgs &a, int m0) {
-  for (int g = lo; g < hi; g += kGroup) {
-    float2 acc[kGroup];
-#pragma unroll
-    for (int i = 0; i < kGroup; i++) {
-      acc[i] = make_float2(0.f, 0.f);
-      const int k = g + i;
-      if (k < hi) {
-        const float4 *yq = reinterpret_cast<const float4 *>(sm.Ys + k * kYStride);
-        float2 t = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < (R + 1) / 2; q++) {
-          const float4 y2 = yq[q];
-          const float2 yy[2] = {make_float2(y2.x, y2.y), make_float2(y2.z, y2.w)};
-#pragma unroll
-          for (int j = 0; j < 2; j++) {
-            const int r = 2 * q + j;
-            if (r < R) {
-              t.x = fmaf(u[r].x, yy[j].x, fmaf(u[r].y, yy[j].y, t.x));
-              t.y = fmaf(u[r].y, yy[j].x, fmaf(-u[r].x, yy[j].y, t.y));
-            }
-          }
-        }
-        const float2 x = sm.Xs[k * kTileW + lane];
-        acc[i] = make_float2(t.x * x.x + t.y * x.y, t.y * x.x - t.x * x.y);
-      }
-    }
-    const float2 v = warp_reduce8(acc, lane);
-    const int k = g + ((lane >> 2) & 7);
-    if ((lane & 3) == 0 && k < hi) {
-      unsigned long long *acc = block_acc(a);
-      atomicAdd(acc + m0 + k, (unsigned long long)__float2ll_rn(v.x * a.fx_scale));
-      atomicAdd(acc + a.M + m0 + k, (unsigned long long)__float2ll_rn(v.y * a.fx_scale));
-    }
-  }
-}
-
-template <bool BACK, bool FWD, bool ADJ>
-__device__ __forceinline__ void process_subtile_sep(const StepArgs &a, const SubTile st, float mean, bool &prestaged,
-                                                    const SepSmem &sm, const float2 *C0 = nullptr) {
-  const int lane = threadIdx.x & 31, warp = gthread() >> 5;
-  const int mc = a.M < a.chunk ? a.M : a.chunk;
-  const int nchunks = (a.M + mc - 1) / mc;
-  const int ix = st.x0 + lane;
-  const bool col_ok = ix < a.W;
-
-  if (BACK) {
-    float2 S[kRowsMax];
-#pragma unroll
-    for (int r = 0; r < kRowsMax; r++) S[r] = make_float2(0.f, 0.f);
-    for (int ch = 0; ch < nchunks; ch++) {
-      const int m0 = ch * mc, n = min(mc, a.M - m0);
-      const bool pre = C0 && ch == 0;
-      group_sync();  // earlier readers of the tables are done
-      stage_sep<true, ADJ>(a, m0, n, st, sm, !prestaged, mean, !pre);
-      prestaged = false;
-      group_sync();
-      int lo, hi;
-      warp_traps(n, warp, lo, hi);
-      const float2 *C = pre ? C0 : sm.Cs;
-      HOT_WITH_ROWS(st.rows, (back_traps_sep<R>(sm, C, lo, hi, lane, S)));
-    }
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-      if (h * kHalfRows >= st.rows) break;
-      group_sync();  // Sp and the phasor rows are free
-#pragma unroll
-      for (int i = 0; i < kHalfRows; i++)
-        if (h * kHalfRows + i < st.rows) sm.Sp[(warp * kHalfRows + i) * kTileW + lane] = S[h * kHalfRows + i];
-      group_sync();
-      if (warp < kHalfRows && h * kHalfRows + warp < st.rows) {
-        const int r = h * kHalfRows + warp;
-        float2 s = sm.Sp[warp * kTileW + lane];
-#pragma unroll
-        for (int w = 1; w < kWarps; w++) {
-          const float2 q = sm.Sp[(w * kHalfRows + warp) * kTileW + lane];
-          s.x += q.x;
-          s.y += q.y;
-        }
-        const size_t j = (size_t)(st.y0 + r) * a.W + ix;
-        if (ADJ) {
-          if (col_ok) {
-            float sp, cp;
-            sincosf(a.phi[j], &sp, &cp);
-            a.grad[j] = (cp * s.y - sp * s.x) * a.inv_n;  // Im[(cos - i sin)(S.x + i S.y)] / N
-          }
-        } else {
-          const float ph = atan2f(s.y, s.x);
-          if (col_ok) a.phi[j] = ph;
-          if (FWD) {  // u = e^{i phi} of the stored phase (so that a resumed run is identical)
-            float2 u = make_float2(0.f, 0.f);
-            if (col_ok) sincosf(ph, &u.y, &u.x);
-            sm.Us[r * kTileW + lane] = u;
-          }
-        }
-      }
-    }
-  } else if (FWD) {
-    group_sync();  // earlier readers of the phasors and of the tables are done
-    for (int r = warp; r < st.rows; r += kWarps) {
-      float2 u = make_float2(0.f, 0.f);
-      if (col_ok) sincosf(a.phi[(size_t)(st.y0 + r) * a.W + ix], &u.y, &u.x);
-      sm.Us[r * kTileW + lane] = u;
-    }
-  }
-
-  if (FWD) {
-    group_sync();  // the phasors are complete
-    float2 u[kRowsMax];
-#pragma unroll
-    for (int r = 0; r < kRowsMax; r++) u[r] = r < st.rows ? sm.Us[r * kTileW + lane] : make_float2(0.f, 0.f);
-    for (int ch = 0; ch < nchunks; ch++) {
-      const int m0 = ch * mc, n = min(mc, a.M - m0);
-      if (!BACK || nchunks > 1) {  // with one chunk the back-projection's tables are still staged
-        if (ch) group_sync();
-        stage_sep<false>(a, m0, n, st, sm);
-        group_sync();
-      }
-      int lo, hi;
-      warp_traps(n, warp, lo, hi);
-      HOT_WITH_ROWS(st.rows, (forward_traps_sep<R>(sm, lo, hi, lane, u, a, m0)));
-    }
-  }
-}
-
-template <bool BACK, bool FWD, bool ADJ = false>
-// Two resident blocks per SM: the complex accumulators and tables of the separable loops need
-// more than the 80 registers of three blocks (measured 15 % faster at 512^2, M = 100).
-__global__ void __launch_bounds__(kThreads, 2) gsw_sep_kernel(StepArgs a) {
-  static_assert(!ADJ || (BACK && !FWD), "the adjoint is a back-projection without forward field");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const SepSmem sm(smem_raw, a.chunk);
-  const int mc = a.M < a.chunk ? a.M : a.chunk;
-  const int t_begin = a.first[blockIdx.x], t_end = a.first[blockIdx.x + 1];
-
-  allow_dependents();
-  bool prestaged = false;
-  if (BACK && t_begin < t_end) {
-    stage_sep<false>(a, 0, mc, a.sub[t_begin], sm);
-    prestaged = true;
-  }
-  grid_dependency_wait();
-  if (FWD)
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * a.M * a.copies; i += gridDim.x * kThreads) a.acc_clear[i] = 0ull;
-  LateWeight lw;
-  const bool gsw = BACK && !ADJ && !a.G;
-  if (gsw) gsw_prologue<true>(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, a.trace);
-  for (int t = t_begin; t < t_end; t++)
-    process_subtile_sep<BACK, FWD, ADJ>(a, a.sub[t], 1.f, prestaged, sm, gsw ? sm.C0 : nullptr);
-  if (gsw) write_weights<true>(a, lw, gridDim.x);
-}
-
-// Batched launch: the sub-tiles of up to kBatchMax holograms (SubTile::pad = hologram index)
-// in one grid.  The holograms' parameters travel in the launch itself (a __grid_constant__
-// argument read through the constant cache, as the single-hologram kernel reads its own).
-// Every block that meets a hologram computes its <|V|> and coefficients itself; the weights
-// of hologram h are written by block owner[h].
-constexpr int kBatchMax = 22;  // keeps the launch argument under 4 KB
-
-struct BatchArgs {
-  StepArgs holo[kBatchMax];
-  int owner[kBatchMax];
-  const SubTile *sub;
-  const int *first;  // [gridDim.x + 1]
-  int count;
-};
-static_assert(sizeof(BatchArgs) <= 4096, "launch argument above 4 KB");
-
-// MODE: kModeAccurate, kModeFast or kModeSeparable (the separable kernel's staging capacity is
-// the batch's chunk, the same for all holograms of a launch).
-template <int MODE, bool BACK, bool FWD>
-__global__ void __launch_bounds__(kThreads, MODE == kModeSeparable ? 2 : 4)
-    gsw_batch_kernel(const __grid_constant__ BatchArgs b) {
-  constexpr bool FAST = MODE == kModeFast, SEP = MODE == kModeSeparable;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int t_begin = b.first[blockIdx.x], t_end = b.first[blockIdx.x + 1];
-  const int cap = b.holo[0].chunk;
-  float2 *const C0 = SEP ? SepSmem(smem_raw, cap).C0 : StepSmem(smem_raw).C0;
-
-  allow_dependents();
-  bool prestaged = false;
-  if (BACK && t_begin < t_end) {
-    const SubTile st0 = b.sub[t_begin];
-    const StepArgs &a0 = b.holo[st0.pad];
-    const int mc0 = a0.M < a0.chunk ? a0.M : a0.chunk;
-    if constexpr (SEP) {
-      stage_sep<false>(a0, 0, mc0, st0, SepSmem(smem_raw, cap));
-    } else {
-      const StepSmem sm(smem_raw);
-      stage_tables<false>(a0, 0, mc0, st0, sm.Xs, sm.Ys, sm.Cs);
-    }
-    prestaged = true;
-  }
-  grid_dependency_wait();
-  if (FWD)  // clear the buffers the next launch accumulates into, for every hologram
-    for (int h = 0; h < b.count; h++) {
-      unsigned long long *clr = b.holo[h].acc_clear;
-      const int n2 = 2 * b.holo[h].M * b.holo[h].copies;
-      for (int i = blockIdx.x * kThreads + threadIdx.x; i < n2; i += gridDim.x * kThreads) clr[i] = 0ull;
-    }
-  int cur = -1;
-  LateWeight lw;  // the owner block writes all weights of a hologram, after its sub-tiles
-  for (int t = t_begin; t < t_end; t++) {
-    const SubTile st = b.sub[t];
-    const StepArgs &a = b.holo[st.pad];
-    if (BACK && st.pad != cur) {
-      if (cur >= 0) write_weights<SEP>(b.holo[cur], lw, 1);
-      const int mc = a.M < a.chunk ? a.M : a.chunk;
-      gsw_prologue<SEP>(a, mc, C0, b.owner[st.pad] == (int)blockIdx.x ? 0 : a.M, 1, lw);
-    }
-    cur = st.pad;
-    if constexpr (SEP)
-      process_subtile_sep<BACK, FWD, false>(a, st, 1.f, prestaged, SepSmem(smem_raw, cap), BACK ? C0 : nullptr);
-    else
-      process_subtile<FAST, BACK, FWD, false>(a, st, 1.f, prestaged, StepSmem(smem_raw), BACK ? C0 : nullptr);
-  }
-  if (BACK && cur >= 0) write_weights<SEP>(b.holo[cur], lw, 1);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1753,15 +1036,12 @@ __device__ __forceinline__ bool grid_sync(const GridSync &g, unsigned int &epoch
 struct PersistArgs {
   StepArgs step[6];
   int iters;
-  int k0;  // one-exponential form: the first launch it runs (1: launch 0 was its own launch before it)
   GridSync sync;
   float *trace;  // NULL, or [iters][2]: e, u of the field read by iteration k (convergence trace)
 };
 
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, MODE == kModeSeparable ? 2 : 4)
-    gsw_persistent_kernel(const __grid_constant__ PersistArgs p) {
-  constexpr bool FAST = MODE == kModeFast;
+template <bool FAST>
+__global__ void __launch_bounds__(kThreads, 4) gsw_persistent_kernel(const __grid_constant__ PersistArgs p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StepArgs &a0 = p.step[0];
   const int mc = a0.M < a0.chunk ? a0.M : a0.chunk;
@@ -1775,48 +1055,16 @@ __global__ void __launch_bounds__(kThreads, MODE == kModeSeparable ? 2 : 4)
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * a.M * a.copies; i += gridDim.x * kThreads) a.acc_clear[i] = 0ull;
     const float mean = 1.f;  // coefficients without the common factor <|V|> (see gsw_prologue)
     LateWeight lw;
-    if constexpr (MODE == kModeSeparable) {
-      const SepSmem sm(smem_raw, mc);
-      if (k > 0) gsw_prologue<true>(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, p.trace ? p.trace + 2 * (k - 1) : nullptr);
-      for (int t = t_begin; t < t_end; t++) {
-        bool prestaged = resident && k > 0;
-        if (k == 0)
-          process_subtile_sep<false, true, false>(a, a.sub[t], 0.f, prestaged, sm);
-        else
-          process_subtile_sep<true, true, false>(a, a.sub[t], mean, prestaged, sm, sm.C0);
-      }
-    } else {
-      const StepSmem sm(smem_raw);
-      if (k > 0) gsw_prologue<false>(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, p.trace ? p.trace + 2 * (k - 1) : nullptr);
-      for (int t = t_begin; t < t_end; t++) {
-        bool prestaged = resident && k > 0;
-        if (k == 0)
-          process_subtile<FAST, false, true, false>(a, a.sub[t], 0.f, prestaged, sm);
-        else
-          process_subtile<FAST, true, true, false>(a, a.sub[t], mean, prestaged, sm, sm.C0);
-      }
+    const StepSmem sm(smem_raw);
+    if (k > 0) gsw_prologue(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, p.trace ? p.trace + 2 * (k - 1) : nullptr);
+    for (int t = t_begin; t < t_end; t++) {
+      bool prestaged = resident && k > 0;
+      if (k == 0)
+        process_subtile<FAST, false, true, false>(a, a.sub[t], 0.f, prestaged, sm);
+      else
+        process_subtile<FAST, true, true, false>(a, a.sub[t], mean, prestaged, sm, sm.C0);
     }
-    if (k > 0) write_weights<MODE == kModeSeparable>(a, lw, gridDim.x);
-  }
-}
-
-// The persistent form of the one-exponential step (same schedule, same arithmetic, same bits).
-template <bool FAST, int TMAX, int R>
-__global__ void __launch_bounds__(kThreads, 2) gsw_once_persistent_kernel(const __grid_constant__ PersistArgs p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const OnceSmem sm(smem_raw, R);
-  const StepArgs &a0 = p.step[0];
-  const int t_begin = a0.first[blockIdx.x], t_end = a0.first[blockIdx.x + 1];
-  unsigned int epoch = 0u;
-  for (int k = p.k0; k <= p.iters; k++) {
-    const StepArgs &a = p.step[k % 6];
-    if (k > p.k0 && !grid_sync(p.sync, epoch)) return;
-    once_stage_first<R>(a, sm, t_begin, t_end);
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * a.M * a.copies; i += gridDim.x * kThreads) a.acc_clear[i] = 0ull;
-    if (k == 0)
-      once_block<FAST, false, TMAX, R>(a, sm, t_begin, t_end, nullptr, false);
-    else
-      once_block<FAST, true, TMAX, R>(a, sm, t_begin, t_end, p.trace ? p.trace + 2 * (k - 1) : nullptr, k == p.iters);
+    if (k > 0) write_weights(a, lw, gridDim.x);
   }
 }
 
@@ -1825,11 +1073,12 @@ __global__ void __launch_bounds__(kThreads, 2) gsw_once_persistent_kernel(const 
 // A row band (rows y_off .. y_off+H-1 of a hologram of H_total rows) takes the row parts of
 // its global rows.
 // Y4t, Y4r (optional): the shifted copies of the row parts (StepArgs::Y4), [4][M][ldy4], and
-// Yc2 (optional) the two shifted copies of Yc (StepArgs::Yc), [2][M][ldy4], whose entries outside
-// the shifted rows stay as they are (zero from allocation).
+// Xq, Yq (optional) the tile kernels' tables (TileArgs, strips of 64 columns); entries outside the
+// image stay as they are (zero from allocation).
 static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off, int M, const double *abc, float *Xt,
                                     float *Yt, float *Xr, float *Yr, float2 *Xc, float2 *Yc, float *Y4t = nullptr,
-                                    float *Y4r = nullptr, int ldy4 = 0, float2 *Yc2 = nullptr) {
+                                    float *Y4r = nullptr, int ldy4 = 0, float2 *Xq = nullptr, float4 *Yq = nullptr,
+                                    int Mp = 0, int ldp = 0) {
   const long long total = (long long)M * (W + H);
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
@@ -1852,6 +1101,7 @@ static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off,
       Xt[(size_t)m * W + i] = tf;
       Xr[(size_t)m * W + i] = rf;
       if (Xc) Xc[(size_t)m * W + i] = make_float2((float)cs, (float)sn);
+      if (Xq) Xq[((size_t)(i >> 6) * Mp + m) * 64 + (i & 63)] = make_float2((float)cs, (float)sn);
     } else {
       Yt[(size_t)m * H + (i - W)] = tf;
       Yr[(size_t)m * H + (i - W)] = rf;
@@ -1861,8 +1111,11 @@ static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off,
           Y4r[((size_t)sh * M + m) * ldy4 + (i - W) + sh] = rf;
         }
       if (Yc) Yc[(size_t)m * H + (i - W)] = make_float2((float)cs, (float)sn);
-      if (Yc2)
-        for (int sh = 0; sh < 2; sh++) Yc2[((size_t)sh * M + m) * ldy4 + (i - W) + sh] = make_float2((float)cs, (float)sn);
+      if (Yq) {
+        float *const y = reinterpret_cast<float *>(Yq + (size_t)m * ldp + ((i - W) >> 1)) + ((i - W) & 1);
+        y[0] = (float)cs;
+        y[2] = (float)sn;
+      }
     }
   }
 }

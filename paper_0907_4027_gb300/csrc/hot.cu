@@ -12,8 +12,8 @@
 
 #include "../../include/hot.h"
 #include "gsw_kernels.cuh"
-#include "once.h"
 #include "tc.h"
+#include "tile.h"
 
 namespace {
 
@@ -74,18 +74,15 @@ struct hot_ctx {
   int sched_bps = 0, sched_bps_max = 0;  // resident blocks per SM in the schedule; occupancy limit
   int tile_merge = 1;  // hot_set_block_merge: schedule blocks per launched block of the GSW step (1, 2, 4)
   int groups = 1;      // schedule blocks per launched block of the direct GSW step (1 or 4)
-  // one-exponential step of the direct modes (hot_set_once; M <= hot::kOnceMaxM): requested,
-  // shape in effect (hot::once_shape; 0: the direct step kernels) and its own schedule
+  // register-tiled kernels (tile_kernels.cuh): the separable mode, and the accurate and fast modes
+  // unless hot_set_once turned them to the direct step kernels; their own schedule
   bool once_req = true;
-  int once = 0;
-  hot::SubTile *osub = nullptr;  // [on_sub]
-  int *ofirst = nullptr;         // [ogrid + 1]
-  int ogrid = 0, on_sub = 0;
-  // the same block runs cut into sub-tiles of hot::kOnceFwdRows rows: the forward field of given phases
-  hot::SubTile *ofsub = nullptr;
-  int *offirst = nullptr;
-  // the unit phasors u_j = S_j/|S_j| of phi, written by the last step of a one-exponential hot_gsw
-  // (hot::StepArgs::u_out); valid while phi is the phases that step wrote.  The next hot_gsw's first
+  bool once = false;  // in effect: the state keeps unit phasors (accurate and fast, M <= hot::kOnceMaxM)
+  hot::SubTile *tsub = nullptr;  // tiles (rows = row pairs)
+  int *tfirst = nullptr;         // [tgrid * (kWarps / tteam) + 1]
+  int tgrid = 0, tteam = 1, tpairs = 2;
+  // the unit phasors u_j = S_j/|S_j| of phi, written by the last step of a hot_gsw whose state
+  // keeps them (once); valid while phi is the phases that step wrote.  The next hot_gsw's first
   // forward field then reads them (gsw_from_u) and so adds the terms an uninterrupted run adds.
   float2 *ubuf = nullptr;  // [N]
   bool u_valid = false, gsw_from_u = false;
@@ -97,8 +94,10 @@ struct hot_ctx {
   float *Xt = nullptr, *Yt = nullptr, *Xr = nullptr, *Yr = nullptr;  // tables
   float *Y4t = nullptr, *Y4r = nullptr;  // [4][M][ldy4] shifted row tables (hot::StepArgs::Y4)
   int ldy4 = 0;
-  float2 *Xc = nullptr, *Yc = nullptr;                               // complex tables (separable)
-  float2 *Yc2 = nullptr;  // [2][M][ldy4] row-shifted copies of Yc (hot::StepArgs::Yc)
+  float2 *Xc = nullptr, *Yc = nullptr;                               // complex tables (tensor mode)
+  float2 *Xq = nullptr;   // the tile kernels' tables (hot::TileArgs)
+  float4 *Yq = nullptr;
+  int Mp = 0, ldp = 0;
   float *w = nullptr;                                          // [2][M] weights (home: w[0])
   unsigned long long *acc = nullptr;                           // [3][copies][2][M] fixed-point field sums
   long long *Vsum = nullptr;                                   // [2][M] sums of the last forward
@@ -142,17 +141,23 @@ namespace {
 
 bool finite_pos(double v) { return std::isfinite(v) && v > 0; }
 
-// Copies of each fixed-point accumulator buffer (StepArgs::copies).  With few traps all blocks
-// add into the same 2M addresses at nearly the same moment; 8 copies (block b adds into copy
-// b % 8) spread those atomics.  The separable kernel reads the copies; the direct kernels,
-// whose registers are fully used, keep one.  Storage is sized for the largest count.
-int acc_copies(const hot_ctx *c) { return (c->precision == HOT_PREC_SEPARABLE && c->M <= 512) ? 8 : 1; }
-
-// Modes whose step kernels are the separable ones: HOT_PREC_SEPARABLE, and HOT_PREC_TENSOR for
+// Modes whose kernels evaluate no pair exponential: HOT_PREC_SEPARABLE, and HOT_PREC_TENSOR for
 // every launch outside the GSW loop (forward field and adjoint of given phases, superposition).
 bool separable_kernels(const hot_ctx *c) {
   return c->precision == HOT_PREC_SEPARABLE || c->precision == HOT_PREC_TENSOR;
 }
+// The register-tiled kernels (otherwise the direct step kernels, on request: hot_set_once).
+bool tile_kernels(const hot_ctx *c) { return separable_kernels(c) || c->once_req; }
+
+// Copies of each fixed-point accumulator buffer (StepArgs::copies).  With few traps all blocks
+// add into the same 2M addresses at nearly the same moment; 8 copies (block b adds into copy
+// b % 8) spread those atomics.  The tile kernels read the copies; the direct kernels,
+// whose registers are fully used, and the tensor-core kernels keep one.  Storage is sized for the
+// largest count.
+int acc_copies(const hot_ctx *c) {
+  return (c->precision != HOT_PREC_TENSOR && tile_kernels(c) && c->M <= 512) ? 8 : 1;
+}
+
 size_t acc_elems(int M) { return 6 * (size_t)M * (M <= 512 ? 8 : 1); }
 
 // Pixels of the whole hologram (all row bands): the normalisation 1/N of Eq. 1.
@@ -183,7 +188,8 @@ void free_traps(hot_ctx *c) {
   dfree(c->Y4r);
   dfree(c->Xc);
   dfree(c->Yc);
-  dfree(c->Yc2);
+  dfree(c->Xq);
+  dfree(c->Yq);
   dfree(c->w);
   dfree(c->acc);
   dfree(c->Vsum);
@@ -269,8 +275,6 @@ hot::StepArgs make_step_args(const hot_ctx *c, int k, const float *phi, const fl
   a.Y = fast ? c->Yr : c->Yt;
   a.Y4 = fast ? c->Y4r : c->Y4t;
   a.ldy4 = c->ldy4;
-  a.Xc = c->Xc;
-  a.Yc = c->Yc2;
   a.phi = c->phi;
   const size_t M2 = 2 * (size_t)c->M * acc_copies(c);
   a.copies = acc_copies(c);
@@ -292,11 +296,8 @@ hot::StepArgs make_step_args(const hot_ctx *c, int k, const float *phi, const fl
   return a;
 }
 
-// Traps staged at once by the separable kernel (its shared memory is sized by it).
-int sep_chunk(const hot_ctx *c) { return std::max(1, std::min(c->M, c->tile_chunk)); }
-
 template <bool FAST, bool BACK, bool FWD, bool ADJ = false>
-int launch_tile(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const float2 *G = nullptr,
+int launch_direct(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const float2 *G = nullptr,
                 float *grad = nullptr) {
   const hot::StepArgs a = make_step_args(c, k, phi, G, grad);
   const int smem = hot::step_smem_bytes(c->M, BACK);
@@ -310,29 +311,33 @@ int launch_tile(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const f
   return check_launch(c, "gsw_step_kernel");
 }
 
-template <bool BACK, bool FWD, bool ADJ = false>
-int launch_sep(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const float2 *G = nullptr,
-               float *grad = nullptr) {
-  hot::StepArgs a = make_step_args(c, k, phi, G, grad);
-  a.chunk = sep_chunk(c);
-  Probe p(c, BACK && FWD ? HOT_KERNEL_STEP : FWD ? HOT_KERNEL_FORWARD : HOT_KERNEL_OTHER);
-  launch(c, hot::gsw_sep_kernel<BACK, FWD, ADJ>, c->grid, hot::kThreads, hot::sep_smem_bytes(a.chunk), pdl, a);
-  return check_launch(c, "gsw_sep_kernel");
+// Parameters of a tile-kernel launch: launch k of a sequence (make_step_args).
+hot::TileArgs make_tile_args(const hot_ctx *c, int k, const float *phi, const float2 *G, float *grad) {
+  hot::TileArgs t = {};
+  t.s = make_step_args(c, k, phi, G, grad);
+  t.s.sub = c->tsub;
+  t.s.first = c->tfirst;
+  t.X = c->Xq;
+  t.Y = c->Yq;
+  t.Mp = c->Mp;
+  t.ldp = c->ldp;
+  t.team = c->tteam;
+  t.pairs = c->tpairs;
+  return t;
 }
 
-// The one-exponential step (BACK: weight update, back-projection and forward field) or its
-// forward field of given phases, on the context's one-exponential schedule.
-template <bool BACK>
-int launch_once(hot_ctx *c, bool pdl, int k, const float *phi, bool last) {
-  hot::StepArgs a = make_step_args(c, k, phi, nullptr, nullptr);
-  a.u = c->ubuf;
-  a.once_flags = (last ? hot::kOnceLast : 0) | (!BACK && !phi && c->gsw_from_u ? hot::kOnceReadU : 0);
-  a.sub = BACK ? c->osub : c->ofsub;
-  a.first = BACK ? c->ofirst : c->offirst;
-  a.chunk = c->M;
-  Probe p(c, BACK ? HOT_KERNEL_STEP : HOT_KERNEL_FORWARD);
+// last: the last launch of a call (with unit phasors as the state, phases are written only then).
+template <bool BACK, bool FWD, bool ADJ = false>
+int launch_tile(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const float2 *G = nullptr,
+                float *grad = nullptr, bool last = true) {
+  hot::TileArgs t = make_tile_args(c, k, phi, G, grad);
+  if (c->once && FWD) {
+    t.s.u = c->ubuf;
+    t.s.once_flags = BACK ? hot::kOnceState | (last ? hot::kOnceLast : 0) : !phi && c->gsw_from_u ? hot::kOnceReadU : 0;
+  }
+  Probe p(c, BACK && FWD ? HOT_KERNEL_STEP : FWD ? HOT_KERNEL_FORWARD : HOT_KERNEL_OTHER);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(c->ogrid);
+  cfg.gridDim = dim3(c->tgrid);
   cfg.blockDim = dim3(hot::kThreads);
   cfg.stream = c->st;
   cudaLaunchAttribute attr[1];
@@ -340,23 +345,17 @@ int launch_once(hot_ctx *c, bool pdl, int k, const float *phi, bool last) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  hot_once::launch_step(c->once, c->precision == HOT_PREC_FAST, BACK, cfg, a);
-  return check_launch(c, "gsw_once_kernel");
+  hot_tile::launch(BACK, FWD, ADJ, cfg, t);
+  return check_launch(c, "gsw_tile_kernel");
 }
 
-// The step kernel of the context's mode (accurate / fast direct evaluation, or separable).
+// The kernel of the context's mode: register-tiled, or the direct step kernels.
 template <bool BACK, bool FWD, bool ADJ = false>
 int launch_mode(hot_ctx *c, bool pdl, int k, const float *phi = nullptr, const float2 *G = nullptr,
                 float *grad = nullptr, bool last = true) {
-  if (separable_kernels(c)) return launch_sep<BACK, FWD, ADJ>(c, pdl, k, phi, G, grad);
-  if (c->once && FWD && !ADJ && !G) {
-    // the forward field a call opens with, of phases the caller set: the separable kernel
-    // (complex tables, FMA only) at about half the cost of evaluating every exponential
-    if (!BACK && !phi && !c->gsw_from_u) return launch_sep<false, true>(c, pdl, k);
-    return launch_once<BACK>(c, pdl, k, phi, last);
-  }
-  if (c->precision == HOT_PREC_FAST) return launch_tile<true, BACK, FWD, ADJ>(c, pdl, k, phi, G, grad);
-  return launch_tile<false, BACK, FWD, ADJ>(c, pdl, k, phi, G, grad);
+  if (tile_kernels(c)) return launch_tile<BACK, FWD, ADJ>(c, pdl, k, phi, G, grad, last);
+  if (c->precision == HOT_PREC_FAST) return launch_direct<true, BACK, FWD, ADJ>(c, pdl, k, phi, G, grad);
+  return launch_direct<false, BACK, FWD, ADJ>(c, pdl, k, phi, G, grad);
 }
 
 // Raises the dynamic shared-memory limit of every step-kernel variant to what M needs.
@@ -374,24 +373,17 @@ int set_step_smem(int M) {
   HOT_CUDA(cudaFuncSetAttribute(hot::gsw_step_kernel<false, true, true, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * back));
   HOT_CUDA(cudaFuncSetAttribute(hot::gsw_step_kernel<true, true, true, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * back));
   HOT_CUDA(cudaFuncSetAttribute(hot::gsw_step_kernel<false, true, true, false, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * back));
-  const int sep = hot::sep_smem_bytes(hot::kChunk);
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_sep_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sep));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_sep_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sep));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_sep_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sep));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_sep_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sep));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_persistent_kernel<hot::kModeAccurate>, cudaFuncAttributeMaxDynamicSharedMemorySize, back));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_persistent_kernel<hot::kModeFast>, cudaFuncAttributeMaxDynamicSharedMemorySize, back));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_persistent_kernel<hot::kModeSeparable>, cudaFuncAttributeMaxDynamicSharedMemorySize, sep));
+  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_persistent_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, back));
+  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_persistent_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, back));
   return HOT_OK;
 }
 
 // The W/32 x H row segments dealt out to G blocks in equal contiguous runs (to within one
-// segment), each run cut into sub-tiles of at most `rows` rows -- evenly, or (full) into
-// sub-tiles of exactly `rows` rows and one shorter remainder; block b walks sub-tiles
-// first[b] .. first[b + 1] - 1.
+// segment), each run cut evenly into sub-tiles of at most `rows` rows; block b walks sub-tiles
+// first[b] .. first[b + 1] - 1.  (The tile kernels: strips of kTileCols columns, H in row pairs.)
 void cut_schedule(int W, int H, int G, int rows, std::vector<hot::SubTile> &sub, std::vector<int> &first,
-                  bool full = false) {
-  const int strips = (W + hot::kTileW - 1) / hot::kTileW;
+                  int strip_cols = hot::kTileW) {
+  const int strips = (W + strip_cols - 1) / strip_cols;
   const long long U = (long long)strips * H;
   sub.clear();
   first.assign(G + 1, 0);
@@ -405,9 +397,8 @@ void cut_schedule(int W, int H, int G, int rows, std::vector<hot::SubTile> &sub,
       const int L = (int)(run_end - s);
       const int nsub = (L + rows - 1) / rows;
       for (int i = 0; i < nsub; i++) {
-        const int r0 = row + (full ? i * rows : (int)((long long)L * i / nsub));
-        const int r1 = full ? std::min(r0 + rows, row + L) : row + (int)((long long)L * (i + 1) / nsub);
-        sub.push_back({strip * hot::kTileW, r0, r1 - r0, 0});
+        const int r0 = row + (int)((long long)L * i / nsub), r1 = row + (int)((long long)L * (i + 1) / nsub);
+        sub.push_back({strip * strip_cols, r0, r1 - r0, 0});
       }
       s = run_end;
     }
@@ -415,51 +406,66 @@ void cut_schedule(int W, int H, int G, int rows, std::vector<hot::SubTile> &sub,
   first[G] = (int)sub.size();
 }
 
-// The one-exponential step's schedule (one wave of its blocks, sub-tiles of its R rows), when
-// the context's mode and trap count allow it and it is requested; otherwise c->once = 0.
-int build_once_schedule(hot_ctx *c, int sms) {
-  c->once = 0;
-  c->ogrid = 0;
-  c->on_sub = 0;
-  dfree(c->osub);
-  dfree(c->ofirst);
-  dfree(c->ofsub);
-  dfree(c->offirst);
-  const int shape = hot::once_shape(c->M);
-  if (!c->once_req || !shape || (c->precision != HOT_PREC_FAST && c->precision != HOT_PREC_ACCURATE)) return HOT_OK;
-  int per_sm = 0, rc = HOT_OK;
-  HOT_CUDA(hot_once::occupancy(shape, &per_sm));
-  if (per_sm < 1) return HOT_OK;  // no room: the direct kernels
-  const long long U = (long long)((c->W + hot::kTileW - 1) / hot::kTileW) * c->H;
-  const int G = (int)std::min<long long>((long long)sms * per_sm, U);
+// Warps that share a tile of the tile kernels (hot::TileArgs::team).  A warp's step over two traps
+// costs about its row pairs + 4 (the fixed part: ring, column phasors, lane sums), so tiles want to
+// be tall; few warps per tile make the exchange of partial superpositions cheap.  Hence the smallest
+// team that still gets 6 row pairs.  us per iteration with 2 / 4 / 8 warps: 512^2, M = 100
+// 24.9 / 17.8 / 15.9; 768^2, M = 100 40.6 / 32.8 / 35.6; 801 x 603, M = 37 17.9 / 15.6 / 17.7;
+// 1920 x 1152, M = 100 101 / 104 / 110 (1 warp: 106).  At most 128 traps of a sum are added in a
+// row (FP32 rounding; 1920 x 1152, M = 1000: 914 / 883 / 866), and every warp gets a trap pair.
+int tile_team(int M, long long row_pairs, int sms) {
+  int team = hot::kWarps;
+  while (team > 2 && row_pairs * (team / 2) >= 6LL * sms * 2 * hot::kWarps && M <= 128 * (team / 2)) team /= 2;
+  while (team > 2 && (M + 1) / 2 < team) team /= 2;
+  return team;
+}
+
+// The tile kernels' schedule: one wave of their blocks, the strips' row pairs dealt out to the
+// teams in equal runs, cut into tiles of at most hot::kTilePairs pairs.
+int build_tile_schedule(hot_ctx *c, int sms) {
+  c->once = false;
+  c->tgrid = 0;
+  dfree(c->tsub);
+  dfree(c->tfirst);
+  if (!tile_kernels(c)) return HOT_OK;
+  const int P = (c->H + 1) / 2;
+  const long long U = (long long)((c->W + hot::kTileCols - 1) / hot::kTileCols) * P;
+  const int team = tile_team(c->M, U, sms), teams = hot::kWarps / team;
   std::vector<hot::SubTile> sub;
   std::vector<int> first;
-  std::vector<hot::SubTile> fsub;
-  std::vector<int> ffirst;
-  cut_schedule(c->W, c->H, G, hot::once_rows(shape), sub, first, true);
-  cut_schedule(c->W, c->H, G, hot::kOnceFwdRows, fsub, ffirst, true);
-  rc = dalloc(&c->osub, sub.size());
-  if (rc == HOT_OK) rc = dalloc(&c->ofirst, first.size());
-  if (rc == HOT_OK) rc = dalloc(&c->ofsub, fsub.size());
-  if (rc == HOT_OK) rc = dalloc(&c->offirst, ffirst.size());
+  int G = 0, pairs = 0, per_sm = 0;
+  // two blocks per SM, or the one that fits beside very many traps' coefficients
+  for (int want = 2; want >= 1; want--) {
+    G = (int)std::min<long long>((long long)sms * want, (U + teams - 1) / teams);
+    cut_schedule(c->W, P, G * teams, hot::kTilePairs, sub, first, hot::kTileCols);
+    pairs = 2;
+    for (hot::SubTile &t : sub) {
+      t.y0 *= 2;
+      pairs = std::max(pairs, t.rows);
+    }
+    HOT_CUDA(hot_tile::occupancy(c->M, pairs, &per_sm));
+    if (per_sm >= want) break;
+  }
+  if (per_sm < 1) return fail(HOT_ECUDA, "no tile kernel for %d traps", c->M);
+  int rc = dalloc(&c->tsub, sub.size());
+  if (rc == HOT_OK) rc = dalloc(&c->tfirst, first.size());
   if (rc != HOT_OK) return rc;
-  HOT_CUDA(cudaMemcpy(c->osub, sub.data(), sizeof(hot::SubTile) * sub.size(), cudaMemcpyHostToDevice));
-  HOT_CUDA(cudaMemcpy(c->ofirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
-  HOT_CUDA(cudaMemcpy(c->ofsub, fsub.data(), sizeof(hot::SubTile) * fsub.size(), cudaMemcpyHostToDevice));
-  HOT_CUDA(cudaMemcpy(c->offirst, ffirst.data(), sizeof(int) * ffirst.size(), cudaMemcpyHostToDevice));
-  if (!c->ubuf) {
+  HOT_CUDA(cudaMemcpy(c->tsub, sub.data(), sizeof(hot::SubTile) * sub.size(), cudaMemcpyHostToDevice));
+  HOT_CUDA(cudaMemcpy(c->tfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+  c->once = !separable_kernels(c) && c->M <= hot::kOnceMaxM;
+  if (c->once && !c->ubuf) {
     rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
     if (rc != HOT_OK) return rc;
   }
-  c->ogrid = G;
-  c->on_sub = (int)sub.size();
-  c->once = shape;
+  c->tgrid = G;
+  c->tteam = team;
+  c->tpairs = pairs;
   return HOT_OK;
 }
 
 // One wave of persistent blocks (SMs x resident blocks per SM: as many as fit, at most
 // tile_bps); the W/32 x H row segments are dealt out in equal contiguous runs, cut into
-// sub-tiles of <= tile_rows rows.  Also the one-exponential step's schedule.
+// sub-tiles of <= tile_rows rows.  Also the tile kernels' schedule.
 int build_schedule(hot_ctx *c) {
   drop_graphs(c);  // graphs hold the old schedule
   int rc = set_step_smem(c->M);
@@ -469,19 +475,14 @@ int build_schedule(hot_ctx *c) {
   // the per-iteration and the persistent kernels share the schedule (so that they compute the
   // same bits): as many blocks per SM as both can keep resident
   int per_sm_p = 0;
-  if (separable_kernels(c)) {
-    const int smem = hot::sep_smem_bytes(sep_chunk(c));
-    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_sep_kernel<true, true>, hot::kThreads, smem));
-    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_p, hot::gsw_persistent_kernel<hot::kModeSeparable>,
-                                                           hot::kThreads, smem));
-  } else {
+  {
     const int smem = hot::step_smem_bytes(c->M, true);
     HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_step_kernel<true, true, true>,
                                                            hot::kThreads, smem));
-    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_p, hot::gsw_persistent_kernel<hot::kModeFast>,
+    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_p, hot::gsw_persistent_kernel<true>,
                                                            hot::kThreads, smem));
     int per_sm_a = 0;
-    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, hot::gsw_persistent_kernel<hot::kModeAccurate>,
+    HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, hot::gsw_persistent_kernel<false>,
                                                            hot::kThreads, smem));
     per_sm_p = std::min(per_sm_p, per_sm_a);
   }
@@ -525,11 +526,11 @@ int build_schedule(hot_ctx *c) {
   HOT_CUDA(cudaMemcpy(c->first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
   c->grid = G;
   c->n_sub = (int)sub.size();
-  return build_once_schedule(c, sms);
+  return build_tile_schedule(c, sms);
 }
 
 // One step-kernel launch (launch k of the sequence): weight update + back-projection and/or
-// forward field.  last: the last launch of a call (the one-exponential step writes the phases only
+// forward field.  last: the last launch of a call (with unit phasors as the state the phases are written only
 // then; every other kernel writes them at each launch).
 int launch_step(hot_ctx *c, bool back, bool fwd, bool pdl, int k, bool last = true) {
   if (back && fwd) return launch_mode<true, true>(c, pdl, k, nullptr, nullptr, nullptr, last);
@@ -565,7 +566,7 @@ int launch_build_tables(hot_ctx *c) {
   const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   Probe p(c, HOT_KERNEL_OTHER);
   hot::build_tables_kernel<<<blocks, 256, 0, c->st>>>(c->W, c->H, c->H_total, c->y_off, c->M, c->abc, c->Xt, c->Yt,
-                                                      c->Xr, c->Yr, c->Xc, c->Yc, c->Y4t, c->Y4r, c->ldy4, c->Yc2);
+                                                      c->Xr, c->Yr, c->Xc, c->Yc, c->Y4t, c->Y4r, c->ldy4, c->Xq, c->Yq, c->Mp, c->ldp);
   int rc = check_launch(c, "build_tables_kernel");
   if (rc == HOT_OK && c->tc) {  // the tensor-core operands derive from the tables
     cudaError_t e = hot_tc::plan_refresh(c->tc, c->st);
@@ -619,22 +620,9 @@ int launch_tc(hot_ctx *c, bool pdl, int k) {
 // The whole sequence of enqueue_gsw's step launches as one cooperative launch (all blocks
 // resident; the grid is one wave by construction of the schedule).
 int launch_persistent(hot_ctx *c, int iters) {
-  hot::PersistArgs p = {};
-  for (int j = 0; j < 6; j++) {
-    p.step[j] = make_step_args(c, j, nullptr, nullptr, nullptr);
-    if (c->precision == HOT_PREC_SEPARABLE) p.step[j].chunk = sep_chunk(c);
-  }
-  if (c->once)
-    for (int j = 0; j < 6; j++) p.step[j].u = c->ubuf;
-  p.step[0].once_flags = c->gsw_from_u ? hot::kOnceReadU : 0;  // launch 0: the forward field of phi
-  p.k0 = 0;
-  p.iters = iters;
-  p.trace = c->tracing ? c->trace : nullptr;
-  p.sync.count = c->sync;
-  p.sync.err = reinterpret_cast<int *>(c->sync + 2);
-  p.sync.limit_ns = (long long)(c->wait_limit_s * 1e9);
+  const hot::GridSync sync = {c->sync, reinterpret_cast<int *>(c->sync + 2), (long long)(c->wait_limit_s * 1e9)};
+  float *const trace = c->tracing ? c->trace : nullptr;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(c->grid);
   cfg.blockDim = dim3(hot::kThreads);
   cfg.stream = c->st;
   cudaLaunchAttribute attr[1];
@@ -644,29 +632,31 @@ int launch_persistent(hot_ctx *c, int iters) {
   cfg.numAttrs = 1;
   HOT_CUDA(cudaMemsetAsync(c->sync, 0, sizeof(unsigned int), c->st));  // arrival count
   Probe probe(c, HOT_KERNEL_STEP);
-  if (c->once) {
-    if (!c->gsw_from_u) {  // launch 0 as in enqueue_gsw: the separable forward field of phi
-      const int rc = launch_sep<false, true>(c, false, 0);
-      if (rc != HOT_OK) return rc;
-      p.k0 = 1;
-    }
+  if (tile_kernels(c)) {
+    hot::TilePersistArgs p = {};
     for (int j = 0; j < 6; j++) {
-      p.step[j].sub = c->osub;
-      p.step[j].first = c->ofirst;
-      p.step[j].chunk = c->M;
+      p.step[j] = make_tile_args(c, j, nullptr, nullptr, nullptr);
+      if (c->once) p.step[j].s.u = c->ubuf;
+      p.step[j].s.once_flags = (c->once ? hot::kOnceState : 0) | (c->gsw_from_u ? hot::kOnceReadU : 0);
     }
-    cfg.gridDim = dim3(c->ogrid);
-    hot_once::launch_persistent(c->once, c->precision == HOT_PREC_FAST, cfg, p);
-  } else if (c->precision == HOT_PREC_SEPARABLE) {
-    cfg.dynamicSmemBytes = hot::sep_smem_bytes(sep_chunk(c));
-    cudaLaunchKernelEx(&cfg, hot::gsw_persistent_kernel<hot::kModeSeparable>, p);
-  } else if (c->precision == HOT_PREC_FAST) {
-    cfg.dynamicSmemBytes = hot::step_smem_bytes(c->M, true);
-    cudaLaunchKernelEx(&cfg, hot::gsw_persistent_kernel<hot::kModeFast>, p);
-  } else {
-    cfg.dynamicSmemBytes = hot::step_smem_bytes(c->M, true);
-    cudaLaunchKernelEx(&cfg, hot::gsw_persistent_kernel<hot::kModeAccurate>, p);
+    p.iters = iters;
+    p.sync = sync;
+    p.trace = trace;
+    cfg.gridDim = dim3(c->tgrid);
+    hot_tile::launch_persistent(cfg, p);
+    return check_launch(c, "gsw_tile_persistent_kernel");
   }
+  hot::PersistArgs p = {};
+  for (int j = 0; j < 6; j++) p.step[j] = make_step_args(c, j, nullptr, nullptr, nullptr);
+  p.iters = iters;
+  p.trace = trace;
+  p.sync = sync;
+  cfg.gridDim = dim3(c->grid);
+  cfg.dynamicSmemBytes = hot::step_smem_bytes(c->M, true);
+  if (c->precision == HOT_PREC_FAST)
+    cudaLaunchKernelEx(&cfg, hot::gsw_persistent_kernel<true>, p);
+  else
+    cudaLaunchKernelEx(&cfg, hot::gsw_persistent_kernel<false>, p);
   return check_launch(c, "gsw_persistent_kernel");
 }
 
@@ -801,10 +791,8 @@ void hot_destroy(hot_ctx *c) {
   dfree(c->phi);
   dfree(c->sub);
   dfree(c->first);
-  dfree(c->osub);
-  dfree(c->ofirst);
-  dfree(c->ofsub);
-  dfree(c->offirst);
+  dfree(c->tsub);
+  dfree(c->tfirst);
   dfree(c->ubuf);
   dfree(c->metrics);
   dfree(c->u8);
@@ -864,9 +852,16 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
       rc = fail(HOT_ECUDA, "hot_set_traps: clearing the shifted row tables failed");
     if (rc == HOT_OK) rc = dalloc(&c->Xc, (size_t)M * c->W);
     if (rc == HOT_OK) rc = dalloc(&c->Yc, (size_t)M * c->H);
-    if (rc == HOT_OK) rc = dalloc(&c->Yc2, 2 * (size_t)M * c->ldy4);
-    if (rc == HOT_OK && cudaMemsetAsync(c->Yc2, 0, sizeof(float2) * 2 * (size_t)M * c->ldy4, c->st) != cudaSuccess)
-      rc = fail(HOT_ECUDA, "hot_set_traps: clearing the shifted complex row table failed");
+    // the tile kernels' tables, zero past the image: whole strips, whole trap pairs, row pairs read
+    // kTilePairs at a time
+    const size_t nx = (size_t)((c->W + hot::kTileCols - 1) / hot::kTileCols) * hot::kTileCols;
+    c->Mp = (M + 1) & ~1;
+    c->ldp = (c->H + 1) / 2 + hot::kTilePairs;
+    if (rc == HOT_OK) rc = dalloc(&c->Xq, c->Mp * nx);
+    if (rc == HOT_OK) rc = dalloc(&c->Yq, (size_t)c->Mp * c->ldp);
+    if (rc == HOT_OK && (cudaMemsetAsync(c->Xq, 0, sizeof(float2) * c->Mp * nx, c->st) != cudaSuccess ||
+                         cudaMemsetAsync(c->Yq, 0, sizeof(float4) * (size_t)c->Mp * c->ldp, c->st) != cudaSuccess))
+      rc = fail(HOT_ECUDA, "hot_set_traps: clearing the tile kernels' tables failed");
     if (rc == HOT_OK) rc = dalloc(&c->w, 2 * (size_t)M);
     if (rc == HOT_OK) rc = dalloc(&c->acc, acc_elems(M));
     if (rc == HOT_OK) rc = dalloc(&c->Vsum, 2 * (size_t)M);
@@ -924,10 +919,9 @@ int hot_set_precision(hot_ctx *c, int precision) {
       precision != HOT_PREC_TENSOR)
     return fail(HOT_EINVAL, "hot_set_precision: unknown mode %d", precision);
   const bool was_sep = separable_kernels(c);
-  const bool copies_change = (precision == HOT_PREC_SEPARABLE) != (c->precision == HOT_PREC_SEPARABLE);
-  if (was_sep != (precision == HOT_PREC_SEPARABLE || precision == HOT_PREC_TENSOR) || copies_change)
-    HOT_CUDA(cudaStreamSynchronize(c->st));
   const bool resched = was_sep != (precision == HOT_PREC_SEPARABLE || precision == HOT_PREC_TENSOR);
+  const bool copies_change = (precision == HOT_PREC_TENSOR) != (c->precision == HOT_PREC_TENSOR);
+  if (resched || copies_change) HOT_CUDA(cudaStreamSynchronize(c->st));
   c->precision = precision;
   c->u_valid = false;
   if (resched && c->M) return build_schedule(c);  // the two kernels' occupancies differ
@@ -957,13 +951,13 @@ int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
     c->trace_iters = iters;
   }
   const bool had_u = c->u_valid;
-  c->gsw_from_u = c->u_valid && c->once && c->ubuf;
+  c->gsw_from_u = c->u_valid && c->once;
   c->u_valid = false;
   const int rc = (c->use_graphs && !c->profiling && !c->persistent) ? launch_gsw_graph(c, iters) : enqueue_gsw(c, iters);
   c->gsw_from_u = false;
   if (rc != HOT_OK) return rc;
-  // the last step of the one-exponential form left u_j of the phases it wrote in ubuf
-  c->u_valid = iters > 0 ? c->once && c->ubuf : had_u;
+  // where the state keeps unit phasors, the last step left u_j of the phases it wrote in ubuf
+  c->u_valid = iters > 0 ? c->once : had_u;
   c->have_fields = true;
   if (eff_out || unif_out) {
     if (c->persistent || c->precision == HOT_PREC_TENSOR) {
@@ -1253,7 +1247,7 @@ int hot_get_phasors(hot_ctx *c, float *u) {
   if (!c || !u) return fail(HOT_EINVAL, "hot_get_phasors: NULL argument");
   if (!c->M) return fail(HOT_ESTATE, "hot_get_phasors: no traps set");
   if (!c->u_valid)
-    return fail(HOT_ESTATE, "hot_get_phasors: no unit phasors of the current phases (a one-exponential hot_gsw leaves them)");
+    return fail(HOT_ESTATE, "hot_get_phasors: no unit phasors of the current phases (hot_gsw leaves them in the accurate and fast modes with up to 128 traps)");
   const int rc = check_wait_error(c, "hot_get_phasors");
   if (rc != HOT_OK) return rc;
   HOT_CUDA(cudaMemcpyAsync(u, c->ubuf, sizeof(float2) * (size_t)c->W * c->H, cudaMemcpyDeviceToHost, c->st));
@@ -1264,7 +1258,7 @@ int hot_get_phasors(hot_ctx *c, float *u) {
 int hot_set_phasors(hot_ctx *c, const float *u) {
   if (!c || !u) return fail(HOT_EINVAL, "hot_set_phasors: NULL argument");
   if (!c->M) return fail(HOT_ESTATE, "hot_set_phasors: no traps set");
-  if (!c->once || !c->ubuf) return fail(HOT_ESTATE, "hot_set_phasors: the one-exponential step is not in effect");
+  if (!c->once) return fail(HOT_ESTATE, "hot_set_phasors: unit phasors are not in effect (hot_set_once)");
   const size_t n = 2 * (size_t)c->W * c->H;
   for (size_t i = 0; i < n; i++)
     if (!std::isfinite(u[i]) || std::fabs(u[i]) > 2.f)
@@ -1348,7 +1342,8 @@ struct hot_batch {
     hot::SubTile *sub = nullptr;
     int *first = nullptr;
     std::vector<int> owner;                  // block that writes each hologram's weights
-    std::vector<hot::StepArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
+    std::vector<hot::TileArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
+    int M = 1, pairs = 2;                    // shared-memory layout (hot::TileBatchArgs)
     hot::FinalizeArgs *fin[6] = {};          // finalize descriptors for iters % 6
   };
   std::vector<Group> groups;
@@ -1370,44 +1365,13 @@ struct hot_batch {
 
 namespace {
 
-int batch_mode(const hot_batch *b) {
-  return b->precision == HOT_PREC_SEPARABLE ? hot::kModeSeparable
-                                            : b->precision == HOT_PREC_FAST ? hot::kModeFast : hot::kModeAccurate;
-}
-
-// Dynamic shared memory of the batch kernels: the separable one stages `chunk` complex traps.
-int batch_smem(const hot_batch *b) {
-  return b->precision == HOT_PREC_SEPARABLE ? hot::sep_smem_bytes(b->chunk) : hot::step_smem_bytes(0, true);
-}
-
-template <int MODE>
-int batch_set_smem() {
-  const int bytes = MODE == hot::kModeSeparable ? hot::sep_smem_bytes(hot::kChunk) : hot::step_smem_bytes(0, true);
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_batch_kernel<MODE, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_batch_kernel<MODE, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  return HOT_OK;
-}
-
-// Resident blocks per SM of the batch's fused kernel at its current staging chunk.
+// Resident blocks per SM of the batch's kernel, with shared memory for its largest trap count.
 int batch_occupancy(hot_batch *b) {
-  int per_sm = 0;
-  const int smem = batch_smem(b);
-  cudaError_t e;
-  switch (batch_mode(b)) {
-    case hot::kModeSeparable:
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeSeparable, true, true>,
-                                                        hot::kThreads, smem);
-      break;
-    case hot::kModeFast:
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeFast, true, true>,
-                                                        hot::kThreads, smem);
-      break;
-    default:
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeAccurate, true, true>,
-                                                        hot::kThreads, smem);
-  }
+  int M = 1;
+  for (const hot_ctx *c : b->ctx) M = std::max(M, c->M);
+  cudaError_t e = hot_tile::occupancy(M, hot::kTilePairs, &b->per_sm_max);
   if (e != cudaSuccess) return fail(HOT_ECUDA, "batch occupancy query: %s", cudaGetErrorString(e));
-  b->per_sm_max = per_sm < 1 ? 1 : per_sm;
+  if (b->per_sm_max < 1) b->per_sm_max = 1;
   return HOT_OK;
 }
 
@@ -1435,42 +1399,12 @@ void batch_free(hot_batch *b) {
   b->chain_ev.clear();
 }
 
-// Step-kernel parameters of context c for launch k of a sequence (buffers rotate as in hot_gsw).
-hot::StepArgs step_args(const hot_ctx *c, int k, int chunk) {
-  hot::StepArgs a = {};
-  const bool fast = c->precision == HOT_PREC_FAST;
-  const size_t M2 = 2 * (size_t)c->M * acc_copies(c);
-  a.W = c->W;
-  a.H = c->H;
-  a.M = c->M;
-  a.chunk = chunk;
-  a.copies = acc_copies(c);
-  a.X = fast ? c->Xr : c->Xt;
-  a.Y = fast ? c->Yr : c->Yt;
-  a.Y4 = fast ? c->Y4r : c->Y4t;
-  a.ldy4 = c->ldy4;
-  a.Xc = c->Xc;
-  a.Yc = c->Yc2;
-  a.phi = c->phi;
-  a.acc_in = c->acc + M2 * ((k + 2) % 3);
-  a.acc_out = c->acc + M2 * (k % 3);
-  a.acc_clear = c->acc + M2 * ((k + 1) % 3);
-  a.w_in = c->w + (size_t)c->M * ((k + 1) & 1);
-  a.w_out = c->w + (size_t)c->M * (k & 1);
-  a.fx_scale = ldexpf(1.0f, c->fx_shift);
-  a.inv_fx_n = (float)(1.0 / (n_total(c) * ldexp(1.0, c->fx_shift)));
-  a.angle_units = fast ? 1.0f : 0.15915494309189535f;
-  a.angle_eta = fast ? hot::kFastEta : 0.0f;
-  a.inv_n = (float)(1.0 / (n_total(c)));
-  return a;
-}
-
 double pairs_of(const hot_ctx *c) { return n_total(c) * (double)c->M; }
 
-// One group's work schedule: the row segments of its holograms in order, each weighted by its
-// trap count, dealt out to one wave of G blocks in equal shares (a segment goes to the block
-// that holds the midpoint of its weight interval); each block's run of rows in a strip is cut
-// into equal sub-tiles of <= rows rows.
+// One group's work schedule: the strips' row pairs of its holograms in order, each weighted by its
+// trap count, dealt out to one wave of G blocks in equal shares (a row pair goes to the block
+// that holds the midpoint of its weight interval); each block's run of pairs in a strip is cut
+// into equal tiles of <= rows / 2 pairs (the default 14: hot::kTilePairs).
 int build_group(hot_batch *b, hot_batch::Group &g) {
   const int count = (int)g.members.size();
   const int per_sm = b->bps > 0 ? std::min(b->bps, b->per_sm_max) : b->per_sm_max;
@@ -1478,10 +1412,12 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   long long segments = 0;
   for (int h : g.members) {
     const hot_ctx *c = b->ctx[h];
-    const long long seg = (long long)((c->W + hot::kTileW - 1) / hot::kTileW) * c->H;
+    const long long seg = (long long)((c->W + hot::kTileCols - 1) / hot::kTileCols) * ((c->H + 1) / 2);
     segments += seg;
     T += (long double)seg * c->M;
+    g.M = std::max(g.M, c->M);
   }
+  const int pairs = b->rows >= hot::kRowsMax ? hot::kTilePairs : (b->rows + 1) / 2;
   const int G = (int)std::min<long long>((long long)b->sms * per_sm, segments);
   std::vector<hot::SubTile> sub;
   std::vector<int> first(G + 1, 0), owner(count, -1);
@@ -1489,7 +1425,7 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   int cur_b = 0;
   for (int i = 0; i < count; i++) {
     const hot_ctx *c = b->ctx[g.members[i]];
-    const int strips = (c->W + hot::kTileW - 1) / hot::kTileW;
+    const int strips = (c->W + hot::kTileCols - 1) / hot::kTileCols, P = (c->H + 1) / 2;
     for (int s = 0; s < strips; s++) {
       auto block_of = [&](int row) {
         const long double mid = w0 + ((long double)row + 0.5L) * c->M;
@@ -1497,32 +1433,41 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
         return bb < 0 ? 0 : (bb >= G ? G - 1 : bb);
       };
       int r = 0;
-      while (r < c->H) {  // the run of rows of this strip that goes to block bb, cut evenly
+      while (r < P) {  // the run of row pairs of this strip that goes to block bb, cut evenly
         const int bb = block_of(r);
         int r1 = r + 1;
-        while (r1 < c->H && block_of(r1) == bb) r1++;
+        while (r1 < P && block_of(r1) == bb) r1++;
         while (cur_b < bb) first[++cur_b] = (int)sub.size();
         if (owner[i] < 0) owner[i] = bb;
-        const int L = r1 - r, nsub = (L + b->rows - 1) / b->rows;
+        const int L = r1 - r, nsub = (L + pairs - 1) / pairs;
         for (int q = 0; q < nsub; q++) {
           const int q0 = r + (int)((long long)L * q / nsub), q1 = r + (int)((long long)L * (q + 1) / nsub);
-          sub.push_back({s * hot::kTileW, q0, q1 - q0, i});
+          sub.push_back({s * hot::kTileCols, 2 * q0, q1 - q0, i});
+          g.pairs = std::max(g.pairs, q1 - q0);
         }
         r = r1;
       }
-      w0 += (long double)c->H * c->M;
+      w0 += (long double)P * c->M;
     }
   }
   while (cur_b < G) first[++cur_b] = (int)sub.size();
   g.grid = G;
   g.n_sub = (int)sub.size();
   g.owner = owner;
-  for (int k = 0; k < 6; k++) {
-    g.holo[k].resize(count);
-    for (int i = 0; i < count; i++) g.holo[k][i] = step_args(b->ctx[g.members[i]], k == 0 ? 6 : k, b->chunk);
-  }
   int rc = dalloc(&g.sub, sub.size());
   if (rc == HOT_OK) rc = dalloc(&g.first, first.size());
+  for (int k = 0; k < 6; k++) {
+    g.holo[k].resize(count);
+    for (int i = 0; i < count; i++) {
+      hot::TileArgs &t = g.holo[k][i];
+      t = make_tile_args(b->ctx[g.members[i]], k == 0 ? 6 : k, nullptr, nullptr, nullptr);
+      t.s.sub = g.sub;
+      t.s.first = g.first;
+      t.s.trace = nullptr;
+      t.team = hot::kWarps;
+      t.pairs = g.pairs;
+    }
+  }
   for (int r6 = 0; rc == HOT_OK && r6 < 6; r6++) {  // finalize after `iters` iterations, iters % 6 == r6
     rc = dalloc(&g.fin[r6], (size_t)count);
     std::vector<hot::FinalizeArgs> fs(count);
@@ -1592,34 +1537,31 @@ int batch_schedule(hot_batch *b) {
   return HOT_OK;
 }
 
-template <int MODE, bool BACK>
-int batch_launch(hot_batch *b, const hot_batch::Group &g, int k, bool pdl) {
-  hot::BatchArgs a = {};
+template <bool BACK>
+int batch_launch(hot_batch *b, const hot_batch::Group &g, int k) {
+  hot::TileBatchArgs a = {};
   const int count = (int)g.members.size();
   for (int i = 0; i < count; i++) {
     a.holo[i] = g.holo[k % 6][i];
     a.owner[i] = g.owner[i];
   }
-  a.sub = g.sub;
   a.first = g.first;
   a.count = count;
-  hot_ctx tmp;  // launch() needs a context only for the stream
-  tmp.st = b->st;
-  launch(&tmp, hot::gsw_batch_kernel<MODE, BACK, true>, g.grid, hot::kThreads, batch_smem(b), pdl, a);
+  a.M = g.M;
+  a.pairs = g.pairs;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.grid);
+  cfg.blockDim = dim3(hot::kThreads);
+  cfg.stream = b->st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  hot_tile::launch_batch(BACK, cfg, a);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_batch_kernel: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_tile_batch_kernel: %s", cudaGetErrorString(e));
   return HOT_OK;
-}
-
-// A start stamp, then the groups in order: forward field of the starting phases (k = 0),
-// iterations 1..iters, and the per-hologram finalize with its completion stamp.
-template <bool BACK>
-int batch_launch_mode(hot_batch *b, const hot_batch::Group &g, int k, bool pdl) {
-  switch (batch_mode(b)) {
-    case hot::kModeSeparable: return batch_launch<hot::kModeSeparable, BACK>(b, g, k, pdl);
-    case hot::kModeFast: return batch_launch<hot::kModeFast, BACK>(b, g, k, pdl);
-    default: return batch_launch<hot::kModeAccurate, BACK>(b, g, k, pdl);
-  }
 }
 
 constexpr int kTensorChains = 8;
@@ -1683,8 +1625,8 @@ int batch_enqueue(hot_batch *b, int iters) {
   if (e0 != cudaSuccess) return fail(HOT_ECUDA, "launch of stamp_kernel: %s", cudaGetErrorString(e0));
   for (size_t gi = 0; gi < b->groups.size(); gi++) {
     const hot_batch::Group &g = b->groups[gi];
-    int rc = batch_launch_mode<false>(b, g, 0, true);
-    for (int k = 1; k <= iters && rc == HOT_OK; k++) rc = batch_launch_mode<true>(b, g, k, true);
+    int rc = batch_launch<false>(b, g, 0);
+    for (int k = 1; k <= iters && rc == HOT_OK; k++) rc = batch_launch<true>(b, g, k);
     if (rc != HOT_OK) return rc;
     hot_ctx tmp;
     tmp.st = b->st;
@@ -1893,30 +1835,29 @@ int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chun
     return time_runs(c->st, iters, us, [&]() { return restore_state(c, saved, c->st); },
                      [&]() { return hot_gsw(c, iters, nullptr, nullptr); });
   };
-  // The one-exponential step, where it applies, against the best tiling of the direct kernels
-  // (which also serve the adjoint and the superposition).
-  const bool once_req = c->once_req;
-  double once_us = 0;
-  if (once_req && c->once) {
-    rc = timed_gsw(&once_us);
-    if (rc == HOT_OK) rc = hot_set_once(c, 0);
-  }
+  // The tile kernels, where they apply, against the best tiling of the direct kernels; the
+  // separable mode has no others.
+  const bool once_req = c->once_req, tile = tile_kernels(c);
   Tiling best = {c->tile_rows, c->sched_bps, c->tile_chunk, c->tile_merge};
-  double best_us = 0;
-  if (rc == HOT_OK) rc = tune_tiling(
-      kMaxBlocksPerSm, best, best_us,
-      [&](const Tiling &t) {
-        c->tile_merge = t.merge;  // applied by the schedule that hot_set_tiling rebuilds
-        return hot_set_tiling(c, t.rows, t.bps, t.chunk);
-      },
-      timed_gsw, !separable_kernels(c));
-  if (rc == HOT_OK && once_req && once_us > 0 && once_us < best_us) {
-    rc = hot_set_once(c, 1);
-    best_us = once_us;
-  } else if (once_req && once_us > 0) {
-    c->once_req = false;  // the direct kernels were faster (hot_get_once reports it)
-  } else if (rc != HOT_OK) {
-    c->once_req = once_req;
+  double best_us = 0, tile_us = 0;
+  if (tile) rc = timed_gsw(&tile_us);
+  if (separable_kernels(c)) {
+    best_us = tile_us;
+  } else {
+    if (rc == HOT_OK && tile) rc = hot_set_once(c, 0);
+    if (rc == HOT_OK) rc = tune_tiling(
+        kMaxBlocksPerSm, best, best_us,
+        [&](const Tiling &t) {
+          c->tile_merge = t.merge;  // applied by the schedule that hot_set_tiling rebuilds
+          return hot_set_tiling(c, t.rows, t.bps, t.chunk);
+        },
+        timed_gsw, true);
+    if (rc == HOT_OK && tile && tile_us < best_us) {
+      rc = hot_set_once(c, 1);
+      best_us = tile_us;
+    } else if (rc != HOT_OK) {
+      c->once_req = once_req;
+    }
   }
   c->profiling = profiling;
   const int rc2 = restore_state(c, saved, c->st);
@@ -1955,10 +1896,7 @@ int hot_batch_create(hot_batch **out, int count, hot_ctx *const *ctxs, void *cud
   b->precision = ctxs[0]->precision;
   b->dev = ctxs[0]->dev;
   const bool tensor = b->precision == HOT_PREC_TENSOR;
-  int rc = tensor                                     ? HOT_OK
-           : batch_mode(b) == hot::kModeSeparable ? batch_set_smem<hot::kModeSeparable>()
-           : batch_mode(b) == hot::kModeFast      ? batch_set_smem<hot::kModeFast>()
-                                                  : batch_set_smem<hot::kModeAccurate>();
+  int rc = HOT_OK;
   if (rc == HOT_OK && cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess)
     rc = fail(HOT_ECUDA, "hot_batch_create: device query failed");
   if (rc == HOT_OK) rc = dalloc(&b->stamps, (size_t)count + 1);

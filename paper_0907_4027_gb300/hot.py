@@ -285,7 +285,7 @@ def hot_get_block_merge(ctx: int) -> dict:
 
 
 def hot_set_once(ctx: int, on: bool) -> None:
-    """The one-exponential GSW step of the accurate and fast modes (M <= 128): on (default) or off."""
+    """Accurate and fast modes: the register-tiled kernels (default) or the direct step kernels (off)."""
     _ok(lib.hot_set_once(_vp(ctx), 1 if on else 0), "hot_set_once")
 
 
@@ -408,7 +408,7 @@ def hot_set_state(ctx: int, phi, w) -> None:
 
 
 def hot_get_phasors(ctx: int, N: int):
-    """The unit phasors the last one-exponential step left for the current phases (float32 [N][2]),
+    """The unit phasors the last step left for the current phases (float32 [N][2]),
     or None when there are none (HOT_ESTATE)."""
     u = np.empty(2 * N, dtype=np.float32)
     rc = lib.hot_get_phasors(_vp(ctx), u.ctypes.data_as(_vp))
@@ -579,7 +579,7 @@ class Hologram:
         return hot_get_trace(self.ctx, iters + 1)
 
     def get_state(self):
-        """(phi, w, u) host copies -- phases, weights and the unit phasors the last one-exponential
+        """(phi, w, u) host copies -- phases, weights and the unit phasors the last
         step left for them (None otherwise): resume elsewhere with set_state, bit for bit."""
         phi, w = hot_get_state(self.ctx, self.N, self.M)
         return phi, w, hot_get_phasors(self.ctx, self.N)
