@@ -78,9 +78,8 @@ struct hot_ctx {
   // unless hot_set_once turned them to the direct step kernels; their own schedule
   bool once_req = true;
   bool once = false;  // in effect: the state keeps unit phasors (accurate and fast, M <= hot::kOnceMaxM)
-  hot::SubTile *tsub = nullptr;  // tiles (rows = row pairs)
-  int *tfirst = nullptr;         // [tgrid * (kWarps / tteam) + 1]
-  int tgrid = 0, tteam = 1, tpairs = 2;
+  hot::SubTile *tsub = nullptr;  // [teams][tstride] (hot::TileArgs)
+  int tgrid = 0, tteam = 1, tpairs = 3, tstride = 1;
   // the unit phasors u_j = S_j/|S_j| of phi, written by the last step of a hot_gsw whose state
   // keeps them (once); valid while phi is the phases that step wrote.  The next hot_gsw's first
   // forward field then reads them (gsw_from_u) and so adds the terms an uninterrupted run adds.
@@ -316,7 +315,7 @@ hot::TileArgs make_tile_args(const hot_ctx *c, int k, const float *phi, const fl
   hot::TileArgs t = {};
   t.s = make_step_args(c, k, phi, G, grad);
   t.s.sub = c->tsub;
-  t.s.first = c->tfirst;
+  t.stride = c->tstride;
   t.X = c->Xq;
   t.Y = c->Yq;
   t.Mp = c->Mp;
@@ -406,18 +405,28 @@ void cut_schedule(int W, int H, int G, int rows, std::vector<hot::SubTile> &sub,
   first[G] = (int)sub.size();
 }
 
-// Warps that share a tile of the tile kernels (hot::TileArgs::team).  A warp's step over two traps
-// costs about its row pairs + 4 (the fixed part: ring, column phasors, lane sums), so tiles want to
-// be tall; few warps per tile make the exchange of partial superpositions cheap.  Hence the smallest
-// team that still gets 6 row pairs.  us per iteration with 2 / 4 / 8 warps: 512^2, M = 100
-// 24.9 / 17.8 / 15.9; 768^2, M = 100 40.6 / 32.8 / 35.6; 801 x 603, M = 37 17.9 / 15.6 / 17.7;
-// 1920 x 1152, M = 100 101 / 104 / 110 (1 warp: 106).  At most 128 traps of a sum are added in a
-// row (FP32 rounding; 1920 x 1152, M = 1000: 914 / 883 / 866), and every warp gets a trap pair.
+// Warps that share a tile of the tile kernels (hot::TileArgs::team): the cheapest by a model of a
+// team's time, in units of one warp step over two traps on one row pair.  A step costs its row pairs
+// + 4 (ring, column phasors, lane sums), a tile 2 per row pair + 6 (exchange of the partial
+// superpositions, phasors).  Measured us per iteration with 1 / 2 / 4 / 8 warps (the model's
+// choice in brackets): 256^2, M = 16 7.9 / 5.9 / 4.9 / [4.9]; 768^2, M = 8 8.3 / [8.5] / 9.4 / 12.3;
+// 801 x 603, M = 37 25 / 17.3 / [15.5] / 17.4; 768^2, M = 100 56 / 39 / [32] / 35; 512^2, M = 100
+// 40 / 24 / 17.4 / [15.9]; 1920 x 1152, M = 100 [103] / 98 / 101 / 107.  At most 128 traps are added
+// in a row (FP32 rounding of S_j).
 int tile_team(int M, long long row_pairs, int sms) {
-  int team = hot::kWarps;
-  while (team > 2 && row_pairs * (team / 2) >= 6LL * sms * 2 * hot::kWarps && M <= 128 * (team / 2)) team /= 2;
-  while (team > 2 && (M + 1) / 2 < team) team /= 2;
-  return team;
+  int best = hot::kWarps;
+  double best_cost = 1e300;
+  for (int team = hot::kWarps; team >= 1 && M <= 128 * team; team /= 2) {
+    const long long teams = 2LL * sms * (hot::kWarps / team);
+    const double run = (double)((row_pairs + teams - 1) / teams), n = std::ceil(run / hot::kTilePairs);
+    const double rp = std::ceil(run / n), steps = std::ceil((M + 1) / 2 / (double)team);
+    const double cost = n * (steps * (rp + 4) + 2 * rp + 6);
+    if (cost < best_cost) {
+      best = team;
+      best_cost = cost;
+    }
+  }
+  return best;
 }
 
 // The tile kernels' schedule: one wave of their blocks, the strips' row pairs dealt out to the
@@ -426,7 +435,6 @@ int build_tile_schedule(hot_ctx *c, int sms) {
   c->once = false;
   c->tgrid = 0;
   dfree(c->tsub);
-  dfree(c->tfirst);
   if (!tile_kernels(c)) return HOT_OK;
   const int P = (c->H + 1) / 2;
   const long long U = (long long)((c->W + hot::kTileCols - 1) / hot::kTileCols) * P;
@@ -438,23 +446,28 @@ int build_tile_schedule(hot_ctx *c, int sms) {
   for (int want = 2; want >= 1; want--) {
     G = (int)std::min<long long>((long long)sms * want, (U + teams - 1) / teams);
     cut_schedule(c->W, P, G * teams, hot::kTilePairs, sub, first, hot::kTileCols);
-    pairs = 2;
-    for (hot::SubTile &t : sub) {
-      t.y0 *= 2;
-      pairs = std::max(pairs, t.rows);
-    }
-    HOT_CUDA(hot_tile::occupancy(c->M, pairs, &per_sm));
+    pairs = 3;
+    for (const hot::SubTile &t : sub) pairs = std::max(pairs, t.rows);
+    HOT_CUDA(hot_tile::occupancy(c->M, team, pairs, &per_sm));
     if (per_sm >= want) break;
   }
   if (per_sm < 1) return fail(HOT_ECUDA, "no tile kernel for %d traps", c->M);
-  int rc = dalloc(&c->tsub, sub.size());
-  if (rc == HOT_OK) rc = dalloc(&c->tfirst, first.size());
-  if (rc != HOT_OK) return rc;
-  HOT_CUDA(cudaMemcpy(c->tsub, sub.data(), sizeof(hot::SubTile) * sub.size(), cudaMemcpyHostToDevice));
-  HOT_CUDA(cudaMemcpy(c->tfirst, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+  int stride = 1;
+  for (int i = 0; i < G * teams; i++) stride = std::max(stride, first[i + 1] - first[i]);
+  std::vector<hot::SubTile> tiles((size_t)G * teams * stride, hot::SubTile{0, 0, 0, 0});
+  for (int i = 0; i < G * teams; i++)
+    for (int j = first[i]; j < first[i + 1]; j++) {
+      hot::SubTile &t = tiles[(size_t)i * stride + j - first[i]] = sub[j];
+      t.y0 *= 2;
+      t.pad = first[i + 1] - j;
+    }
+  const int rc0 = dalloc(&c->tsub, tiles.size());
+  if (rc0 != HOT_OK) return rc0;
+  HOT_CUDA(cudaMemcpy(c->tsub, tiles.data(), sizeof(hot::SubTile) * tiles.size(), cudaMemcpyHostToDevice));
+  c->tstride = stride;
   c->once = !separable_kernels(c) && c->M <= hot::kOnceMaxM;
   if (c->once && !c->ubuf) {
-    rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
+    const int rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
     if (rc != HOT_OK) return rc;
   }
   c->tgrid = G;
@@ -792,7 +805,6 @@ void hot_destroy(hot_ctx *c) {
   dfree(c->sub);
   dfree(c->first);
   dfree(c->tsub);
-  dfree(c->tfirst);
   dfree(c->ubuf);
   dfree(c->metrics);
   dfree(c->u8);
@@ -1343,7 +1355,7 @@ struct hot_batch {
     int *first = nullptr;
     std::vector<int> owner;                  // block that writes each hologram's weights
     std::vector<hot::TileArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
-    int M = 1, pairs = 2;                    // shared-memory layout (hot::TileBatchArgs)
+    int M = 1, pairs = 3;                    // shared-memory layout (hot::TileBatchArgs)
     hot::FinalizeArgs *fin[6] = {};          // finalize descriptors for iters % 6
   };
   std::vector<Group> groups;
@@ -1369,7 +1381,7 @@ namespace {
 int batch_occupancy(hot_batch *b) {
   int M = 1;
   for (const hot_ctx *c : b->ctx) M = std::max(M, c->M);
-  cudaError_t e = hot_tile::occupancy(M, hot::kTilePairs, &b->per_sm_max);
+  cudaError_t e = hot_tile::occupancy(M, hot::kWarps, hot::kTilePairs, &b->per_sm_max);
   if (e != cudaSuccess) return fail(HOT_ECUDA, "batch occupancy query: %s", cudaGetErrorString(e));
   if (b->per_sm_max < 1) b->per_sm_max = 1;
   return HOT_OK;

@@ -31,9 +31,9 @@ cudaError_t set_smem() {
 
 }  // namespace
 
-cudaError_t occupancy(int M, int pairs, int *per_sm) {
+cudaError_t occupancy(int M, int team, int pairs, int *per_sm) {
   int a = 0, b = 0, c = 0;
-  const int smem = hot::tile_smem_bytes(M, pairs);
+  const int smem = hot::tile_smem_bytes(M, team, pairs);
   *per_sm = 0;
   cudaError_t e = set_smem();
   if (e == cudaSuccess)
@@ -47,7 +47,7 @@ cudaError_t occupancy(int M, int pairs, int *per_sm) {
 }
 
 cudaError_t launch(bool back, bool fwd, bool adj, cudaLaunchConfig_t cfg, const hot::TileArgs &a) {
-  cfg.dynamicSmemBytes = hot::tile_smem_bytes(a.s.M, a.pairs);
+  cfg.dynamicSmemBytes = hot::tile_smem_bytes(a.s.M, a.team, a.pairs);
   if (adj) return cudaLaunchKernelEx(&cfg, hot::gsw_tile_kernel<true, false, true>, a);
   if (back && fwd) return cudaLaunchKernelEx(&cfg, hot::gsw_tile_kernel<true, true, false>, a);
   if (back) return cudaLaunchKernelEx(&cfg, hot::gsw_tile_kernel<true, false, false>, a);
@@ -55,12 +55,12 @@ cudaError_t launch(bool back, bool fwd, bool adj, cudaLaunchConfig_t cfg, const 
 }
 
 cudaError_t launch_persistent(cudaLaunchConfig_t cfg, const hot::TilePersistArgs &p) {
-  cfg.dynamicSmemBytes = hot::tile_smem_bytes(p.step[0].s.M, p.step[0].pairs);
+  cfg.dynamicSmemBytes = hot::tile_smem_bytes(p.step[0].s.M, p.step[0].team, p.step[0].pairs);
   return cudaLaunchKernelEx(&cfg, hot::gsw_tile_persistent_kernel, p);
 }
 
 cudaError_t launch_batch(bool back, cudaLaunchConfig_t cfg, const hot::TileBatchArgs &b) {
-  cfg.dynamicSmemBytes = hot::tile_smem_bytes(b.M, b.pairs);
+  cfg.dynamicSmemBytes = hot::tile_smem_bytes(b.M, hot::kWarps, b.pairs);
   return back ? cudaLaunchKernelEx(&cfg, hot::gsw_tile_batch_kernel<true>, b)
               : cudaLaunchKernelEx(&cfg, hot::gsw_tile_batch_kernel<false>, b);
 }

@@ -8,7 +8,7 @@
 namespace hot_tile {
 
 // Blocks per SM that the step, the batched and the persistent kernel both keep resident (0: a block does not fit).
-cudaError_t occupancy(int M, int pairs, int *per_sm);
+cudaError_t occupancy(int M, int team, int pairs, int *per_sm);
 
 // One launch with the grid, block, stream and attributes of cfg (its dynamic shared memory is set
 // here): the GSW step (back, fwd), the field of given phases (fwd), a superposition (back) or the

@@ -31,30 +31,47 @@ constexpr int kTilePairs = 8;     // row pairs of a tile at most
 constexpr int kRing = 3;          // stages of a warp's table ring, two traps each
 constexpr int kStageX = kTileCols * 8, kStageY = kTilePairs * 16;  // bytes of a trap in a stage
 constexpr int kStageBytes = 2 * (kStageX + kStageY);
-constexpr int kSumGroup = 4;      // traps whose field sums a warp reduces together
+constexpr int kSumGroup = 8;      // traps whose field sums a warp reduces together
+constexpr int kSumStride = 36;    // ... and the stride of their lane sums: eight lanes' columns of four traps
+                                  // fall on different banks (33: 858 us per iteration at 1920 x 1152,
+                                  // M = 1000 in groups of 4; 36: 840)
 
 struct TileArgs {
-  StepArgs s;        // sub: tiles (rows = row pairs, y0 even), first: per team
+  StepArgs s;        // sub: tiles (rows = row pairs, y0 even)
   const float2 *X;   // [strips][Mp][kTileCols] column phasors of the 64-column strips, zero from W on
   const float4 *Y;   // [Mp][ldp] row phasors by row pair: (re, re, im, im), zero from H on
   int Mp, ldp;       // Mp: M rounded up to a whole number of trap pairs (the added trap: zeros)
   int team;          // warps that share a tile
-  int pairs;         // row pairs of the tallest tile, at least 2 (shared memory is sized by it)
+  int stride;        // team i's tiles are sub[i stride], ...; the first one's pad says how many
+  int pairs;         // row pairs of the tallest tile, at least 3 (shared memory is sized by it)
 };
 
-constexpr int kSumBytes = kSumGroup * 33 * 8;  // a warp's scratch for the lane sums of kSumGroup traps
 
-__host__ __device__ constexpr int tile_smem_bytes(int M, int pairs) {
-  return (M + 1) / 2 * 16 + kThreads * 8 + kWarps * (kRing * kStageBytes + kSumBytes + pairs * 1024);
+constexpr int kSumBytes = kSumGroup * kSumStride * 8;  // lane sums of kSumGroup traps
+constexpr int kOwnMax = 32;  // traps a block keeps for its weight updates (more are read again)
+
+__host__ __device__ constexpr int tile_smem_bytes(int M, int team, int pairs) {
+  return (M + 1) / 2 * 16 + kWarps * (kRing * kStageBytes + pairs * 1024) + (team > 1 ? kWarps / team * kSumBytes : 0);
+}
+
+// What the weight update at a launch's end keeps from its start (static shared memory: no register
+// holds an address across the trap loops, where they are short).
+struct OwnWeights {
+  ff part[kThreads];    // the threads' shares of sum |V_m|
+  float2 own[kOwnMax];  // weight and |V_m| of the block's own traps
+};
+__device__ __forceinline__ OwnWeights &own_weights() {
+  __shared__ OwnWeights w;
+  return w;
 }
 
 struct TileSmem {
   float2 *C;            // [Mp] coefficients (0 for the added trap)
-  ff *part;             // [kThreads] the threads' shares of sum |V_m|
   unsigned char *ring;  // this warp's stages
-  float2 *sums;         // [kSumGroup][33] this warp's lane sums of the current traps
   float4 *S;            // [team][2 pairs][32] the team's partial superpositions (rows 2p, 2p+1: re, re, im, im);
                         // the first part then takes the tile's unit phasors
+  float2 *sums;         // [kSumGroup][kSumStride] lane sums of the warp's current traps: in its part of S, or apart
+                        // where the phasors are
   int team, g;          // warps of the team, this warp's place in it
   int part_stride;      // float4 from one warp's part of S to the next
   __device__ __forceinline__ TileSmem(unsigned char *raw, int M, int team_, int pairs)
@@ -63,13 +80,11 @@ struct TileSmem {
     g = warp & (team - 1);
     C = reinterpret_cast<float2 *>(raw);
     raw += (M + 1) / 2 * 16;
-    part = reinterpret_cast<ff *>(raw);
-    raw += kThreads * 8;
     ring = raw + warp * kRing * kStageBytes;
     raw += kWarps * kRing * kStageBytes;
     S = reinterpret_cast<float4 *>(raw) + (warp - g) * part_stride;
-    raw += kWarps * pairs * 1024;
-    sums = reinterpret_cast<float2 *>(raw + warp * kSumBytes);
+    sums = reinterpret_cast<float2 *>(g == 0 && team > 1 ? raw + kWarps * pairs * 1024 + warp / team * kSumBytes
+                                                         : raw + warp * pairs * 1024);
   }
   // Barrier of the team (ids 2 .. 9).
   __device__ __forceinline__ void sync() const {
@@ -101,7 +116,6 @@ struct TileStream {
   int k, pass, fill;
   const float2 *x;
   const float4 *y;
-  int use = 0;  // the consumer's stage (byte offset)
   __device__ __forceinline__ TileStream(const TileArgs &args, const TileSmem &sm, int passes_, int t_begin, int t_end)
       : a(args), ring((unsigned)__cvta_generic_to_shared(sm.ring)), passes(passes_), tile(t_begin), end(t_end), k(0),
         pass(0), fill(0), x(nullptr), y(nullptr) {
@@ -147,9 +161,7 @@ struct TileStream {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(kRing - 2) : "memory");
     __syncwarp();
     issue();
-    const int st = use;
-    use = use == (kRing - 1) * kStageBytes ? 0 : use + kStageBytes;
-    return st;
+    return fill;  // kRing - 1 stages ahead of the stage to read: the one after the stage just filled
   }
 };
 
@@ -157,7 +169,8 @@ struct TileStream {
 // <|V|> (arg S_j does not depend on it), into C, and the threads' shares of sum |V_m| into part;
 // explicit coefficients a.G instead when given.  trace: NULL, or where block 0 writes e and u
 // (Eq. 4) of the fields read.  The block synchronises afterwards.
-__device__ __forceinline__ void tile_prologue(const StepArgs &a, const TileSmem &sm, float *trace) {
+// own, stride: the traps whose weights the block writes (own + stride k, tile_weights).
+__device__ __forceinline__ void tile_prologue(const StepArgs &a, const TileSmem &sm, int own, int stride, float *trace) {
   const int t = threadIdx.x;
   if (t == 0 && (a.M & 1)) sm.C[a.M] = make_float2(0.f, 0.f);
   if (a.G) {
@@ -173,13 +186,15 @@ __device__ __forceinline__ void tile_prologue(const StepArgs &a, const TileSmem 
     const float r = 1.f / am;  // (w / |V|) (V / |V|): no |V|^2 in the denominator, which could underflow
     sm.C[m] = am < 1e-30f ? make_float2(w, 0.f) : make_float2((w * r) * (v.x * r), (w * r) * (v.y * r));
     s = ff_add(s, {am, 0.f});
+    const int k = (m - own) / stride;
+    if (m >= own && k * stride == m - own && k < kOwnMax) own_weights().own[k] = make_float2(w, am);
     if (tr) {
       si = ff_add(si, {I, 0.f});
       mx = fmaxf(mx, I);
       mn = fminf(mn, I);
     }
   }
-  sm.part[t] = s;
+  own_weights().part[t] = s;
   if (!tr) return;
   __shared__ ff tpart[kWarps];
   __shared__ float ext[2][kWarps];
@@ -215,7 +230,7 @@ __device__ __forceinline__ void tile_weights(const StepArgs &a, const TileSmem &
   if (own >= a.M) return;
   __shared__ ff wpart[kWarps];
   const int t = threadIdx.x;
-  ff s = sm.part[t];
+  ff s = own_weights().part[t];
 #pragma unroll
   for (int o = 16; o; o >>= 1)
     s = ff_add(s, {__shfl_down_sync(0xffffffffu, s.hi, o), __shfl_down_sync(0xffffffffu, s.lo, o)});
@@ -225,8 +240,11 @@ __device__ __forceinline__ void tile_weights(const StepArgs &a, const TileSmem &
 #pragma unroll
   for (int i = 1; i < kWarps; i++) q = ff_add(q, wpart[i]);
   const float mean = (q.hi + q.lo) / (float)a.M;
-  for (int m = own + stride * t; m < a.M; m += stride * kThreads)
-    a.w_out[m] = update_from<false>(field_from_sums<true>(a, m), __ldcg(a.w_in + m), mean, 1.f).x;
+  for (int k = t; own + stride * k < a.M; k += kThreads) {
+    const int m = own + stride * k;
+    const float2 wv = k < kOwnMax ? own_weights().own[k] : make_float2(__ldcg(a.w_in + m), sqrtf(abs2(field_from_sums<true>(a, m))));
+    a.w_out[m] = wv.y < 1e-30f ? wv.x : wv.x * mean / wv.y;  // (Sec. 3; a vanishing field keeps its weight)
+  }
 }
 
 // S_{r, c} += (c_m X_m(c)) Y_m(r) of a stage's two traps on the lane's RP row pairs x 2 columns.
@@ -305,8 +323,8 @@ __device__ __forceinline__ void tile_forward(const unsigned char *st, int lane, 
     v[k] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < 2; q++) {
-      const float2 x = X[k * kTileCols + 32 * q], t2 = unpack2(t[k][q]), a2 = unpack2(A[k][q]), b2 = unpack2(B[k][q]);
-      const float tr = t2.x + t2.y, ti = (a2.x + a2.y) - (b2.x + b2.y);
+      const float2 x = X[k * kTileCols + 32 * q], t2 = unpack2(t[k][q]), d2 = unpack2(fma2(B[k][q], pack2(-1.f, -1.f), A[k][q]));
+      const float tr = t2.x + t2.y, ti = d2.x + d2.y;
       v[k].x = fmaf(ti, x.y, fmaf(tr, x.x, v[k].x));
       v[k].y = fmaf(-tr, x.y, fmaf(ti, x.x, v[k].y));
     }
@@ -369,26 +387,31 @@ __device__ __forceinline__ void tile_fields(const StepArgs &a, const TileSmem &s
       P[p][q] = u.x;
       Q[p][q] = u.y;
     }
+  if (sm.team == 1) __syncwarp();  // (the phasors lie in the scratch)
   float2 *const vb = sm.sums;
   unsigned long long *const out = block_acc(a);
   for (int k = 0; k < 2 * T; k += 2) {
     float2 v2[2];
     tile_forward<RP>(sm.ring + in.next(), lane, P, Q, v2);
-    const int j = k & (kSumGroup - 1);  // 0 or 2
-    vb[j * 33 + lane] = v2[0];
-    vb[(j + 1) * 33 + lane] = v2[1];
-    if (j + 2 == kSumGroup || k + 2 == 2 * T) {  // the group's totals: lane l sums trap l / 8
+    const int j = k & (kSumGroup - 1);
+    vb[j * kSumStride + lane] = v2[0];
+    vb[(j + 1) * kSumStride + lane] = v2[1];
+    if (j + 2 == kSumGroup || k + 2 == 2 * T) {  // the group's totals: lane l sums trap l / 4
       __syncwarp();
-      const int tr = lane >> 3, sub = lane & 7;
-      float2 v = vb[tr * 33 + sub];
+      const int tr = lane >> 2, sub = lane & 3;
+      float2 v8[8];
 #pragma unroll
-      for (int i = 1; i < 4; i++) {
-        const float2 q = vb[tr * 33 + sub + 8 * i];
-        v.x += q.x;
-        v.y += q.y;
-      }
+      for (int i = 0; i < 8; i++) v8[i] = vb[tr * kSumStride + sub + 4 * i];
 #pragma unroll
-      for (int o = 4; o; o >>= 1) {
+      for (int w = 4; w; w >>= 1)
+#pragma unroll
+        for (int i = 0; i < w; i++) {
+          v8[i].x += v8[i + w].x;
+          v8[i].y += v8[i + w].y;
+        }
+      float2 v = v8[0];
+#pragma unroll
+      for (int o = 2; o; o >>= 1) {
         v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
         v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
       }
@@ -416,14 +439,14 @@ __device__ __forceinline__ void tile_one(const StepArgs &a, const TileSmem &sm, 
       const unsigned char *const stage = sm.ring + in.next();
       tile_back<RP>(stage, C[k], lane, P, Q);
     }
-    sm.sync();  // the phasors of the tile before are read
+    sm.sync();  // the phasors and lane sums of the tile before are read
     ulonglong2 *const mine = reinterpret_cast<ulonglong2 *>(sm.S + sm.g * sm.part_stride);
 #pragma unroll
     for (int p = 0; p < RP; p++)
 #pragma unroll
       for (int q = 0; q < 2; q++) mine[(2 * p + q) * 32 + lane] = make_ulonglong2(P[p][q], Q[p][q]);
   }
-  sm.sync();  // the team's superpositions are written (FWD alone: the phasors of the tile before read)
+  sm.sync();  // the team's superpositions are written (FWD alone: the phasors and lane sums of the tile before read)
 #pragma unroll 1
   for (int i = sm.g; i < 2 * RP; i += sm.team) {
     const int row = st.y0 + (i & ~1), col = st.x0 + 32 * (i & 1) + lane;
@@ -477,15 +500,15 @@ __global__ void __launch_bounds__(kThreads, 2) gsw_tile_kernel(const __grid_cons
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StepArgs &a = t.s;
   const TileSmem sm(smem_raw, a.M, t.team, t.pairs);
-  const int id = blockIdx.x * (kWarps / t.team) + (threadIdx.x >> 5) / t.team;
-  const int t_begin = a.first[id], t_end = a.first[id + 1];
+  const int t_begin = (blockIdx.x * (kWarps / t.team) + (threadIdx.x >> 5) / t.team) * t.stride;
+  const int t_end = t_begin + a.sub[t_begin].pad;
   allow_dependents();
   TileStream in(t, sm, (BACK ? 1 : 0) + (FWD ? 1 : 0), t_begin, t_end);  // the tables are constant during a sequence
   grid_dependency_wait();
   if (FWD)
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < 2 * a.M * a.copies; i += gridDim.x * kThreads) a.acc_clear[i] = 0ull;
   if (BACK) {
-    tile_prologue(a, sm, a.trace);
+    tile_prologue(a, sm, blockIdx.x, gridDim.x, a.trace);
     __syncthreads();
   }
   tile_run<BACK, FWD, ADJ>(a, sm, in, t_begin, t_end, a.once_flags);
@@ -505,8 +528,8 @@ static __global__ void __launch_bounds__(kThreads, 2) gsw_tile_persistent_kernel
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const TileArgs &t0 = p.step[0];
   const TileSmem sm(smem_raw, t0.s.M, t0.team, t0.pairs);
-  const int id = blockIdx.x * (kWarps / t0.team) + (threadIdx.x >> 5) / t0.team;
-  const int t_begin = t0.s.first[id], t_end = t0.s.first[id + 1];
+  const int t_begin = (blockIdx.x * (kWarps / t0.team) + (threadIdx.x >> 5) / t0.team) * t0.stride;
+  const int t_end = t_begin + t0.s.sub[t_begin].pad;
   unsigned int epoch = 0u;
   for (int k = 0; k <= p.iters; k++) {
     const TileArgs &t = p.step[k % 6];
@@ -521,7 +544,7 @@ static __global__ void __launch_bounds__(kThreads, 2) gsw_tile_persistent_kernel
     if (k == 0) {
       tile_run<false, true, false>(a, sm, in, t_begin, t_end, a.once_flags & ~kOnceLast);
     } else {
-      tile_prologue(a, sm, p.trace ? p.trace + 2 * (k - 1) : nullptr);
+      tile_prologue(a, sm, blockIdx.x, gridDim.x, p.trace ? p.trace + 2 * (k - 1) : nullptr);
       __syncthreads();
       tile_run<true, true, false>(a, sm, in, t_begin, t_end, (a.once_flags & ~(kOnceReadU | kOnceLast)) | (k == p.iters ? kOnceLast : 0));
       tile_weights(a, sm, blockIdx.x, gridDim.x);
@@ -571,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, 2) gsw_tile_batch_kernel(const __gri
     if (t == t1) break;
     if (BACK) {
       __syncthreads();  // the readers of the previous hologram's coefficients are done
-      tile_prologue(a, sm, nullptr);
+      tile_prologue(a, sm, b.owner[h] == (int)blockIdx.x ? 0 : a.M, 1, nullptr);
       __syncthreads();
     }
     tile_run<BACK, true, false>(a, sm, in, t, t1, 0);
