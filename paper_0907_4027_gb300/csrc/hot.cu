@@ -89,6 +89,7 @@ struct hot_ctx {
   // state
   float *phi = nullptr;  // [N]
   int M = 0;
+  unsigned char *io = nullptr;  // one allocation: abc, w, Vsum (in this order: see IoBytes)
   double *abc = nullptr;                                       // [M][3]
   float *Xt = nullptr, *Yt = nullptr, *Xr = nullptr, *Yr = nullptr;  // tables
   float *Y4t = nullptr, *Y4r = nullptr;  // [4][M][ldy4] shifted row tables (hot::StepArgs::Y4)
@@ -133,7 +134,22 @@ struct hot_ctx {
   std::vector<Graph> graphs;
   // HOT_PREC_TENSOR: operands and launch shapes of the tensor-core iteration (built on first use)
   hot_tc::Plan *tc = nullptr;
-  float2 *G = nullptr;  // [M] adjoint coefficients of hot_intensity_loss (allocated on first use)
+  float2 *G = nullptr;  // [M] coefficients of hot_intensity_loss and hot_superposition (allocated on first use)
+  // Pinned staging of the small transfers: what the calls send (abc and weights, coefficients), whose
+  // last copy ev_in ends, then what they read back.  A copy from pageable memory stops the host for
+  // the stream's work and a round trip, as a synchronisation before the buffer's release does.
+  unsigned char *pin = nullptr;
+  cudaEvent_t ev_in = nullptr;
+  bool waits = false;  // a launch with bounded waits was queued since the last look at their error flag
+};
+
+// Layout of hot_ctx::io and of the pinned staging for M traps, in bytes.
+struct IoBytes {
+  size_t abc, w, Vsum, end;  // io: abc [M][3] double, w [2][M] float, Vsum [2][M] int64
+  size_t back;               // pin: [0, back) sent (as io's abc and w); from back on: w, Vsum, 2 metrics, 3 words
+  explicit IoBytes(size_t M) : abc(0), w(24 * M), Vsum(32 * M), end(48 * M), back(32 * M) {}
+  size_t read() const { return end - w; }                 // bytes of w and Vsum
+  size_t pinned() const { return back + read() + 32; }
 };
 
 namespace {
@@ -178,7 +194,12 @@ void free_traps(hot_ctx *c) {
   drop_graphs(c);
   hot_tc::plan_destroy(c->tc);
   c->tc = nullptr;
-  dfree(c->abc);
+  dfree(c->io);
+  c->abc = nullptr;
+  c->w = nullptr;
+  c->Vsum = nullptr;
+  if (c->pin) cudaFreeHost(c->pin);
+  c->pin = nullptr;
   dfree(c->Xt);
   dfree(c->Yt);
   dfree(c->Xr);
@@ -189,9 +210,7 @@ void free_traps(hot_ctx *c) {
   dfree(c->Yc);
   dfree(c->Xq);
   dfree(c->Yq);
-  dfree(c->w);
   dfree(c->acc);
-  dfree(c->Vsum);
   dfree(c->G);
   c->M = 0;
   c->have_fields = false;
@@ -673,19 +692,78 @@ int launch_persistent(hot_ctx *c, int iters) {
   return check_launch(c, "gsw_persistent_kernel");
 }
 
-// Reads the barrier's error flag (synchronises): after a wait ran out, the accumulators and the
-// barrier are reset and HOT_ETIMEOUT is returned; the phases are then undefined.
-int check_wait_error(hot_ctx *c, const char *who) {
-  unsigned int st[3] = {0, 0, 0};  // [2]: error flag of the bounded waits
-  HOT_CUDA(cudaMemcpyAsync(st, c->sync, sizeof st, cudaMemcpyDeviceToHost, c->st));
-  HOT_CUDA(cudaStreamSynchronize(c->st));
-  if (!st[2]) return HOT_OK;
-  HOT_CUDA(cudaMemsetAsync(c->sync, 0, sizeof st, c->st));
+// After a bounded wait ran out: the accumulators and the barrier are reset; the phases are undefined.
+int wait_ran_out(hot_ctx *c, const char *who) {
+  HOT_CUDA(cudaMemsetAsync(c->sync, 0, 3 * sizeof(unsigned int), c->st));
   if (c->M) HOT_CUDA(cudaMemsetAsync(c->acc, 0, sizeof(unsigned long long) * acc_elems(c->M), c->st));
   HOT_CUDA(cudaStreamSynchronize(c->st));
   c->have_fields = false;
   c->u_valid = false;
   return fail(HOT_ETIMEOUT, "%s: a bounded device-side wait ran out (limit %.3g s)", who, c->wait_limit_s);
+}
+
+// Reads the barrier's error flag (synchronises): HOT_ETIMEOUT after a wait ran out.
+int check_wait_error(hot_ctx *c, const char *who) {
+  unsigned int st[3] = {0, 0, 0};  // [2]: error flag of the bounded waits
+  HOT_CUDA(cudaMemcpyAsync(st, c->sync, sizeof st, cudaMemcpyDeviceToHost, c->st));
+  HOT_CUDA(cudaStreamSynchronize(c->st));
+  c->waits = false;
+  return st[2] ? wait_ran_out(c, who) : HOT_OK;
+}
+
+// What read_back leaves in the pinned staging.
+const float *read_w(const hot_ctx *c) { return reinterpret_cast<const float *>(c->pin + IoBytes(c->M).back); }
+const long long *read_sums(const hot_ctx *c) {
+  const IoBytes b(c->M);
+  return reinterpret_cast<const long long *>(c->pin + b.back + b.Vsum - b.w);
+}
+const float *read_metrics(const hot_ctx *c) {
+  const IoBytes b(c->M);
+  return reinterpret_cast<const float *>(c->pin + b.back + b.read());
+}
+
+// Brings weights and field sums (fields) and the metrics (metrics) to the pinned staging with one
+// synchronisation, which also looks at the error flag if a launch with bounded waits was queued.
+int read_back(hot_ctx *c, const char *who, bool fields, bool metrics) {
+  const IoBytes b(c->M);
+  unsigned char *const back = c->pin + b.back;
+  unsigned int *const flag = reinterpret_cast<unsigned int *>(back + b.read() + 8);
+  if (fields) HOT_CUDA(cudaMemcpyAsync(back, c->io + b.w, b.read(), cudaMemcpyDeviceToHost, c->st));
+  if (metrics) HOT_CUDA(cudaMemcpyAsync(back + b.read(), c->metrics, 2 * sizeof(float), cudaMemcpyDeviceToHost, c->st));
+  if (c->waits) HOT_CUDA(cudaMemcpyAsync(flag, c->sync, 3 * sizeof(unsigned int), cudaMemcpyDeviceToHost, c->st));
+  HOT_CUDA(cudaStreamSynchronize(c->st));
+  if (c->waits) {
+    c->waits = false;
+    if (flag[2]) return wait_ran_out(c, who);
+  }
+  return HOT_OK;
+}
+
+// Waits until the last copy out of the pinned staging is done, so that it can be filled again.  A
+// stream under capture is refused: a replay would send what the staging holds by then.
+int staging_free(hot_ctx *c, const char *who) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  HOT_CUDA(cudaStreamIsCapturing(c->st, &st));
+  if (st != cudaStreamCaptureStatusNone) return fail(HOT_ECUDA, "%s: the stream is being captured", who);
+  HOT_CUDA(cudaEventSynchronize(c->ev_in));
+  return HOT_OK;
+}
+
+// e and u to the caller's non-NULL outputs (synchronises); nothing when both are NULL.
+int return_metrics(hot_ctx *c, const char *who, double *eff_out, double *unif_out) {
+  if (!eff_out && !unif_out) return HOT_OK;
+  const int rc = read_back(c, who, false, true);
+  if (rc != HOT_OK) return rc;
+  if (eff_out) *eff_out = read_metrics(c)[0];
+  if (unif_out) *unif_out = read_metrics(c)[1];
+  return HOT_OK;
+}
+
+// Queues the copy of the first `bytes` of the staging, from byte `from`, to dst.
+int send_staged(hot_ctx *c, void *dst, size_t from, size_t bytes) {
+  HOT_CUDA(cudaMemcpyAsync(dst, c->pin + from, bytes, cudaMemcpyHostToDevice, c->st));
+  HOT_CUDA(cudaEventRecord(c->ev_in, c->st));
+  return HOT_OK;
 }
 
 int enqueue_gsw(hot_ctx *c, int iters) {
@@ -810,6 +888,7 @@ void hot_destroy(hot_ctx *c) {
   dfree(c->u8);
   dfree(c->sync);
   dfree(c->trace);
+  if (c->ev_in) cudaEventDestroy(c->ev_in);
   delete c;
 }
 
@@ -822,22 +901,6 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
   if (w0)
     for (int m = 0; m < M; m++)
       if (!finite_pos(w0[m])) return fail(HOT_EINVAL, "hot_set_traps: weight %d not finite and > 0", m);
-  // Eq. 2 in turns per pixel index: a = x p/(lambda f), b = y p/(lambda f), c = z p^2/(2 lambda f^2)
-  double *abc = static_cast<double *>(malloc(sizeof(double) * 3 * M));
-  float *wh = static_cast<float *>(malloc(sizeof(float) * M));
-  if (!abc || !wh) {
-    free(abc);
-    free(wh);
-    return fail(HOT_ENOMEM, "hot_set_traps: out of host memory");
-  }
-  const double lin = c->pitch / (c->lam * c->focal);
-  const double quad = c->pitch * c->pitch / (2.0 * c->lam * c->focal * c->focal);
-  for (int m = 0; m < M; m++) {
-    abc[3 * m] = xyz_m[3 * m] * lin;
-    abc[3 * m + 1] = xyz_m[3 * m + 1] * lin;
-    abc[3 * m + 2] = xyz_m[3 * m + 2] * quad;
-    wh[m] = w0 ? (float)w0[m] : 1.0f;
-  }
   int rc = HOT_OK;
   if (M != c->M) {
     cudaStreamSynchronize(c->st);
@@ -845,12 +908,23 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
     c->M = M;
     rc = build_schedule(c);
     c->M = 0;
-    if (rc != HOT_OK) {
-      free(abc);
-      free(wh);
-      return rc;
+    if (rc != HOT_OK) return rc;
+    const IoBytes io((size_t)M);
+    rc = dalloc(&c->io, io.end);
+    if (rc == HOT_OK) {
+      c->abc = reinterpret_cast<double *>(c->io + io.abc);
+      c->w = reinterpret_cast<float *>(c->io + io.w);
+      c->Vsum = reinterpret_cast<long long *>(c->io + io.Vsum);
+      if (cudaHostAlloc(reinterpret_cast<void **>(&c->pin), io.pinned(), cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        c->pin = nullptr;
+        rc = fail(HOT_ENOMEM, "hot_set_traps: no pinned memory");
+      }
     }
-    rc = dalloc(&c->abc, 3 * (size_t)M);
+    if (rc == HOT_OK && !c->ev_in && cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming) != cudaSuccess) {
+      c->ev_in = nullptr;
+      rc = fail(HOT_ECUDA, "hot_set_traps: cudaEventCreate failed");
+    }
     if (rc == HOT_OK) rc = dalloc(&c->Xt, (size_t)M * c->W);
     if (rc == HOT_OK) rc = dalloc(&c->Xr, (size_t)M * c->W);
     if (rc == HOT_OK) rc = dalloc(&c->Yt, (size_t)M * c->H);
@@ -874,25 +948,30 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
     if (rc == HOT_OK && (cudaMemsetAsync(c->Xq, 0, sizeof(float2) * c->Mp * nx, c->st) != cudaSuccess ||
                          cudaMemsetAsync(c->Yq, 0, sizeof(float4) * (size_t)c->Mp * c->ldp, c->st) != cudaSuccess))
       rc = fail(HOT_ECUDA, "hot_set_traps: clearing the tile kernels' tables failed");
-    if (rc == HOT_OK) rc = dalloc(&c->w, 2 * (size_t)M);
     if (rc == HOT_OK) rc = dalloc(&c->acc, acc_elems(M));
-    if (rc == HOT_OK) rc = dalloc(&c->Vsum, 2 * (size_t)M);
     if (rc == HOT_OK && cudaMemsetAsync(c->acc, 0, sizeof(unsigned long long) * acc_elems(M), c->st) != cudaSuccess)
       rc = fail(HOT_ECUDA, "hot_set_traps: clearing the field accumulators failed");
     if (rc != HOT_OK) {
       free_traps(c);
-      free(abc);
-      free(wh);
       return rc;
     }
     c->M = M;
   }
-  cudaError_t e = cudaMemcpyAsync(c->abc, abc, sizeof(double) * 3 * M, cudaMemcpyHostToDevice, c->st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->w, wh, sizeof(float) * M, cudaMemcpyHostToDevice, c->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);  // host buffers are released below
-  free(abc);
-  free(wh);
-  if (e != cudaSuccess) return fail(HOT_ECUDA, "hot_set_traps: %s", cudaGetErrorString(e));
+  rc = staging_free(c, "hot_set_traps");
+  if (rc != HOT_OK) return rc;
+  // Eq. 2 in turns per pixel index: a = x p/(lambda f), b = y p/(lambda f), c = z p^2/(2 lambda f^2)
+  double *const abc = reinterpret_cast<double *>(c->pin);
+  float *const wh = reinterpret_cast<float *>(c->pin + IoBytes(M).w);
+  const double lin = c->pitch / (c->lam * c->focal);
+  const double quad = c->pitch * c->pitch / (2.0 * c->lam * c->focal * c->focal);
+  for (int m = 0; m < M; m++) {
+    abc[3 * m] = xyz_m[3 * m] * lin;
+    abc[3 * m + 1] = xyz_m[3 * m + 1] * lin;
+    abc[3 * m + 2] = xyz_m[3 * m + 2] * quad;
+    wh[m] = w0 ? (float)w0[m] : 1.0f;
+  }
+  rc = send_staged(c, c->io, 0, IoBytes(M).w + sizeof(float) * M);
+  if (rc != HOT_OK) return rc;
   c->have_fields = false;
   c->u_valid = false;
   return launch_build_tables(c);
@@ -901,14 +980,14 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
 int hot_set_weights(hot_ctx *c, const double *w) {
   if (!c || !w) return fail(HOT_EINVAL, "hot_set_weights: NULL argument");
   if (!c->M) return fail(HOT_ESTATE, "hot_set_weights: no traps set");
-  std::vector<float> wf(c->M);
-  for (int m = 0; m < c->M; m++) {
+  for (int m = 0; m < c->M; m++)
     if (!finite_pos(w[m])) return fail(HOT_EINVAL, "hot_set_weights: weight %d not finite and > 0", m);
-    wf[m] = (float)w[m];
-  }
-  HOT_CUDA(cudaMemcpyAsync(c->w, wf.data(), sizeof(float) * c->M, cudaMemcpyHostToDevice, c->st));
-  HOT_CUDA(cudaStreamSynchronize(c->st));
-  return HOT_OK;
+  const int rc = staging_free(c, "hot_set_weights");
+  if (rc != HOT_OK) return rc;
+  const size_t at = IoBytes(c->M).w;
+  float *const wf = reinterpret_cast<float *>(c->pin + at);
+  for (int m = 0; m < c->M; m++) wf[m] = (float)w[m];
+  return send_staged(c, c->w, at, sizeof(float) * c->M);
 }
 
 int hot_set_phase(hot_ctx *c, const float *phi, int on_device) {
@@ -971,18 +1050,8 @@ int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
   // where the state keeps unit phasors, the last step left u_j of the phases it wrote in ubuf
   c->u_valid = iters > 0 ? c->once : had_u;
   c->have_fields = true;
-  if (eff_out || unif_out) {
-    if (c->persistent || c->precision == HOT_PREC_TENSOR) {
-      const int rc2 = check_wait_error(c, "hot_gsw");
-      if (rc2 != HOT_OK) return rc2;
-    }
-    float m[2];
-    HOT_CUDA(cudaMemcpyAsync(m, c->metrics, sizeof m, cudaMemcpyDeviceToHost, c->st));
-    HOT_CUDA(cudaStreamSynchronize(c->st));
-    if (eff_out) *eff_out = m[0];
-    if (unif_out) *unif_out = m[1];
-  }
-  return HOT_OK;
+  if (c->persistent || c->precision == HOT_PREC_TENSOR) c->waits = true;
+  return return_metrics(c, "hot_gsw", eff_out, unif_out);
 }
 
 int hot_phase_out(hot_ctx *c, void *dst, int fmt, int on_device) {
@@ -1019,13 +1088,10 @@ int hot_get_fields(hot_ctx *c, double *V, double *w) {
   if (!c) return fail(HOT_EINVAL, "hot_get_fields: NULL context");
   if (!c->M) return fail(HOT_ESTATE, "hot_get_fields: no traps set");
   if (V && !c->have_fields) return fail(HOT_ESTATE, "hot_get_fields: no forward evaluation since the last change");
-  const int rc = check_wait_error(c, "hot_get_fields");
+  const int rc = read_back(c, "hot_get_fields", V || w, false);
   if (rc != HOT_OK) return rc;
-  std::vector<long long> vs(V ? 2 * c->M : 0);
-  std::vector<float> wf(w ? c->M : 0);
-  if (V) HOT_CUDA(cudaMemcpyAsync(vs.data(), c->Vsum, sizeof(long long) * 2 * c->M, cudaMemcpyDeviceToHost, c->st));
-  if (w) HOT_CUDA(cudaMemcpyAsync(wf.data(), c->w, sizeof(float) * c->M, cudaMemcpyDeviceToHost, c->st));
-  HOT_CUDA(cudaStreamSynchronize(c->st));
+  const long long *const vs = read_sums(c);
+  const float *const wf = read_w(c);
   const double inv = 1.0 / (n_total(c) * ldexp(1.0, c->fx_shift));
   for (int m = 0; V && m < c->M; m++) {  // fixed-point sums -> V_m
     V[2 * m] = (double)vs[m] * inv;
@@ -1051,23 +1117,15 @@ int hot_field(hot_ctx *c, const float *phi, float *V) {
 int hot_superposition(hot_ctx *c, const double *coef) {
   if (!c || !coef) return fail(HOT_EINVAL, "hot_superposition: NULL argument");
   if (!c->M) return fail(HOT_ESTATE, "hot_superposition: no traps set");
-  std::vector<float> cf(2 * (size_t)c->M);
-  for (int i = 0; i < 2 * c->M; i++) {
+  for (int i = 0; i < 2 * c->M; i++)
     if (!std::isfinite(coef[i])) return fail(HOT_EINVAL, "hot_superposition: coefficient %d not finite", i / 2);
-    cf[i] = (float)coef[i];
-  }
-  float2 *d = nullptr;
-  int rc = dalloc(&d, c->M);
+  int rc = c->G ? HOT_OK : dalloc(&c->G, c->M);
+  if (rc == HOT_OK) rc = staging_free(c, "hot_superposition");
   if (rc != HOT_OK) return rc;
-  cudaError_t e = cudaMemcpyAsync(d, cf.data(), sizeof(float) * cf.size(), cudaMemcpyHostToDevice, c->st);
-  if (e != cudaSuccess) rc = fail(HOT_ECUDA, "hot_superposition: %s", cudaGetErrorString(e));
-  if (rc == HOT_OK)
-    rc = launch_mode<true, false>(c, false, 0, nullptr, d);
-  if (rc == HOT_OK) {
-    e = cudaStreamSynchronize(c->st);  // the coefficients are freed below
-    if (e != cudaSuccess) rc = fail(HOT_ECUDA, "hot_superposition: %s", cudaGetErrorString(e));
-  }
-  dfree(d);
+  float *const cf = reinterpret_cast<float *>(c->pin);
+  for (int i = 0; i < 2 * c->M; i++) cf[i] = (float)coef[i];
+  rc = send_staged(c, c->G, 0, 2 * sizeof(float) * c->M);
+  if (rc == HOT_OK) rc = launch_mode<true, false>(c, false, 0, nullptr, c->G);
   c->have_fields = false;
   c->u_valid = false;
   return rc;
@@ -1137,6 +1195,7 @@ int hot_sharded_begin(hot_ctx *c) {
   int rc = HOT_OK;
   if (c->precision == HOT_PREC_TENSOR) {
     rc = ensure_tc_plan(c);
+    c->waits = true;
     if (rc == HOT_OK) rc = launch_tc(c, false, 0);
   } else {
     rc = launch_step(c, false, true, false, 0);
@@ -1172,26 +1231,16 @@ int hot_sharded_end(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
   c->shard_k = -1;
   if (rc != HOT_OK) return rc;
   c->have_fields = true;
-  if (eff_out || unif_out) {
-    float m[2];
-    HOT_CUDA(cudaMemcpyAsync(m, c->metrics, sizeof m, cudaMemcpyDeviceToHost, c->st));
-    HOT_CUDA(cudaStreamSynchronize(c->st));
-    if (eff_out) *eff_out = m[0];
-    if (unif_out) *unif_out = m[1];
-  }
-  return HOT_OK;
+  return return_metrics(c, "hot_sharded_end", eff_out, unif_out);
 }
 
 int hot_get_metrics(hot_ctx *c, double *eff_out, double *unif_out) {
   if (!c) return fail(HOT_EINVAL, "hot_get_metrics: NULL context");
   if (!c->M || !c->have_fields) return fail(HOT_ESTATE, "hot_get_metrics: no forward evaluation since the last change");
-  const int rc = check_wait_error(c, "hot_get_metrics");
+  const int rc = read_back(c, "hot_get_metrics", false, true);
   if (rc != HOT_OK) return rc;
-  float m[2];
-  HOT_CUDA(cudaMemcpyAsync(m, c->metrics, sizeof m, cudaMemcpyDeviceToHost, c->st));
-  HOT_CUDA(cudaStreamSynchronize(c->st));
-  if (eff_out) *eff_out = m[0];
-  if (unif_out) *unif_out = m[1];
+  if (eff_out) *eff_out = read_metrics(c)[0];
+  if (unif_out) *unif_out = read_metrics(c)[1];
   return HOT_OK;
 }
 
@@ -1956,6 +2005,7 @@ int hot_batch_gsw(hot_batch *b, int iters) {
       for (auto *c : b->ctx) {
         c->have_fields = true;
         c->u_valid = false;  // the batch kernels wrote the phases
+        if (b->precision == HOT_PREC_TENSOR) c->waits = true;
       }
       b->ran = true;
       return HOT_OK;
@@ -1986,6 +2036,7 @@ int hot_batch_gsw(hot_batch *b, int iters) {
   for (auto *c : b->ctx) {
     c->have_fields = true;
     c->u_valid = false;  // the batch kernels wrote the phases
+    if (b->precision == HOT_PREC_TENSOR) c->waits = true;
   }
   b->ran = true;
   return HOT_OK;
