@@ -1072,13 +1072,11 @@ __global__ void __launch_bounds__(kThreads, 4) gsw_persistent_kernel(const __gri
 // abc: [M][3] = a_m, b_m, c_m in turns (see the file header).  Writes turns and radians.
 // A row band (rows y_off .. y_off+H-1 of a hologram of H_total rows) takes the row parts of
 // its global rows.
-// Y4t, Y4r (optional): the shifted copies of the row parts (StepArgs::Y4), [4][M][ldy4], and
-// Xq, Yq (optional) the tile kernels' tables (TileArgs, strips of 64 columns); entries outside the
-// image stay as they are (zero from allocation).
+// Y4t, Y4r (optional): the shifted copies of the row parts (StepArgs::Y4), [4][M][ldy4]; entries
+// outside the shifted rows stay as they are (zero from allocation).
 static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off, int M, const double *abc, float *Xt,
-                                    float *Yt, float *Xr, float *Yr, float2 *Xc, float2 *Yc, float *Y4t = nullptr,
-                                    float *Y4r = nullptr, int ldy4 = 0, float2 *Xq = nullptr, float4 *Yq = nullptr,
-                                    int Mp = 0, int ldp = 0) {
+                                    float *Yt, float *Xr, float *Yr, float *Y4t = nullptr, float *Y4r = nullptr,
+                                    int ldy4 = 0) {
   const long long total = (long long)M * (W + H);
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
        idx += (long long)gridDim.x * blockDim.x) {
@@ -1095,13 +1093,9 @@ static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off,
     t -= rint(t);  // [-1/2, 1/2] turns
     // turns (accurate mode); radians scaled by 1 + kFastEta (fast mode, see cis)
     const float tf = (float)t, rf = (float)(t * (6.283185307179586476925286766559 * (1.0 + (double)kFastEta)));
-    double sn = 0.0, cs = 1.0;
-    if (Xc) sincospi(2.0 * t, &sn, &cs);
     if (i < W) {
       Xt[(size_t)m * W + i] = tf;
       Xr[(size_t)m * W + i] = rf;
-      if (Xc) Xc[(size_t)m * W + i] = make_float2((float)cs, (float)sn);
-      if (Xq) Xq[((size_t)(i >> 6) * Mp + m) * 64 + (i & 63)] = make_float2((float)cs, (float)sn);
     } else {
       Yt[(size_t)m * H + (i - W)] = tf;
       Yr[(size_t)m * H + (i - W)] = rf;
@@ -1110,12 +1104,6 @@ static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off,
           Y4t[((size_t)sh * M + m) * ldy4 + (i - W) + sh] = tf;
           Y4r[((size_t)sh * M + m) * ldy4 + (i - W) + sh] = rf;
         }
-      if (Yc) Yc[(size_t)m * H + (i - W)] = make_float2((float)cs, (float)sn);
-      if (Yq) {
-        float *const y = reinterpret_cast<float *>(Yq + (size_t)m * ldp + ((i - W) >> 1)) + ((i - W) & 1);
-        y[0] = (float)cs;
-        y[2] = (float)sn;
-      }
     }
   }
 }

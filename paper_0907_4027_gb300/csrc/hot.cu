@@ -592,20 +592,76 @@ int launch_finalize(hot_ctx *c, bool pdl, int iters) {
 // Inside the sequence every kernel is a programmatic dependent of the one before it (except
 // when profiling, where events separate the launches); the first one waits normally for
 // whatever preceded hot_gsw in the stream (trap tables, phases).
-// Phase tables of the context's traps (Eq. 2 split into column and row parts).
+// Phase tables of the context's traps (Eq. 2 split into column and row parts): the tile kernels',
+// and those of the direct kernels and of the tensor mode where they are allocated.
 int launch_build_tables(hot_ctx *c) {
-  const long long total = (long long)c->M * (c->W + c->H);
-  const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
   Probe p(c, HOT_KERNEL_OTHER);
-  hot::build_tables_kernel<<<blocks, 256, 0, c->st>>>(c->W, c->H, c->H_total, c->y_off, c->M, c->abc, c->Xt, c->Yt,
-                                                      c->Xr, c->Yr, c->Xc, c->Yc, c->Y4t, c->Y4r, c->ldy4, c->Xq, c->Yq, c->Mp, c->ldp);
-  int rc = check_launch(c, "build_tables_kernel");
+  const hot::TileTables t = {c->W, c->H, c->H_total, c->y_off, c->M, c->Mp, c->ldp, c->abc, c->Xq, c->Yq, c->Xc, c->Yc};
+  hot::tile_tables_kernel<<<dim3((c->W + (c->H + 1) / 2 + 127) / 128, c->M), 128, 0, c->st>>>(t);
+  int rc = check_launch(c, "tile_tables_kernel");
+  if (rc == HOT_OK && c->Y4r) {
+    const long long total = (long long)c->M * (c->W + c->H);
+    const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
+    hot::build_tables_kernel<<<blocks, 256, 0, c->st>>>(c->W, c->H, c->H_total, c->y_off, c->M, c->abc, c->Xt, c->Yt,
+                                                        c->Xr, c->Yr, c->Y4t, c->Y4r, c->ldy4);
+    rc = check_launch(c, "build_tables_kernel");
+  }
   if (rc == HOT_OK && c->tc) {  // the tensor-core operands derive from the tables
     cudaError_t e = hot_tc::plan_refresh(c->tc, c->st);
     if (e != cudaSuccess) rc = fail(HOT_ECUDA, "rebuilding the tensor-core operands: %s", cudaGetErrorString(e));
     c->launches++;
   }
   return rc;
+}
+
+// Allocates the tables that only the direct kernels or only the tensor mode read, once the context
+// is in such a mode.  *added: whether there are new ones (to be built).
+int alloc_mode_tables(hot_ctx *c, int M, bool *added) {
+  int rc = HOT_OK;
+  *added = false;
+  if (!tile_kernels(c) && !c->Y4r) {
+    rc = dalloc(&c->Xt, (size_t)M * c->W);
+    if (rc == HOT_OK) rc = dalloc(&c->Xr, (size_t)M * c->W);
+    if (rc == HOT_OK) rc = dalloc(&c->Yt, (size_t)M * c->H);
+    if (rc == HOT_OK) rc = dalloc(&c->Yr, (size_t)M * c->H);
+    // shifted row tables: rows y0 .. y0 + 15 of copy (4 - y0 % 4) % 4 start 16-byte aligned
+    c->ldy4 = (c->H + 18 + 3) & ~3;
+    const size_t n4 = 4 * (size_t)M * c->ldy4;
+    if (rc == HOT_OK) rc = dalloc(&c->Y4t, n4);
+    if (rc == HOT_OK) rc = dalloc(&c->Y4r, n4);
+    if (rc == HOT_OK && (cudaMemsetAsync(c->Y4t, 0, sizeof(float) * n4, c->st) != cudaSuccess ||
+                         cudaMemsetAsync(c->Y4r, 0, sizeof(float) * n4, c->st) != cudaSuccess))
+      rc = fail(HOT_ECUDA, "clearing the shifted row tables failed");
+    if (rc != HOT_OK) {
+      dfree(c->Xt);
+      dfree(c->Xr);
+      dfree(c->Yt);
+      dfree(c->Yr);
+      dfree(c->Y4t);
+      dfree(c->Y4r);
+      return rc;
+    }
+    *added = true;
+  }
+  if (c->precision == HOT_PREC_TENSOR && !c->Yc) {
+    rc = dalloc(&c->Xc, (size_t)M * c->W);
+    if (rc == HOT_OK) rc = dalloc(&c->Yc, (size_t)M * c->H);
+    if (rc != HOT_OK) {
+      dfree(c->Xc);
+      return rc;
+    }
+    *added = true;
+  }
+  return HOT_OK;
+}
+
+// After a change of the mode: its schedule (resched) and its tables.
+int enter_mode(hot_ctx *c, bool resched) {
+  if (!c->M) return HOT_OK;
+  bool added = false;
+  int rc = resched ? build_schedule(c) : HOT_OK;
+  if (rc == HOT_OK) rc = alloc_mode_tables(c, c->M, &added);
+  return rc == HOT_OK && added ? launch_build_tables(c) : rc;
 }
 
 // The tensor-core plan of the context's traps (HOT_PREC_TENSOR), built on first use.
@@ -925,19 +981,8 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
       c->ev_in = nullptr;
       rc = fail(HOT_ECUDA, "hot_set_traps: cudaEventCreate failed");
     }
-    if (rc == HOT_OK) rc = dalloc(&c->Xt, (size_t)M * c->W);
-    if (rc == HOT_OK) rc = dalloc(&c->Xr, (size_t)M * c->W);
-    if (rc == HOT_OK) rc = dalloc(&c->Yt, (size_t)M * c->H);
-    if (rc == HOT_OK) rc = dalloc(&c->Yr, (size_t)M * c->H);
-    // shifted row tables: rows y0 .. y0 + 15 of copy (4 - y0 % 4) % 4 start 16-byte aligned
-    c->ldy4 = (c->H + 18 + 3) & ~3;
-    if (rc == HOT_OK) rc = dalloc(&c->Y4t, 4 * (size_t)M * c->ldy4);
-    if (rc == HOT_OK) rc = dalloc(&c->Y4r, 4 * (size_t)M * c->ldy4);
-    if (rc == HOT_OK && (cudaMemsetAsync(c->Y4t, 0, sizeof(float) * 4 * (size_t)M * c->ldy4, c->st) != cudaSuccess ||
-                         cudaMemsetAsync(c->Y4r, 0, sizeof(float) * 4 * (size_t)M * c->ldy4, c->st) != cudaSuccess))
-      rc = fail(HOT_ECUDA, "hot_set_traps: clearing the shifted row tables failed");
-    if (rc == HOT_OK) rc = dalloc(&c->Xc, (size_t)M * c->W);
-    if (rc == HOT_OK) rc = dalloc(&c->Yc, (size_t)M * c->H);
+    bool added;
+    if (rc == HOT_OK) rc = alloc_mode_tables(c, M, &added);
     // the tile kernels' tables, zero past the image: whole strips, whole trap pairs, row pairs read
     // kTilePairs at a time
     const size_t nx = (size_t)((c->W + hot::kTileCols - 1) / hot::kTileCols) * hot::kTileCols;
@@ -1015,8 +1060,7 @@ int hot_set_precision(hot_ctx *c, int precision) {
   if (resched || copies_change) HOT_CUDA(cudaStreamSynchronize(c->st));
   c->precision = precision;
   c->u_valid = false;
-  if (resched && c->M) return build_schedule(c);  // the two kernels' occupancies differ
-  return HOT_OK;
+  return enter_mode(c, resched);  // (the kernels' occupancies differ)
 }
 
 int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
@@ -1871,7 +1915,7 @@ int hot_set_once(hot_ctx *c, int on) {
   c->once_req = on != 0;
   c->u_valid = false;
   drop_graphs(c);
-  return c->M ? build_schedule(c) : HOT_OK;
+  return enter_mode(c, true);
 }
 
 int hot_get_once(const hot_ctx *c, int *requested, int *in_effect) {
@@ -2369,7 +2413,7 @@ extern "C" int hot_field_noalloc(int width, int height, double pitch_m, double w
   HOT_CUDA(cudaGetLastError());
   const long long total = (long long)M * (width + height);
   const int tb = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  hot::build_tables_kernel<<<tb, 256, 0, st>>>(width, height, height, 0, M, abc, Xt, Yt, Xr, Yr, nullptr, nullptr);
+  hot::build_tables_kernel<<<tb, 256, 0, st>>>(width, height, height, 0, M, abc, Xt, Yt, Xr, Yr);
   HOT_CUDA(cudaGetLastError());
 
   int bits = 0;

@@ -47,6 +47,8 @@ def test_tiles_match_oracle(hot, W, H, M, precision):
     coef = rng.normal(size=M) + 1j * rng.normal(size=M)
     phi = rng.uniform(-np.pi, np.pi, w.N).astype(np.float32)
     with hot.Hologram.from_workload(w) as h:
+        h.gsw(0)
+        V0, _ = h.fields()
         h.gsw(1)
         V1, w1 = h.fields()
         phi1 = h.phase("f32")
@@ -60,11 +62,12 @@ def test_tiles_match_oracle(hot, W, H, M, precision):
         g = grad.cpu().numpy().astype(np.float64)
         h.superposition(coef)
         sr = h.phase("f32").astype(np.float64)
-    oV0 = oracle.forward(w.geom, w.xyz, w.phi0)
+    assert rel_err(V0, oracle.forward(w.geom, w.xyz, w.phi0)) < REL_V
     r1 = oracle.gsw(w.geom, w.xyz, 1, w.phi0)
     assert rel_err(V1, r1["V"]) < REL_V
     np.testing.assert_allclose(w1, r1["w"], rtol=REL_V)
-    for got, c in ((phi1.astype(np.float64), oracle.update_weights(oV0, np.ones(M))[1]), (sr, coef)):
+    # the back-projection from the GPU's own fields (the rounding of a weak |V_m| is not its error)
+    for got, c in ((phi1.astype(np.float64), oracle.update_weights(V0, np.ones(M))[1]), (sr, coef)):
         ophi, S = oracle.backproject(w.geom, w.xyz, c, want_S=True)
         d = np.abs(np.angle(np.exp(1j * (got - ophi))))
         assert not (np.abs(S) * d > TOL_S * np.sum(np.abs(c))).any()
