@@ -594,6 +594,8 @@ struct FinalizeArgs {
   float *metrics;                 // [2] out: e, u (Eq. 4)
   float inv_fx_n;
   unsigned long long *done;       // NULL, or out: %globaltimer (ns) when the hologram completed
+  float2 *V;                      // NULL, or [M] out: the fields V_m (hot_field)
+  double inv_V;                   // 1 / (N 2^fx_shift)
 };
 
 constexpr int kFinalizeThreads = 1024;
@@ -623,6 +625,7 @@ __device__ __forceinline__ void finalize_block(const FinalizeArgs &a) {
     }
     a.Vsum[m] = sr;
     a.Vsum[a.M + m] = si;
+    if (a.V) a.V[m] = make_float2((float)((double)sr * a.inv_V), (float)((double)si * a.inv_V));
     const float vr = (float)sr * a.inv_fx_n, vi = (float)si * a.inv_fx_n;
     const float I = vr * vr + vi * vi;
     p.si = ff_add(p.si, {I, 0.f});
@@ -857,73 +860,117 @@ struct LossArgs {
   float *loss;                    // [1] out
 };
 
+// FP64 is what bounds it (~2 operations per clock and SM): the sums go through the warps that hold
+// traps and then one warp, sum log I is the logarithm of the warps' products of mantissas plus
+// their exponents, 1/I is a refined FP32 reciprocal.  (With a logarithm and a division per trap and
+// every thread adding 32 warp totals three times, the loss at 256^2 with 16 traps took 49 us, now
+// 16; at 1024^2 with 256 traps this kernel's share fell from ~40 to ~9 us.)
 constexpr int kLossThreads = 1024;
+constexpr int kLossTraps = 4;  // per thread (HOT_MAX_TRAPS / kLossThreads)
 
-// Sum over the block in a fixed order; every thread gets the total.
-__device__ __forceinline__ double block_sum(double v, double *part) {
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();  // earlier readers of part are done
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int i = 0; i < kLossThreads / 32; i++) t += part[i];
-  return t;
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 static __global__ void __launch_bounds__(kLossThreads) intensity_loss_kernel(LossArgs a) {
-  __shared__ double part[kLossThreads / 32];
+  __shared__ double part[3][kLossThreads / 32];
+  __shared__ int exps[kLossThreads / 32];
   __shared__ float ext[2][kLossThreads / 32];
-  double sI = 0.0, sLog = 0.0;
+  __shared__ double total[3];  // sum I, sum log I, sum (I - mean)^2
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int nw = min(kLossThreads / 32, (a.M + 31) / 32);  // warps that hold traps
+  allow_dependents();
+  grid_dependency_wait();
+  double vr[kLossTraps], vi[kLossTraps], I[kLossTraps], sI = 0.0, prod = 1.0;
+  int ex = 0;
   float mx = -1.f, mn = 3.0e38f;
-  for (int m = threadIdx.x; m < a.M; m += kLossThreads) {
+#pragma unroll
+  for (int k = 0; k < kLossTraps; k++) {
+    const int m = t + k * kLossThreads;
+    if (m >= a.M) break;
     long long sr = 0, si = 0;
     for (int c = 0; c < a.copies; c++) {
-      sr += (long long)a.acc[(size_t)c * 2 * a.M + m];
-      si += (long long)a.acc[(size_t)c * 2 * a.M + a.M + m];
+      sr += (long long)__ldcg(a.acc + (size_t)c * 2 * a.M + m);
+      si += (long long)__ldcg(a.acc + (size_t)c * 2 * a.M + a.M + m);
     }
     a.Vsum[m] = sr;
     a.Vsum[a.M + m] = si;
-    const double vr = (double)sr * a.inv_fx_n, vi = (double)si * a.inv_fx_n, I = vr * vr + vi * vi;
-    sI += I;
-    sLog += log(I);
-    mx = fmaxf(mx, (float)I);
-    mn = fminf(mn, (float)I);
-  }
-  const double e = block_sum(sI, part), slog = block_sum(sLog, part);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    mn = fminf(mn, __shfl_down_sync(0xffffffffu, mn, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    ext[0][threadIdx.x >> 5] = mx;
-    ext[1][threadIdx.x >> 5] = mn;
-  }
-  const double mean = e / a.M;
-  double sVar = 0.0;
-  for (int m = threadIdx.x; m < a.M; m += kLossThreads) {
-    const double vr = (double)a.Vsum[m] * a.inv_fx_n, vi = (double)a.Vsum[a.M + m] * a.inv_fx_n;
-    const double d = vr * vr + vi * vi - mean;
-    sVar += d * d;
-  }
-  const double var = block_sum(sVar, part) / a.M;  // (its barriers also order ext and Vsum)
-  for (int m = threadIdx.x; m < a.M; m += kLossThreads) {
-    const double vr = (double)a.Vsum[m] * a.inv_fx_n, vi = (double)a.Vsum[a.M + m] * a.inv_fx_n;
-    const double I = vr * vr + vi * vi;
-    const double g = -1.0 / I + a.beta * (2.0 / a.M) * (I - mean);
-    a.G[m] = make_float2((float)(2.0 * g * vr), (float)(2.0 * g * vi));
-  }
-  for (int i = threadIdx.x; i < 6 * a.M * a.copies; i += kLossThreads) a.acc_all[i] = 0ull;
-  if (threadIdx.x == 0) {
-    float hi = ext[0][0], lo = ext[1][0];
-    for (int i = 1; i < kLossThreads / 32; i++) {
-      hi = fmaxf(hi, ext[0][i]);
-      lo = fminf(lo, ext[1][i]);
+    vr[k] = (double)sr * a.inv_fx_n;
+    vi[k] = (double)si * a.inv_fx_n;
+    I[k] = vr[k] * vr[k] + vi[k] * vi[k];
+    sI += I[k];
+    const int hi = __double2hiint(I[k]), e = hi >> 20;  // I = mantissa in [1/2, 1) x 2^(e - 1022) (I >= 0)
+    if (e > 0 && e < 0x7ff) {
+      prod *= __hiloint2double((hi & 0xfffff) | 0x3fe00000, __double2loint(I[k]));
+      ex += e - 1022;
+    } else {
+      prod *= I[k];  // 0: the logarithm is -infinity
     }
-    *a.loss = (float)(-slog + a.beta * var);
-    a.metrics[0] = (float)e;
-    a.metrics[1] = (hi + lo > 0.f) ? 1.f - (hi - lo) / (hi + lo) : 0.f;
+    mx = fmaxf(mx, (float)I[k]);
+    mn = fminf(mn, (float)I[k]);
+  }
+  if (warp < nw) {
+    sI = warp_sum(sI);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      prod *= __shfl_xor_sync(0xffffffffu, prod, o);  // (128 mantissas: >= 2^-128)
+      ex += __shfl_xor_sync(0xffffffffu, ex, o);
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    }
+    if (lane == 0) {
+      part[0][warp] = sI;
+      part[1][warp] = prod;
+      exps[warp] = ex;
+      ext[0][warp] = mx;
+      ext[1][warp] = mn;
+    }
+  }
+  __syncthreads();  // (every read of the accumulators is done)
+  if (warp == 0) {
+    const bool in = lane < nw;
+    const double e = warp_sum(in ? part[0][lane] : 0.0);
+    const double slog = warp_sum(in ? log(part[1][lane]) + exps[lane] * 0.693147180559945309417232 : 0.0);
+    float hi = in ? ext[0][lane] : -1.f, lo = in ? ext[1][lane] : 3.0e38f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    }
+    if (lane == 0) {
+      total[0] = e;
+      total[1] = slog;
+      a.metrics[0] = (float)e;
+      a.metrics[1] = (hi + lo > 0.f) ? 1.f - (hi - lo) / (hi + lo) : 0.f;
+    }
+  }
+  __syncthreads();
+  const double mean = total[0] / a.M;
+  double sVar = 0.0;
+#pragma unroll
+  for (int k = 0; k < kLossTraps; k++) {
+    const int m = t + k * kLossThreads;
+    if (m >= a.M) break;
+    const double d = I[k] - mean;
+    sVar += d * d;
+    // 1/I to FP64: two Newton steps from the FP32 reciprocal (I >= (2^-61)^2 or 0)
+    double r = (double)(1.f / (float)I[k]);
+    r = r * (2.0 - I[k] * r);
+    r = r * (2.0 - I[k] * r);
+    const double g = a.beta * (2.0 / a.M) * d - r;
+    a.G[m] = make_float2((float)(2.0 * g * vr[k]), (float)(2.0 * g * vi[k]));
+  }
+  if (warp < nw) {
+    sVar = warp_sum(sVar);
+    if (lane == 0) part[2][warp] = sVar;
+  }
+  for (int i = t; i < 6 * a.M * a.copies; i += kLossThreads) a.acc_all[i] = 0ull;
+  __syncthreads();
+  if (warp == 0) {
+    const double var = warp_sum(lane < nw ? part[2][lane] : 0.0) / a.M;
+    if (lane == 0) *a.loss = (float)(-total[1] + a.beta * var);
   }
 }
 
@@ -1106,12 +1153,6 @@ static __global__ void build_tables_kernel(int W, int H, int H_total, int y_off,
         }
     }
   }
-}
-
-// Fixed-point field sums -> float32 complex fields V_m (for callers of hot_field).
-static __global__ void sums_to_fields_kernel(int M, const long long *Vsum, double inv, float2 *V) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < M) V[m] = make_float2((float)((double)Vsum[m] * inv), (float)((double)Vsum[M + m] * inv));
 }
 
 // Sec. 5 encoding of the phases: uint8 g = rint(phi 256 / 2pi) mod 256 (FP32 decision).

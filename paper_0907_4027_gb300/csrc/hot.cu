@@ -15,6 +15,8 @@
 #include "tc.h"
 #include "tile.h"
 
+static_assert(hot::kLossTraps * hot::kLossThreads >= HOT_MAX_TRAPS, "traps per thread of the loss kernel");
+
 namespace {
 
 thread_local char g_err[512] = "";
@@ -571,7 +573,8 @@ int launch_step(hot_ctx *c, bool back, bool fwd, bool pdl, int k, bool last = tr
 }
 
 // After the last launch (k = iters): Eq. 4 metrics, field sums, weights home, accumulators cleared.
-int launch_finalize(hot_ctx *c, bool pdl, int iters) {
+// V: NULL, or the caller's device buffer for the fields (hot_field).
+int launch_finalize(hot_ctx *c, bool pdl, int iters, float *V = nullptr) {
   hot::FinalizeArgs f = {};  // done = NULL: no completion stamp
   const size_t M2 = 2 * (size_t)c->M * acc_copies(c);
   f.M = c->M;
@@ -582,7 +585,9 @@ int launch_finalize(hot_ctx *c, bool pdl, int iters) {
   f.w_dst = c->w;
   f.Vsum = c->Vsum;
   f.metrics = c->metrics;
-  f.inv_fx_n = (float)(1.0 / (n_total(c) * ldexp(1.0, c->fx_shift)));
+  f.inv_V = 1.0 / (n_total(c) * ldexp(1.0, c->fx_shift));
+  f.inv_fx_n = (float)f.inv_V;
+  f.V = reinterpret_cast<float2 *>(V);
   Probe p(c, HOT_KERNEL_FINISH);
   launch(c, hot::gsw_finalize_kernel, 1, hot::kFinalizeThreads, 0, pdl, f);
   return check_launch(c, "gsw_finalize_kernel");
@@ -1148,12 +1153,9 @@ int hot_get_fields(hot_ctx *c, double *V, double *w) {
 int hot_field(hot_ctx *c, const float *phi, float *V) {
   if (!c || !phi || !V) return fail(HOT_EINVAL, "hot_field: NULL argument");
   if (!c->M) return fail(HOT_ESTATE, "hot_field: no traps set");
+  // the finalize kernel (w stays in w[0]; accumulators cleared) follows as a programmatic dependent
   int rc = launch_mode<false, true>(c, false, 0, phi);
-  if (rc == HOT_OK) rc = launch_finalize(c, false, 0);  // w stays in w[0]; accumulators cleared
-  if (rc != HOT_OK) return rc;
-  const double inv = 1.0 / (n_total(c) * ldexp(1.0, c->fx_shift));
-  hot::sums_to_fields_kernel<<<(c->M + 255) / 256, 256, 0, c->st>>>(c->M, c->Vsum, inv, reinterpret_cast<float2 *>(V));
-  rc = check_launch(c, "sums_to_fields_kernel");
+  if (rc == HOT_OK) rc = launch_finalize(c, !c->profiling, 0, V);
   if (rc == HOT_OK) c->have_fields = true;
   return rc;
 }
@@ -1205,13 +1207,13 @@ int hot_intensity_loss(hot_ctx *c, const float *phi, double beta, float *loss, f
   a.loss = loss;
   {
     Probe p(c, HOT_KERNEL_FINISH);
-    hot::intensity_loss_kernel<<<1, hot::kLossThreads, 0, c->st>>>(a);
+    launch(c, hot::intensity_loss_kernel, 1, hot::kLossThreads, 0, !c->profiling, a);
   }
   rc = check_launch(c, "intensity_loss_kernel");
   if (rc != HOT_OK) return rc;
   c->have_fields = true;
   if (!grad) return HOT_OK;
-  return launch_mode<true, false, true>(c, false, 0, phi, c->G, grad);
+  return launch_mode<true, false, true>(c, !c->profiling, 0, phi, c->G, grad);
 }
 
 int hot_set_band(hot_ctx *c, int total_height, int y0) {
