@@ -17,14 +17,16 @@ constexpr size_t kElem = tc::Op<kPlanOp>::kBytes;
 
 struct Plan {
   int W = 0, H = 0, M = 0;
-  int Kb = 0, Kf = 0;               // K of the back GEMM (2M) and forward GEMM (2W), padded to a K slice
+  // K of the back GEMM (2M) and of the forward GEMM (2W), padded to a K slice: each component has
+  // half of it, in rows of ldb, ldu elements (whole slices)
+  int Kb = 0, Kf = 0, ldb = 0, ldu = 0;
   int rows_h = 0;                   // H padded to the tile height (rows of P and U)
   int bn_back = 64, bn_fwd = 64;    // tile widths of the back and forward GEMMs
-  int rows_b = 0, rows_f = 0;       // rows of Bb (2W) and Bf (2M), padded to the tile width
-  int fwd_splits = 1, fwd_cps = 1;  // K splits of the forward GEMM, K slices per split
+  int rows_b = 0, rows_f = 0;       // 2W and 2M padded to the tile width: B has half as many rows per component
+  int fwd_splits = 1, fwd_cps = 1;  // K splits of the forward GEMM, units (half slices) per split
   int sms = 0;
-  void *bb_hi = nullptr, *bb_lo = nullptr, *bf_hi = nullptr, *bf_lo = nullptr;  // operand elements
-  void *p_hi = nullptr, *p_lo = nullptr, *u_hi = nullptr, *u_lo = nullptr;
+  // operands by component and part: back and forward B (constant), P, U
+  __half *bb[2][2] = {}, *bf[2][2] = {}, *p[2][2] = {}, *u[2][2] = {};
   float2 *YT = nullptr;
   const float2 *Xc = nullptr, *Yc = nullptr;  // the context's complex tables [M][W], [M][H]
   tc::Maps back{}, fwd{};
@@ -49,7 +51,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 
 // A row-major operand matrix [rows][inner] of OP elements (inner a multiple of one K slice, base
 // 16-byte aligned) read in boxes of one 128-byte K slice x box_rows with 128-byte swizzle; rows
-// is a multiple of box_rows, so no box leaves the matrix.
+// is a multiple of box_rows: no box leaves the matrix but the last of a K range that starts inside
+// a slice, whose second half is filled and not used.
 template <int OP>
 cudaError_t encode(CUtensorMap *map, const void *base, int inner, int rows, int box_rows) {
   auto fn = encode_fn();
@@ -107,19 +110,44 @@ cudaError_t launch_gemm_bn(int bn, const tc::Maps &maps, const tc::GemmArgs &g, 
                      : launch_gemm<32, EPI>(maps, g, grid, st, pdl);
 }
 
-// Tile width of a GEMM with `rows` x `cols` outputs: the widest whose tiles still occupy most
-// SMs and add little padding (wider tiles load fewer operand bytes per MMA; L2 bandwidth bounds
-// the narrow ones).
-// split_k: the K range may be split over CTAs (the forward GEMM) when it has >= 4 slices each.
-int pick_width(int rows, int cols, int k_chunks, int sms, bool split_k) {
-  for (int bn : {256, 128, 64}) {
-    if (8 * round_up(cols, bn) > 9 * round_up(cols, 32)) continue;  // > 12.5% more padding than 32
-    const long long tiles = (long long)((rows + tc::kBM - 1) / tc::kBM) * ((cols + bn - 1) / bn);
-    const long long ctas = split_k ? tiles * std::max(1, std::min(k_chunks / 4, sms / (int)std::max(1LL, tiles)))
-                                   : tiles;
-    if (ctas * 5 >= 4LL * sms) return bn;
+// CTAs share K in `splits` ranges of `cps` units each (>= 1, the last not empty) when the tiles alone
+// leave SMs idle.
+void split_range(int tiles, int units, int sms, int *cps, int *splits) {
+  const int want = std::max(1, std::min(units, sms / std::max(tiles, 1)));
+  *cps = (units + want - 1) / want;
+  *splits = (units + *cps - 1) / *cps;
+}
+
+// Tile width of a GEMM with `rows` x `cols` outputs and `units` half slices of K: the one with the least
+// estimated time, waves of CTAs (one per SM) x (units of a CTA x time of a unit + time of the rest).
+// Times in 10 ns, fitted to both GEMMs at 16 sizes and every width (512 .. 1920 columns, 8 .. 1500 traps):
+// a unit of 12 MMAs takes 0.7 us up to 128 columns (issuing both components' MMAs turn about, or waiting
+// without the timer, changed nothing) and 0.95 us at 256 (the MMAs' own rate);
+// the rest (launch, pipeline fill, epilogue) grows with the width, more so where the epilogue forms
+// phases.  Against the widest tiles that still occupied 4 of 5 SMs, an iteration of 1281 x 515 with
+// 1500 traps goes from 166 to 87 us, 512^2 with 400 from 33.6 to 26.0, 1000 x 700 with 300 from 38.7 to
+// 29.4; 1920 x 1152 with 1000 keeps its 256.
+// Widths that add more than 12.5% of padding to what 32 columns need are not taken.
+int pick_width(int rows, int cols, int units, int sms, bool forward) {
+  struct Width {
+    int bn, unit, back, fwd;
+  };
+  static constexpr Width kWidths[] = {{256, 95, 950, 630}, {128, 70, 580, 440}, {64, 74, 380, 340}, {32, 73, 290, 290}};
+  int best = 32;
+  long long least = -1;
+  for (const Width &w : kWidths) {
+    if (8 * round_up(cols, w.bn) > 9 * round_up(cols, 32)) continue;
+    const int tiles = ((rows + tc::kBM - 1) / tc::kBM) * ((cols + w.bn - 1) / w.bn);
+    int cps = units, splits = 1;
+    if (forward) split_range(tiles, units, sms, &cps, &splits);
+    const long long waves = ((long long)tiles * splits + sms - 1) / sms;
+    const long long cost = waves * ((long long)cps * w.unit + (forward ? w.fwd : w.back));
+    if (least < 0 || cost < least) {
+      least = cost;
+      best = w.bn;
+    }
   }
-  return 32;
+  return best;
 }
 
 }  // namespace
@@ -134,18 +162,16 @@ Shape shape_for(int W, int H, int M, int sms) {
   sh.rows_b = round_up(2 * W, sh.bn_back);
   sh.rows_f = round_up(2 * M, sh.bn_fwd);
   // forward GEMM: the K range split over CTAs so that the tiles fill the SMs about once
-  const int tiles_f = (sh.rows_h / tc::kBM) * (sh.rows_f / sh.bn_fwd);
-  const int kcf = sh.Kf / kSliceK;
-  const int splits = std::max(1, std::min(kcf, sms / std::max(tiles_f, 1)));
-  sh.fwd_cps = (kcf + splits - 1) / splits;
-  sh.fwd_splits = (kcf + sh.fwd_cps - 1) / sh.fwd_cps;  // every split has >= 1 slice
+  split_range((sh.rows_h / tc::kBM) * (sh.rows_f / sh.bn_fwd), sh.Kf / kSliceK, sms, &sh.fwd_cps, &sh.fwd_splits);
   return sh;
 }
 
 void plan_destroy(Plan *p) {
   if (!p) return;
-  for (void *b : {p->bb_hi, p->bb_lo, p->bf_hi, p->bf_lo, p->p_hi, p->p_lo, p->u_hi, p->u_lo})
-    if (b) cudaFree(b);
+  for (auto *set : {&p->bb, &p->bf, &p->p, &p->u})
+    for (auto &c : *set)
+      for (__half *b : c)
+        if (b) cudaFree(b);
   if (p->YT) cudaFree(p->YT);
   delete p;
 }
@@ -155,20 +181,22 @@ cudaError_t plan_refresh(Plan *p, cudaStream_t st) {
   t.W = p->W;
   t.H = p->H;
   t.M = p->M;
-  t.Kb = p->Kb;
-  t.Kf = p->Kf;
-  t.rows_b = p->rows_b;
-  t.rows_f = p->rows_f;
+  t.Kp = p->Kb / 2;
+  t.ldb = p->ldb;
+  t.ldu = p->ldu;
+  t.rows_b = p->rows_b / 2;
+  t.rows_f = p->rows_f / 2;
   t.Xc = p->Xc;
   t.Yc = p->Yc;
-  t.bb_hi = p->bb_hi;
-  t.bb_lo = p->bb_lo;
-  t.bf_hi = p->bf_hi;
-  t.bf_lo = p->bf_lo;
+  for (int k = 0; k < 4; k++) {
+    t.b[k >> 1][k & 1] = p->bb[k >> 1][k & 1];
+    t.f[k >> 1][k & 1] = p->bf[k >> 1][k & 1];
+  }
   t.YT = p->YT;
-  const long long total = (long long)p->rows_b * p->Kb + (long long)p->rows_f * p->Kf + (long long)p->H * (p->Kb / 2);
+  const long long total =
+      (long long)t.rows_b * (t.ldb / 2) + (long long)t.rows_f * (t.ldu / 2) + (long long)p->H * (t.Kp / 2);
   const int blocks = (int)std::min<long long>((total + 255) / 256, 8LL * p->sms);
-  return launch(tc::tc_tables_kernel<kPlanOp>, dim3(blocks), 256, 0, st, false, t);
+  return launch(tc::tc_tables_kernel, dim3(blocks), 256, 0, st, false, t);
 }
 
 cudaError_t plan_create(Plan **out, int W, int H, int M, const float2 *Xc, const float2 *Yc, cudaStream_t st,
@@ -194,36 +222,34 @@ cudaError_t plan_create(Plan **out, int W, int H, int M, const float2 *Xc, const
   p->fwd_cps = sh.fwd_cps;
   p->fwd_splits = sh.fwd_splits;
   *what = "allocating the tensor-core operands";
-  const size_t nb = (size_t)p->rows_b * p->Kb, nf = (size_t)p->rows_f * p->Kf;
-  const size_t np = (size_t)p->rows_h * p->Kb, nu = (size_t)p->rows_h * p->Kf;
-  if (e == cudaSuccess) e = alloc_bytes(&p->bb_hi, nb * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->bb_lo, nb * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->bf_hi, nf * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->bf_lo, nf * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->p_hi, np * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->p_lo, np * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->u_hi, nu * kElem);
-  if (e == cudaSuccess) e = alloc_bytes(&p->u_lo, nu * kElem);
+  p->ldb = round_up(p->Kb / 2, kSliceK);
+  p->ldu = round_up(p->Kf / 2, kSliceK);
+  const size_t nb = (size_t)(p->rows_b / 2) * p->ldb, nf = (size_t)(p->rows_f / 2) * p->ldu;
+  const size_t np = (size_t)p->rows_h * p->ldb, nu = (size_t)p->rows_h * p->ldu;
+  for (int k = 0; k < 4; k++) {
+    const int c = k >> 1, part = k & 1;
+    if (e == cudaSuccess) e = alloc(&p->bb[c][part], nb);
+    if (e == cudaSuccess) e = alloc(&p->bf[c][part], nf);
+    if (e == cudaSuccess) e = alloc(&p->p[c][part], np);
+    if (e == cudaSuccess) e = alloc(&p->u[c][part], nu);
+    // padding rows and columns of P and U stay zero (the kernels write only the image)
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->p[c][part], 0, np * kElem, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->u[c][part], 0, nu * kElem, st);
+  }
   if (e == cudaSuccess) e = alloc(&p->YT, (size_t)H * (p->Kb / 2));
-  // padding rows and columns of P and U stay zero (the kernels write only the image)
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->p_hi, 0, np * kElem, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->p_lo, 0, np * kElem, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->u_hi, 0, nu * kElem, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->u_lo, 0, nu * kElem, st);
   if (e == cudaSuccess) {
     *what = "building the tensor-core operand tables";
     e = plan_refresh(p, st);
   }
   if (e == cudaSuccess) {
     *what = "encoding the tensor maps";
-    e = encode<kPlanOp>(&p->back.a_hi, p->p_hi, p->Kb, p->rows_h, tc::kBM);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->back.a_lo, p->p_lo, p->Kb, p->rows_h, tc::kBM);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->back.b_hi, p->bb_hi, p->Kb, p->rows_b, p->bn_back);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->back.b_lo, p->bb_lo, p->Kb, p->rows_b, p->bn_back);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.a_hi, p->u_hi, p->Kf, p->rows_h, tc::kBM);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.a_lo, p->u_lo, p->Kf, p->rows_h, tc::kBM);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.b_hi, p->bf_hi, p->Kf, p->rows_f, p->bn_fwd);
-    if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.b_lo, p->bf_lo, p->Kf, p->rows_f, p->bn_fwd);
+    for (int k = 0; k < 4; k++) {
+      const int c = k >> 1, part = k & 1;
+      if (e == cudaSuccess) e = encode<kPlanOp>(&p->back.a[c][part], p->p[c][part], p->ldb, p->rows_h, tc::kBM);
+      if (e == cudaSuccess) e = encode<kPlanOp>(&p->back.b[c][part], p->bb[c][part], p->ldb, p->rows_b / 2, p->bn_back / 2);
+      if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.a[c][part], p->u[c][part], p->ldu, p->rows_h, tc::kBM);
+      if (e == cudaSuccess) e = encode<kPlanOp>(&p->fwd.b[c][part], p->bf[c][part], p->ldu, p->rows_f / 2, p->bn_fwd / 2);
+    }
   }
   if (e == cudaSuccess) {
     *what = "setting the tensor-core kernels' shared memory";
@@ -245,14 +271,10 @@ cudaError_t plan_create(Plan **out, int W, int H, int M, const float2 *Xc, const
   return cudaSuccess;
 }
 
-cudaError_t launch_forward(Plan *p, const Step &s, cudaStream_t st, bool pdl, bool chain, int *kernels) {
-  *kernels = 0;
-  const long long N = (long long)p->W * p->H;
-  const int blocks = (int)std::min<long long>((N + 255) / 256, 8LL * p->sms);
-  cudaError_t e = launch(tc::tc_phase_kernel<kPlanOp>, dim3(blocks), 256, 0, st, pdl, p->W, p->H, p->Kf,
-                         (const float *)s.phi, p->u_hi, p->u_lo, s.acc_clear, 2 * s.M);
-  if (e != cudaSuccess) return e;
-  ++*kernels;
+namespace {
+
+// The forward GEMM of a step: T = U X^H, weighted and added into s.acc_out.
+cudaError_t forward_gemm(Plan *p, const Step &s, cudaStream_t st, bool chain, int *kernels) {
   tc::GemmArgs g = {};
   g.rows = p->H;
   g.cols = 2 * p->M;
@@ -262,15 +284,35 @@ cudaError_t launch_forward(Plan *p, const Step &s, cudaStream_t st, bool pdl, bo
   g.err = s.err;
   g.W = p->W;
   g.H = p->H;
-  g.Kf = p->Kf;
   g.M = p->M;
-  g.Yc = p->Yc;
+  g.Kp = p->Kb / 2;
+  g.YT = p->YT;
   g.acc_out = s.acc_out;
   g.fx_scale = s.fx_scale;
   const dim3 grid(p->rows_f / p->bn_fwd, p->rows_h / tc::kBM, p->fwd_splits);
-  e = launch_gemm_bn<tc::kEpiFwd>(p->bn_fwd, p->fwd, g, grid, st, chain);
+  const cudaError_t e = launch_gemm_bn<tc::kEpiFwd>(p->bn_fwd, p->fwd, g, grid, st, chain);
   if (e == cudaSuccess) ++*kernels;
   return e;
+}
+
+}  // namespace
+
+cudaError_t launch_forward(Plan *p, const Step &s, cudaStream_t st, bool pdl, bool chain, int *kernels) {
+  *kernels = 0;
+  const long long N = (long long)p->W * p->H;
+  const int blocks = (int)std::min<long long>((N + 511) / 512, 8LL * p->sms);
+  tc::PhaseArgs a = {};
+  a.W = p->W;
+  a.H = p->H;
+  a.ldu = p->ldu;
+  a.phi = s.phi;
+  for (int k = 0; k < 4; k++) a.u[k >> 1][k & 1] = p->u[k >> 1][k & 1];
+  a.acc_clear = s.acc_clear;
+  a.n_clear = 2 * s.M;
+  const cudaError_t e = launch(tc::tc_phase_kernel, dim3(blocks), 256, 0, st, pdl, a);
+  if (e != cudaSuccess) return e;
+  ++*kernels;
+  return forward_gemm(p, s, st, chain, kernels);
 }
 
 cudaError_t launch_iteration(Plan *p, const Step &s, cudaStream_t st, bool pdl, bool chain, int *kernels) {
@@ -278,22 +320,21 @@ cudaError_t launch_iteration(Plan *p, const Step &s, cudaStream_t st, bool pdl, 
   tc::PrepArgs pa = {};
   pa.H = p->H;
   pa.M = p->M;
-  pa.Kb = p->Kb;
+  pa.Kp = p->Kb / 2;
+  pa.ldb = p->ldb;
   pa.acc_in = s.acc_in;
   pa.acc_clear = s.acc_clear;
   pa.w_in = s.w_in;
   pa.w_out = s.w_out;
   pa.YT = p->YT;
-  pa.p_hi = p->p_hi;
-  pa.p_lo = p->p_lo;
+  for (int k = 0; k < 4; k++) pa.p[k >> 1][k & 1] = p->p[k >> 1][k & 1];
   pa.inv_fx_n = s.inv_fx_n;
   pa.trace = s.trace;
   // blocks take even shares of the rows (each block also forms all M coefficients)
-  const long long pairs = (long long)p->H * (p->Kb / 2);
+  const long long pairs = (long long)p->H * (pa.Kp / 2);
   const int prep_blocks =
       (int)std::max<long long>(1, std::min<long long>({(pairs + 255) / 256, 2LL * p->sms, (long long)p->H}));
-  cudaError_t e = launch(tc::tc_prep_kernel<kPlanOp>, dim3(prep_blocks), tc::kPrepThreads,
-                         (int)(sizeof(float2) * p->M), st, pdl, pa);
+  cudaError_t e = launch(tc::tc_prep_kernel, dim3(prep_blocks), tc::kPrepThreads, (int)(sizeof(float2) * p->M), st, pdl, pa);
   if (e != cudaSuccess) return e;
   ++*kernels;
   tc::GemmArgs g = {};
@@ -305,32 +346,14 @@ cudaError_t launch_iteration(Plan *p, const Step &s, cudaStream_t st, bool pdl, 
   g.err = s.err;
   g.W = p->W;
   g.H = p->H;
-  g.Kf = p->Kf;
+  g.ldu = p->ldu;
   g.phi = s.phi;
-  g.u_hi = p->u_hi;
-  g.u_lo = p->u_lo;
+  for (int k = 0; k < 4; k++) g.u[k >> 1][k & 1] = p->u[k >> 1][k & 1];
   const dim3 grid_b(p->rows_b / p->bn_back, p->rows_h / tc::kBM, 1);
   e = launch_gemm_bn<tc::kEpiBack>(p->bn_back, p->back, g, grid_b, st, chain);
   if (e != cudaSuccess) return e;
   ++*kernels;
-  g = {};
-  g.rows = p->H;
-  g.cols = 2 * p->M;
-  g.k_chunks = p->Kf / kSliceK;
-  g.chunks_per_split = p->fwd_cps;
-  g.limit_ns = s.limit_ns;
-  g.err = s.err;
-  g.W = p->W;
-  g.H = p->H;
-  g.Kf = p->Kf;
-  g.M = p->M;
-  g.Yc = p->Yc;
-  g.acc_out = s.acc_out;
-  g.fx_scale = s.fx_scale;
-  const dim3 grid_f(p->rows_f / p->bn_fwd, p->rows_h / tc::kBM, p->fwd_splits);
-  e = launch_gemm_bn<tc::kEpiFwd>(p->bn_fwd, p->fwd, g, grid_f, st, chain);
-  if (e == cudaSuccess) ++*kernels;
-  return e;
+  return forward_gemm(p, s, st, chain, kernels);
 }
 
 namespace {
@@ -361,10 +384,11 @@ cudaError_t gemm_op(int rows, int cols, int K, const float *A, const float *B, f
   tc::Maps maps{};
   if (e == cudaSuccess) {
     *what = "encoding the GEMM tensor maps";
-    e = encode<OP>(&maps.a_hi, buf[0], Kp, ra, tc::kBM);
-    if (e == cudaSuccess) e = encode<OP>(&maps.a_lo, buf[1], Kp, ra, tc::kBM);
-    if (e == cudaSuccess) e = encode<OP>(&maps.b_hi, buf[2], Kp, rb, tile_n);
-    if (e == cudaSuccess) e = encode<OP>(&maps.b_lo, buf[3], Kp, rb, tile_n);
+    for (int part = 0; part < 2; part++) {
+      if (e == cudaSuccess) e = encode<OP>(&maps.a[0][part], buf[part], Kp, ra, tc::kBM);
+      if (e == cudaSuccess) e = encode<OP>(&maps.b[0][part], buf[2 + part], Kp, rb, tile_n / 2);
+      maps.b[1][part] = maps.b[0][part];
+    }
   }
   if (e == cudaSuccess) {
     *what = "running the GEMM";

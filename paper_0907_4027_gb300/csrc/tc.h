@@ -24,11 +24,11 @@ struct Step {
 
 // Launch shapes of the tensor mode for a W x H hologram with M traps on `sms` SMs (host only).
 struct Shape {
-  int Kb, Kf;              // K of the back (2M) and forward (2W) GEMMs, padded to a K slice
+  int Kb, Kf;              // K of the back (2M) and forward (2W) products, padded to a K slice
   int rows_h;              // H padded to the tile height
   int bn_back, bn_fwd;     // tile widths (32, 64, 128 or 256)
   int rows_b, rows_f;      // 2W and 2M padded to the tile widths
-  int fwd_splits, fwd_cps; // K splits of the forward GEMM and K slices per split
+  int fwd_splits, fwd_cps; // K splits of the forward GEMM and units (64 of Kf: half a K slice of both components) per split
 };
 Shape shape_for(int W, int H, int M, int sms);
 

@@ -6,10 +6,16 @@
 //   back-projection (Sec. 4)  S[iy][ix] = sum_m (c_m Y_m(iy)) X_m(ix)        = P . X     (H x M by M x W)
 //   forward field   (Eq. 1)   T[iy][m]  = sum_ix u[iy][ix] conj(X_m(ix))     = U . X^H   (H x W by W x M)
 //                             N V_m     = sum_iy conj(Y_m(iy)) T[iy][m]
-// with u = e^{i phi}.  Each complex product is one real GEMM on the 2x2 real embedding of the
-// complex numbers: operands are stored complex-interleaved (real, imaginary) along K, and the
-// constant right-hand operand holds the blocks [[xr, -xi], [xi, xr]] (back) or [[xr, xi], [-xi, xr]]
-// (forward, the conjugate).  The GEMMs run on tcgen05.mma with FP32 accumulators in tensor
+// with u = e^{i phi}.  Real and imaginary parts are separate matrices.  A tile's right-hand operand
+// is the stack [X_r; X_i] of BN/2 traps or columns, and each K slice of it meets first A_r, then A_i
+// (A = P or U): the two accumulators A_r [X_r | X_i] and A_i [X_r | X_i] hold the four real products,
+// which the drain adds with the signs of X (back) or conj(X) (forward).  (What bounds the GEMMs is
+// the operand traffic from L2: against the 2x2 real embedding [[xr, -xi], [xi, xr]] of B this moves
+// 64 instead of 96 KB per 12 MMAs of a 128 x 256 tile; with the epilogues below, an iteration of 1920 x 1152
+// with 1000 traps went from 119.8 to 99.6 us, 1024^2 with 256 from 41.9 to 27.7, 512^2 with 100 from 17.5 to
+// 15.2, 256^2 with 16 from 12.7 to 11.3.  What bounds the widest tiles now is the MMAs' own rate: leaving out
+// the loads or the drain changes nothing, one MMA in three less saves its 128 cycles and a little more.)
+// The GEMMs run on tcgen05.mma with FP32 accumulators in tensor
 // memory.  A 16-bit or TF32 tensor-core operand keeps 11 significant bits, so every operand is
 // split x = hi + lo and a product takes three MMAs, a_hi b_hi + a_hi b_lo + a_lo b_hi (the omitted
 // a_lo b_lo is ~2^-22 relative): the products keep about FP32 accuracy.  The GSW iteration uses
@@ -18,8 +24,8 @@
 // (kind::tf32, the FP32 exponent range).
 //
 // A CTA computes one 128 x BN tile of a GEMM over a range of K, warp-specialised: one thread of
-// warp 0 issues TMA loads of K slices (one 128-byte row per matrix row, 128-byte swizzle) of A_hi,
-// A_lo, B_hi, B_lo into a ring of shared-memory stages; one thread of warp 1 issues the 12 MMAs of
+// warp 0 issues TMA loads of K slices (one 128-byte row per matrix row, 128-byte swizzle) of A and
+// of B (both parts, hi and lo) into two rings of shared-memory stages; one thread of warp 1 issues the 12 MMAs of
 // a slice into one of 2-4 tensor-memory accumulators and returns the stage to the loader with
 // tcgen05.commit; the drain warps (TMEM lane quadrant = warp % 4, i.e. 32 rows each, and a group
 // of <= 128 columns) add every slice's accumulator into FP32 registers while the MMAs of the next
@@ -73,46 +79,55 @@ __host__ __device__ constexpr int slice_k() {  // K elements per slice: 32 (TF32
 
 constexpr int kEpiPlain = 0, kEpiBack = 1, kEpiFwd = 2;
 
-// Tile width BN (32, 64, 128 or 256 columns): shared-memory stages as fit in 192 KB; the accumulator
-// is drained by 4 warps per group of at most 128 columns (a thread keeps its row's columns of
-// the group in registers), so BN = 256 has two column groups and 8 drain warps.
+// Tile width BN (32, 64, 128 or 256 columns): shared-memory stages as fit in 224 KB; the accumulator
+// is drained by 4 warps per column group (a thread keeps its row's columns of the group in registers).
+// The groups are many for the epilogues' sake, which are chains of latencies: one group of 32, 64 or 128
+// columns and two of 256 took 12.0, 16.1, 22.3, 32.8 and 101 us per iteration at 256^2 / 16, 512^2 / 100,
+// 768^2 / 100, 1024^2 / 256 and 1920 x 1152 / 1000 traps, these take 11.3, 15.2, 19.6, 27.7 and 99.6; groups
+// of 8 columns for BN = 32 (15.6, 20.2) were slower again.
 template <int BN>
 struct Cfg {
   static_assert(BN == 32 || BN == 64 || BN == 128 || BN == 256, "tile width");
-  static constexpr int kStages = BN == 256 ? 2 : BN == 128 ? 3 : 4;
-  static constexpr int kABytes = kBM * kSliceBytes;  // 16 KB
+  // stages of the rings of A and of B: with two stages of A the loads of a step had only the step
+  // before it to arrive in
+  static constexpr int kStagesA = BN >= 128 ? 3 : 4, kStagesB = BN == 256 ? 2 : BN == 128 ? 3 : 4;
+  static constexpr int kABytes = kBM * kSliceBytes;  // 16 KB: one part (hi or lo) of a slice
   static constexpr int kBBytes = BN * kSliceBytes;
-  static constexpr int kStageBytes = 2 * kABytes + 2 * kBBytes;
-  static constexpr int kSmem = kStages * kStageBytes + 1024;  // + slack to align the ring to 1 KB
-  static constexpr int kGroups = BN == 256 ? 2 : 1;           // column groups of the drain
+  static constexpr int kRingBytes = 2 * (kStagesA * kABytes + kStagesB * kBBytes);
+  // the row table under a forward tile, fetched before the K loop, where it fits beside the rings (with it
+  // 12.2, 16.3, 21.7 us at 256^2 / 16, 512^2 / 100, 768^2 / 100 against 12.9, 17.4, 22.3)
+  static constexpr int kYBytes = BN <= 64 ? kBM * (BN / 2) * 8 : 0;
+  static constexpr int kSmem = kRingBytes + kYBytes + 1024;  // + slack to align the rings to 1 KB
+  static constexpr int kGroups = BN >= 64 ? 4 : 2;        // column groups of the drain
   static constexpr int kCols = BN / kGroups;                  // columns per drain warp
   static constexpr int kEpiWarps = 4 * kGroups;               // one per TMEM lane quadrant and group
   static constexpr int kThreads = 32 * (2 + kEpiWarps);       // warp 0: TMA, warp 1: MMA, then drain
   static constexpr int kBufs = BN == 256 ? 2 : 4;             // accumulators in the 512 TMEM columns
   static constexpr int kTmemCols = kBufs * BN;                // a power of two >= 32
 };
-struct BackStage;
-
-// The four operand maps of one GEMM (2-D, box of one 128-byte K slice x rows, 128-byte swizzle).
+// The operand maps of one GEMM (2-D, box of one 128-byte K slice x rows, 128-byte swizzle), by
+// component (real, imaginary; plain GEMM: a[0], and b[0] = b[1]) and part (hi, lo).  B's boxes have
+// BN / 2 rows, one component.
 struct Maps {
-  CUtensorMap a_hi, a_lo, b_hi, b_lo;
+  CUtensorMap a[2][2], b[2][2];
 };
 
 struct GemmArgs {
   int rows, cols;        // GEMM M and N: outputs outside are not written
-  int k_chunks;          // K slices (K / slice_k)
-  int chunks_per_split;  // K slices per CTA: CTA z takes slices z*cps .. min(k_chunks, (z+1)*cps)-1
+  int k_chunks;          // K in units: slices (plain), half slices of one component (back, forward)
+  int chunks_per_split;  // units per CTA: CTA z takes units z*cps .. min(k_chunks, (z+1)*cps)-1
   long long limit_ns;    // bound of every wait
   int *err;              // set to 1 when a wait runs out
   // plain
   float *C;              // [rows][cols]
   // back: S -> phi, U
-  int W, H, Kf;          // pixels; row stride of U (elements)
+  int W, H, ldu;         // pixels; row stride of U (elements)
   float *phi;            // [H][W]
-  void *u_hi, *u_lo;     // [..][Kf] operand elements: (cos phi, sin phi) interleaved, split
+  __half *u[2][2];       // [..][ldu] cos phi, sin phi (component), hi and lo (part)
   // forward: T -> fixed-point field sums
   int M;
-  const float2 *Yc;              // [M][H] Y_m(iy)
+  int Kp;                        // row stride of YT
+  const float2 *YT;              // [H][Kp] Y_m(iy)
   unsigned long long *acc_out;   // [2][M] Re, Im (zero before the first split adds)
   float fx_scale;
 };
@@ -218,6 +233,49 @@ __device__ __forceinline__ void tmem_load32(uint32_t taddr, float *v) {
 #pragma unroll
   for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_load16(uint32_t taddr, float *v) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+      "[%16];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_load8(uint32_t taddr, float *v) {
+  uint32_t r[8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// acc[0 .. N-1] += sign (+-1: exact) times N accumulator columns from taddr (N = 8, 16 or a multiple of 32).
+template <int N>
+__device__ __forceinline__ void drain_columns(uint32_t taddr, float *acc, float sign) {
+  constexpr int STEP = N < 16 ? 8 : N < 32 ? 16 : 32;
+#pragma unroll
+  for (int c = 0; c < N; c += STEP) {
+    float v[STEP];
+    if constexpr (STEP == 8)
+      tmem_load8(taddr + (uint32_t)c, v);
+    else if constexpr (STEP == 32)
+      tmem_load32(taddr + (uint32_t)c, v);
+    else
+      tmem_load16(taddr + (uint32_t)c, v);
+#pragma unroll
+    for (int j = 0; j < STEP; j++) acc[c + j] = fmaf(sign, v[j], acc[c + j]);
+  }
+}
 
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
@@ -263,149 +321,183 @@ __device__ __forceinline__ void unit_phasor(float ph, float &sn, float &cs) {
   __sincosf(x, &sn, &cs);
 }
 
-// Stores a complex value split into the hi and lo operand arrays at element i (even).
-template <int OP>
-__device__ __forceinline__ void store_split(void *hi, void *lo, size_t i, float re, float im) {
-  const float2 r = split2<OP>(re), m = split2<OP>(im);
-  store2<OP>(hi, i, r.x, m.x);
-  store2<OP>(lo, i, r.y, m.y);
+// Two values' hi (x) and lo (y) FP16 parts, packed.
+__device__ __forceinline__ uint2 split_pair(float a, float b) {
+  const __half2 hi = __floats2half2_rn(a, b);
+  const float2 h = __half22float2(hi);
+  const __half2 lo = __floats2half2_rn(a - h.x, b - h.y);
+  return make_uint2(*reinterpret_cast<const uint32_t *>(&hi), *reinterpret_cast<const uint32_t *>(&lo));
 }
 
-// 32 accumulator columns n0 .. n0+31 of one row of the plain GEMM: C.
+// Complex values (re[0], im[0]), (re[1], im[1]) into the split component arrays at elements i, i + 1 (i even).
+__device__ __forceinline__ void store_pair(__half *const (&dst)[2][2], size_t i, float2 re, float2 im) {
+  const uint2 r = split_pair(re.x, re.y), m = split_pair(im.x, im.y);
+  *reinterpret_cast<uint32_t *>(dst[0][0] + i) = r.x;
+  *reinterpret_cast<uint32_t *>(dst[0][1] + i) = r.y;
+  *reinterpret_cast<uint32_t *>(dst[1][0] + i) = m.x;
+  *reinterpret_cast<uint32_t *>(dst[1][1] + i) = m.y;
+}
+
+// N accumulator columns n0 .. of one row of the plain GEMM: C.
+template <int N>
 __device__ __forceinline__ void epilogue_plain(const GemmArgs &a, const float *v, int row, int n0) {
   if (row < a.rows)
 #pragma unroll
-    for (int c = 0; c < 32; c++)
+    for (int c = 0; c < N; c++)
       if (n0 + c < a.cols) a.C[(size_t)row * a.cols + n0 + c] = v[c];
 }
 
-// Back-projection: 32 accumulator columns n0 .. n0+31, columns 2 p, 2 p + 1 = Re S, Im S of pixel
-// ix = n0/2 + p of this thread's row -> phi = arg S (Sec. 4; atan2(0, 0) = 0) and u = e^{i phi}.
-// A thread holds one row, so the 16 pixels are first written to the warp's staging area in
-// shared memory (rows padded against bank conflicts) and then stored row segment by row segment:
-// each store instruction of the warp writes whole 32-byte sectors of one or two rows instead
-// of one word in each of 32 rows.
-struct BackStage {
-  float ph[32][17];  // phases of 16 pixels of 32 rows
-  float uh[32][33];  // (cos, sin) interleaved, high parts
-  float ul[32][33];  // and low parts
-};
-template <int OP>
-__device__ __forceinline__ void epilogue_back(const GemmArgs &a, const float *v, int row0, int n0, BackStage &st) {
-  const int lane = threadIdx.x & 31;
+// The back and forward epilogues start from the tile in shared memory (the rings are free by then),
+// real and imaginary halves of BN / 2 columns in rows of kStage floats: a drain thread holds one row,
+// and its registers can only be walked by straight-line code (64 pixels of atan2, sin and cos: 100 KB
+// of instructions run once, 1.2 warps of the drain waiting for the instruction cache at any time), while the
+// epilogues want short loops and neighbouring columns in neighbouring lanes (measured together with the operands above).
+template <int BN>
+constexpr int kStage = BN + 4;  // floats: 16-byte stores of eight rows fall on different banks
+template <int BN>
+__device__ __forceinline__ void stage_tile(float *tile, const float *acc, int q, int g) {
+  constexpr int HALF = Cfg<BN>::kCols / 2;
+  float *row = tile + (q * 32 + (threadIdx.x & 31)) * kStage<BN> + g * HALF;
 #pragma unroll
-  for (int p = 0; p < 16; p++) {
-    const float ph = atan2f(v[2 * p + 1], v[2 * p]);
-    float sn, cs;
-    unit_phasor(ph, sn, cs);
-    const float2 c2 = split2<OP>(cs), s2 = split2<OP>(sn);
-    st.ph[lane][p] = ph;
-    st.uh[lane][2 * p] = c2.x;
-    st.uh[lane][2 * p + 1] = s2.x;
-    st.ul[lane][2 * p] = c2.y;
-    st.ul[lane][2 * p + 1] = s2.y;
+  for (int c = 0; c < HALF; c += 4) {
+    *reinterpret_cast<float4 *>(row + c) = make_float4(acc[c], acc[c + 1], acc[c + 2], acc[c + 3]);
+    *reinterpret_cast<float4 *>(row + BN / 2 + c) =
+        make_float4(acc[HALF + c], acc[HALF + c + 1], acc[HALF + c + 2], acc[HALF + c + 3]);
   }
-  __syncwarp();
-  const int x0 = n0 >> 1;
-#pragma unroll 4
-  for (int i = 0; i < 16; i++) {  // phases: two rows of 16 pixels per instruction
-    const int r = 2 * i + (lane >> 4), p = lane & 15, iy = row0 + r, ix = x0 + p;
-    if (iy < a.H && ix < a.W) a.phi[(size_t)iy * a.W + ix] = st.ph[r][p];
-  }
-#pragma unroll 4
-  for (int r = 0; r < 32; r++) {  // operand: one row of 16 pixels (128 bytes) per instruction
-    const int iy = row0 + r, ix = x0 + (lane >> 1);
-    if (iy < a.H && ix < a.W) {
-      const size_t o = (size_t)iy * a.Kf + 2 * x0 + lane;
-      store1<OP>(a.u_hi, o, st.uh[r][lane]);
-      store1<OP>(a.u_lo, o, st.ul[r][lane]);
-    }
-  }
-  __syncwarp();
+  asm volatile("bar.sync 1, %0;" ::"n"(32 * Cfg<BN>::kEpiWarps) : "memory");  // the drain warps only
 }
 
-// Forward: the warp's COLS columns c0 .. c0+COLS-1 of the tile (2 p, 2 p + 1 = Re, Im of T[row][m],
-// m = (n0 + c0)/2 + p).  The terms T conj(Y_m(row)) are summed over the tile's 128 rows (in each
-// warp a transposed shuffle reduction after which lane L holds columns COLS/32 L ..; then the four
-// lane quadrants in order) and added into the fixed-point sums, one atomic per trap and component.
-// q: the warp's TMEM lane quadrant, g its column group; ok: its accumulator is complete; failed:
-// the CTA's flag, read after the drain warps' barrier (an incomplete tile adds nothing).
+// Back-projection: S of the tile's pixels -> phi = arg S (Sec. 4; atan2(0, 0) = 0) and u = e^{i phi},
+// split: two neighbouring pixels per thread and step.
 template <int BN>
-__device__ __forceinline__ void epilogue_fwd(const GemmArgs &a, float *z, int row, int n0, float *red, int q, int g,
-                                             bool ok, const int *failed) {
-  constexpr int COLS = Cfg<BN>::kCols, PER = COLS / 32;
-  const int mt0 = (n0 + g * COLS) >> 1;
-#pragma unroll
-  for (int p = 0; p < COLS / 2; p++) {
-    const int m = mt0 + p;
-    const float tr = z[2 * p], ti = z[2 * p + 1];
-    float zr = 0.f, zi = 0.f;
-    if (ok && row < a.H && m < a.M) {
-      const float2 y = __ldg(a.Yc + (size_t)m * a.H + row);
-      zr = fmaf(tr, y.x, ti * y.y);
-      zi = fmaf(ti, y.x, -tr * y.y);
+__device__ __forceinline__ void epilogue_back(const GemmArgs &a, const float *tile, int m0, int x0) {
+  constexpr int PAIRS = BN / 4;  // pixel pairs of a row
+  const bool two = (a.W & 1) == 0;  // rows start 8-byte aligned
+#pragma unroll 1
+  for (int i = threadIdx.x - 64; i < kBM * PAIRS; i += 32 * Cfg<BN>::kEpiWarps) {
+    const int r = i / PAIRS, p = 2 * (i % PAIRS), iy = m0 + r, ix = x0 + p;
+    if (iy >= a.H || ix >= a.W) continue;
+    const float2 re = *reinterpret_cast<const float2 *>(tile + r * kStage<BN> + p);
+    const float2 im = *reinterpret_cast<const float2 *>(tile + r * kStage<BN> + BN / 2 + p);
+    float2 ph, cs, sn;
+    ph.x = atan2f(im.x, re.x);
+    ph.y = atan2f(im.y, re.y);
+    unit_phasor(ph.x, sn.x, cs.x);
+    unit_phasor(ph.y, sn.y, cs.y);
+    float *out = a.phi + (size_t)iy * a.W + ix;
+    if (ix + 1 >= a.W) {  // an odd row's last pixel: the padding of U stays zero
+      out[0] = ph.x;
+      cs.y = sn.y = 0.f;
+    } else if (two) {
+      *reinterpret_cast<float2 *>(out) = ph;
+    } else {
+      out[0] = ph.x;
+      out[1] = ph.y;
     }
-    z[2 * p] = zr;
-    z[2 * p + 1] = zi;
+    store_pair(a.u, (size_t)iy * a.ldu + ix, cs, sn);
   }
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16, n = COLS; o >= 1; o >>= 1, n >>= 1) {
-    const bool upper = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < n / 2; i++) {
-      const float send = upper ? z[i] : z[i + n / 2];
-      const float keep = upper ? z[i + n / 2] : z[i];
-      z[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
+}
+
+// The rows of YT under a forward tile into shared memory [kBM][BN / 2], by the drain warps (16-byte pieces:
+// t0 and Kp are even); rows and traps beyond the image are not fetched and not read.
+template <int BN>
+__device__ __forceinline__ void fetch_rows(const GemmArgs &a, unsigned char *y, int m0, int t0) {
+  constexpr int PIECES = BN / 4;
+  for (int i = threadIdx.x - 64; i < kBM * PIECES; i += 32 * Cfg<BN>::kEpiWarps) {
+    const int r = i / PIECES, m = t0 + 2 * (i % PIECES);
+    if (m0 + r < a.H && m < a.Kp)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(y) + 16 * i),
+                   "l"(a.YT + (size_t)(m0 + r) * a.Kp + m)
+                   : "memory");
   }
+}
+
+// Forward: the tile's T[row][m] times conj(Y_m(row)), summed over its rows -- a thread takes one trap
+// and every PARTS-th row, in four partial sums -- and added into the fixed-point sums, one atomic
+// per trap and component.  The partial sums meet in red.
+template <int BN>
+__device__ __forceinline__ void epilogue_fwd(const GemmArgs &a, const float *tile, float4 *red, const float2 *ys, int m0, int t0) {
+  constexpr int TRAPS = BN / 2, THREADS = 32 * Cfg<BN>::kEpiWarps, PARTS = THREADS / TRAPS;
+  const int t = threadIdx.x - 64, j = t % TRAPS, part = t / TRAPS, m = t0 + j;
+  const int rows = min(kBM, a.H - m0);
+  float2 v[4];
 #pragma unroll
-  for (int i = 0; i < PER; i++) red[(g * 4 + q) * COLS + PER * lane + i] = z[i];
-  asm volatile("bar.sync 1, %0;" ::"n"(32 * Cfg<BN>::kEpiWarps) : "memory");  // the drain warps only
-  const int t = threadIdx.x - 64;  // index among the drain threads
-  if (t < BN && !*(const volatile int *)failed) {
-    const int gg = t / COLS, j = t % COLS;
-    const int m = (n0 + t) >> 1;
-    if (m < a.M) {
-      const float *r = red + gg * 4 * COLS + j;
-      const float s = ((r[0] + r[COLS]) + r[2 * COLS]) + r[3 * COLS];
-      // |s| <= N, so s * 2^fx_shift rounds to an integer below 2^61
-      atomicAdd(a.acc_out + (size_t)(t & 1) * a.M + m, (unsigned long long)__float2ll_rn(s * a.fx_scale));
+  for (int k = 0; k < 4; k++) v[k] = make_float2(0.f, 0.f);
+  if (m < a.M) {
+    const float *z = tile + j;
+    const float2 *y = a.YT + (size_t)m0 * a.Kp + m;
+#pragma unroll 4
+    for (int r = part; r < kBM; r += 4 * PARTS)
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        const int rr = r + k * PARTS;
+        if (rr < rows) {
+          const float2 yy = Cfg<BN>::kYBytes ? ys[rr * TRAPS + j] : __ldg(y + (size_t)rr * a.Kp);
+          const float tr = z[rr * kStage<BN>], ti = z[rr * kStage<BN> + BN / 2];
+          v[k].x = fmaf(tr, yy.x, fmaf(ti, yy.y, v[k].x));
+          v[k].y = fmaf(ti, yy.x, fmaf(-tr, yy.y, v[k].y));
+        }
+      }
+  }
+  const float2 s = make_float2((v[0].x + v[1].x) + (v[2].x + v[3].x), (v[0].y + v[1].y) + (v[2].y + v[3].y));
+  float2 *const sums = reinterpret_cast<float2 *>(red);
+  sums[t] = s;
+  asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  if (part == 0 && m < a.M) {
+    float2 w = s;
+#pragma unroll
+    for (int k = 1; k < PARTS; k++) {
+      w.x += sums[t + k * TRAPS].x;
+      w.y += sums[t + k * TRAPS].y;
     }
+    // |w| <= N, so w * 2^fx_shift rounds to an integer below 2^61
+    atomicAdd(a.acc_out + m, (unsigned long long)__float2ll_rn(w.x * a.fx_scale));
+    atomicAdd(a.acc_out + a.M + m, (unsigned long long)__float2ll_rn(w.y * a.fx_scale));
   }
 }
 
 // One 128 x BN output tile over a K range: TMA loader (warp 0, one lane), MMA issuer (warp 1,
 // one lane), accumulator drain and epilogue (the other warps).  grid = (N tiles, M tiles, K splits).
+// A step is one slice of one component of A against the slice of B: NA steps per slice of B.
 template <int BN, int EPI, int OP>
 __global__ void __launch_bounds__(Cfg<BN>::kThreads, 1) tc_gemm_kernel(const __grid_constant__ Maps maps,
                                                                        const __grid_constant__ GemmArgs a) {
   using C = Cfg<BN>;
+  constexpr int NA = EPI == kEpiPlain ? 1 : 2, SA = C::kStagesA, SB = C::kStagesB;
+  constexpr int kSteps = kSliceBytes / kMmaKBytes;  // MMA steps along K per slice
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t full[C::kStages], empty[C::kStages], tfull[C::kBufs], tempty[C::kBufs];
+  __shared__ __align__(8) uint64_t full_a[SA], empty_a[SA], full_b[SB], empty_b[SB], tfull[C::kBufs], tempty[C::kBufs];
   __shared__ uint32_t tmem_slot;
-  __shared__ int issued, consumed, failed;
-  __shared__ float red[EPI == kEpiFwd ? 4 * BN : 1];
-  // the ring starts on a 1 KB boundary of the shared window (the 128-byte swizzle pattern repeats
+  __shared__ int issued_a, issued_b, consumed_a, consumed_b, failed;
+  // the rings start on a 1 KB boundary of the shared window (the 128-byte swizzle pattern repeats
   // every 8 rows of 128 bytes and the descriptors assume aligned tiles)
-  unsigned char *ring = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  unsigned char *ring_a = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  unsigned char *ring_b = ring_a + SA * 2 * C::kABytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * kBM;
   const int kc0 = blockIdx.z * a.chunks_per_split;
   const int nk = min(a.k_chunks - kc0, a.chunks_per_split);  // >= 1 (the host sizes the splits)
+  const int nb = NA == 1 ? nk : (nk + 1) / 2;                // slices of B; the last one may be half
+  const int steps = NA * nb;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < C::kStages; s++) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+    for (int s = 0; s < SA; s++) {
+      mbar_init(&full_a[s], 1);
+      mbar_init(&empty_a[s], 1);
+    }
+    for (int s = 0; s < SB; s++) {
+      mbar_init(&full_b[s], 1);
+      mbar_init(&empty_b[s], 1);
     }
     for (int b = 0; b < C::kBufs; b++) {
       mbar_init(&tfull[b], 1);
       mbar_init(&tempty[b], C::kEpiWarps);
     }
-    issued = consumed = failed = 0;
+    issued_a = issued_b = consumed_a = consumed_b = failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.a_hi)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&maps.b_hi)) : "memory");
+  }
+  if (warp == 1 && lane < 8 && (NA == 2 || (lane & 6) != 2)) {  // the operand maps (plain: no second component of A)
+    const CUtensorMap *map = lane < 4 ? &maps.a[lane >> 1][lane & 1] : &maps.b[(lane - 4) >> 1][lane & 1];
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
   }
   if (warp == 0) {  // the whole warp allocates kBufs FP32 accumulators of BN columns
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
@@ -422,83 +514,107 @@ __global__ void __launch_bounds__(Cfg<BN>::kThreads, 1) tc_gemm_kernel(const __g
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int i = 0; i < nk; i++) {
-        const int s = i % C::kStages;
-        const uint32_t ph = (uint32_t)(i / C::kStages) & 1u;
-        if (i >= C::kStages && !mbar_wait(&empty[s], ph ^ 1u, a.limit_ns)) {
+      const int kx0 = kc0 * (NA == 1 ? slice_k<OP>() : slice_k<OP>() / 2);
+      const int nrow = n0 / NA, nhalf = NA == 1 ? BN / 2 : 0;  // B rows of the tile's two halves
+      for (int j = 0; j < steps; j++) {
+        const int i = j / NA, c = j % NA;
+        const int kx = kx0 + i * slice_k<OP>();
+        if (c == 0) {
+          const int s = i % SB;
+          if (i >= SB && !mbar_wait(&empty_b[s], ((uint32_t)(i / SB) & 1u) ^ 1u, a.limit_ns)) {
+            failed = 1;
+            break;
+          }
+          if (*(volatile int *)&failed) break;
+          unsigned char *st = ring_b + s * 2 * C::kBBytes;
+          mbar_expect_tx(&full_b[s], 2 * C::kBBytes);
+          tma_load_2d(st, &maps.b[0][0], kx, nrow, &full_b[s]);
+          tma_load_2d(st + C::kBBytes / 2, &maps.b[1][0], kx, nrow + nhalf, &full_b[s]);
+          tma_load_2d(st + C::kBBytes, &maps.b[0][1], kx, nrow, &full_b[s]);
+          tma_load_2d(st + C::kBBytes + C::kBBytes / 2, &maps.b[1][1], kx, nrow + nhalf, &full_b[s]);
+          *(volatile int *)&issued_b = i + 1;
+        }
+        const int s = j % SA;
+        if (j >= SA && !mbar_wait(&empty_a[s], ((uint32_t)(j / SA) & 1u) ^ 1u, a.limit_ns)) {
           failed = 1;
           break;
         }
         if (*(volatile int *)&failed) break;
-        unsigned char *st = ring + s * C::kStageBytes;
-        mbar_expect_tx(&full[s], C::kStageBytes);
-        const int kx = (kc0 + i) * slice_k<OP>();
-        tma_load_2d(st, &maps.a_hi, kx, m0, &full[s]);
-        tma_load_2d(st + C::kABytes, &maps.a_lo, kx, m0, &full[s]);
-        tma_load_2d(st + 2 * C::kABytes, &maps.b_hi, kx, n0, &full[s]);
-        tma_load_2d(st + 2 * C::kABytes + C::kBBytes, &maps.b_lo, kx, n0, &full[s]);
-        *(volatile int *)&issued = i + 1;
+        unsigned char *st = ring_a + s * 2 * C::kABytes;
+        mbar_expect_tx(&full_a[s], 2 * C::kABytes);
+        tma_load_2d(st, &maps.a[c][0], kx, m0, &full_a[s]);
+        tma_load_2d(st + C::kABytes, &maps.a[c][1], kx, m0, &full_a[s]);
+        *(volatile int *)&issued_a = j + 1;
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     if (lane == 0) {
       constexpr uint32_t idesc = instr_desc<OP>(kBM, BN);
-      for (int i = 0; i < nk; i++) {
-        const int b = i % C::kBufs;
+      for (int j = 0; j < steps; j++) {
+        const int b = j % C::kBufs, i = j / NA;
         // accumulator b is free once the drain warps have emptied its previous slice
-        if (i >= C::kBufs && !mbar_wait(&tempty[b], (uint32_t)(i / C::kBufs - 1) & 1u, a.limit_ns)) {
+        if (j >= C::kBufs && !mbar_wait(&tempty[b], (uint32_t)(j / C::kBufs - 1) & 1u, a.limit_ns)) {
           failed = 1;
           break;
         }
-        const int s = i % C::kStages;
-        const uint32_t ph = (uint32_t)(i / C::kStages) & 1u;
-        if (*(volatile int *)&failed || !mbar_wait(&full[s], ph, a.limit_ns)) {
+        const int sa = j % SA, sb = i % SB;
+        if (*(volatile int *)&failed || !mbar_wait(&full_b[sb], (uint32_t)(i / SB) & 1u, a.limit_ns)) {
           failed = 1;
           break;
         }
+        *(volatile int *)&consumed_b = i + 1;
+        if (!mbar_wait(&full_a[sa], (uint32_t)(j / SA) & 1u, a.limit_ns)) {
+          failed = 1;
+          break;
+        }
+        *(volatile int *)&consumed_a = j + 1;
         tc_fence_after();
-        const uint32_t sa = smem_u32(ring + s * C::kStageBytes);
+        const uint32_t pa = smem_u32(ring_a + sa * 2 * C::kABytes), pb = smem_u32(ring_b + sb * 2 * C::kBBytes);
         const uint32_t d = tmem + (uint32_t)(b * BN);
+        const int n = NA == 2 && (nk & 1) && i == nb - 1 ? kSteps / 2 : kSteps;
 #pragma unroll
-        for (int kk = 0; kk < kSliceBytes / kMmaKBytes; kk++) {
-          const uint32_t off = kk * kMmaKBytes;  // 32 bytes per MMA step along K
-          const uint64_t ahi = smem_desc(sa + off), alo = smem_desc(sa + C::kABytes + off);
-          const uint64_t bhi = smem_desc(sa + 2 * C::kABytes + off);
-          const uint64_t blo = smem_desc(sa + 2 * C::kABytes + C::kBBytes + off);
-          mma<OP>(d, ahi, bhi, idesc, kk != 0);
-          mma<OP>(d, ahi, blo, idesc, 1u);
-          mma<OP>(d, alo, bhi, idesc, 1u);
+        for (int kk = 0; kk < kSteps; kk++) {
+          if (kk < n) {
+            const uint32_t off = kk * kMmaKBytes;  // 32 bytes per MMA step along K
+            const uint64_t ahi = smem_desc(pa + off), alo = smem_desc(pa + C::kABytes + off);
+            const uint64_t bhi = smem_desc(pb + off), blo = smem_desc(pb + C::kBBytes + off);
+            mma<OP>(d, ahi, bhi, idesc, kk != 0);
+            mma<OP>(d, ahi, blo, idesc, 1u);
+            mma<OP>(d, alo, bhi, idesc, 1u);
+          }
         }
-        mma_commit(&empty[s]);  // the stage returns to the loader when these MMAs have read it
-        mma_commit(&tfull[b]);  // and the accumulator goes to the epilogue warps
-        *(volatile int *)&consumed = i + 1;
+        mma_commit(&empty_a[sa]);  // the stages return to the loader when these MMAs have read them
+        if (j % NA == NA - 1) mma_commit(&empty_b[sb]);
+        mma_commit(&tfull[b]);     // and the accumulator goes to the epilogue warps
       }
     }
     __syncwarp();
   } else {
-    // drain: slice i's partial product (accumulator i % kBufs) added into registers in slice order
-    constexpr int COLS = C::kCols;
+    // drain: step j's partial product (accumulator j % kBufs) added into registers in step order.  A
+    // warp's group g holds HALF real (acc[0 ..]) and HALF imaginary parts (acc[HALF ..]) of the tile's
+    // traps or pixels g HALF ..; plain: columns g HALF .. of both halves of the tile.
+    constexpr int COLS = C::kCols, HALF = COLS / 2;
     const int q = warp & 3;          // TMEM lane quadrant of this warp: rows 32q .. 32q+31
-    const int g = (warp - 2) >> 2;   // its column group: columns g COLS .. (g+1) COLS - 1
-    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * COLS);
+    const int g = (warp - 2) >> 2;   // its column group
+    const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(g * HALF);
     float acc[COLS];
 #pragma unroll
     for (int c = 0; c < COLS; c++) acc[c] = 0.f;
     bool ok = true;
-    for (int i = 0; i < nk; i++) {
-      const int b = i % C::kBufs;
-      ok = mbar_wait(&tfull[b], (uint32_t)(i / C::kBufs) & 1u, a.limit_ns);
+    if constexpr (EPI == kEpiFwd && C::kYBytes > 0) fetch_rows<BN>(a, ring_a + C::kRingBytes, m0, n0 / 2);
+    for (int j = 0; j < steps; j++) {
+      const int b = j % C::kBufs;
+      ok = mbar_wait(&tfull[b], (uint32_t)(j / C::kBufs) & 1u, a.limit_ns);
       ok = __all_sync(0xffffffffu, ok) && !*(volatile int *)&failed;
       if (!ok) break;
       tc_fence_after();
-#pragma unroll
-      for (int c = 0; c < COLS; c += 32) {
-        float v[32];
-        tmem_load32(tq + (uint32_t)(b * BN + c), v);
-#pragma unroll
-        for (int j = 0; j < 32; j++) acc[c + j] += v[j];
-      }
+      // the halves of the accumulator: A_c X_r, A_c X_i.  Re: A_r X_r, then -A_i X_i (conj(X): +); Im:
+      // A_r X_i (conj(X): -), then A_i X_r
+      const bool im = NA == 2 && (j & 1);
+      const uint32_t x = tq + (uint32_t)(b * BN);
+      drain_columns<HALF>(x + (im ? BN / 2 : 0), acc, im && EPI == kEpiBack ? -1.f : 1.f);
+      drain_columns<HALF>(x + (im ? 0 : BN / 2), acc + HALF, !im && EPI == kEpiFwd ? -1.f : 1.f);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[b]);
@@ -507,25 +623,37 @@ __global__ void __launch_bounds__(Cfg<BN>::kThreads, 1) tc_gemm_kernel(const __g
       failed = 1;
       atomicExch(a.err, 1);
     }
-    const int row = m0 + q * 32 + lane;
-    if (EPI == kEpiFwd) {
-      epilogue_fwd<BN>(a, acc, row, n0, red, q, g, ok, &failed);
-    } else if (EPI == kEpiBack && ok) {
-      static_assert(sizeof(BackStage) * C::kEpiWarps <= C::kStages * C::kStageBytes, "staging fits the ring");
-      // the ring is free: every MMA that read it has completed (the last slice was drained)
-      BackStage &st = reinterpret_cast<BackStage *>(ring)[warp - 2];
-#pragma unroll
-      for (int c = 0; c < COLS; c += 32) epilogue_back<OP>(a, acc + c, m0 + q * 32, n0 + g * COLS + c, st);
-    } else if (ok) {
-#pragma unroll
-      for (int c = 0; c < COLS; c += 32) epilogue_plain(a, acc + c, row, n0 + g * COLS + c);
+    if constexpr (EPI == kEpiPlain) {
+      const int row = m0 + q * 32 + lane;
+      if (ok) {
+        epilogue_plain<HALF>(a, acc, row, n0 + g * HALF);
+        epilogue_plain<HALF>(a, acc + HALF, row, n0 + BN / 2 + g * HALF);
+      }
+    } else {
+      // The rings are free once the last step was drained: every MMA that read them has completed.
+      // After a failure copies may still be in flight: nothing is staged, and an incomplete tile
+      // adds and writes nothing (the drain warps agree at a barrier).
+      constexpr int THREADS = 32 * C::kEpiWarps;
+      static_assert(kBM * kStage<BN> * 4 + THREADS * 8 <= C::kRingBytes, "the staged tile fits the rings");
+      if constexpr (EPI == kEpiFwd && C::kYBytes > 0) asm volatile("cp.async.wait_all;" ::: "memory");
+      asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+      if (!*(volatile int *)&failed) {
+        float *const tile = reinterpret_cast<float *>(ring_a);
+        stage_tile<BN>(tile, acc, q, g);
+        if constexpr (EPI == kEpiBack)
+          epilogue_back<BN>(a, tile, m0, n0 / 2);
+        else
+          epilogue_fwd<BN>(a, tile, reinterpret_cast<float4 *>(tile + kBM * kStage<BN>),
+                           reinterpret_cast<const float2 *>(ring_a + C::kRingBytes), m0, n0 / 2);
+      }
     }
   }
   __syncthreads();
   if (threadIdx.x == 0 && failed) {
     atomicExch(a.err, 1);
     // copies still in flight: wait (bounded) until they have landed before the CTA exits
-    for (int i = consumed; i < issued; i++) mbar_wait(&full[i % C::kStages], (uint32_t)(i / C::kStages) & 1u, a.limit_ns);
+    for (int j = consumed_a; j < issued_a; j++) mbar_wait(&full_a[j % SA], (uint32_t)(j / SA) & 1u, a.limit_ns);
+    for (int i = consumed_b; i < issued_b; i++) mbar_wait(&full_b[i % SB], (uint32_t)(i / SB) & 1u, a.limit_ns);
   }
   tc_fence_before();
   __syncthreads();
@@ -538,80 +666,83 @@ __global__ void __launch_bounds__(Cfg<BN>::kThreads, 1) tc_gemm_kernel(const __g
 // ---------------------------------------------------------------------------------------------
 // Operand preparation
 
-// Constant right-hand operands from the complex column tables Xc[m][ix] (once per trap set):
-//   back    Bb[n][k], n = 2 ix + r, k = 2 m + s: [[xr, -xi], [xi, xr]][r][s]    (2W x Kb)
-//   forward Bf[n][k], n = 2 m + r,  k = 2 ix + s: [[xr, xi], [-xi, xr]][r][s]   (2M x Kf)
-// and the row table transposed, YT[iy][m] = Y_m(iy) (m < Kb/2, zero beyond M).  Padding rows and
-// columns are zero.  Rows of Bb and Bf are padded to the tile width, Kb and Kf to a K slice.
+// Constant right-hand operands from the complex column tables Xc[m][ix] (once per trap set), by
+// component and part:
+//   back    b[n = ix][k = m]  (W x ldb, rows padded to rows_b),
+//   forward f[n = m][k = ix]  (M x ldu, rows padded to rows_f),
+// and the row table transposed, YT[iy][m] = Y_m(iy) (m < Kp, zero beyond M).  Padding is zero.
 struct TableArgs {
-  int W, H, M, Kb, Kf, rows_b, rows_f;
+  int W, H, M, Kp, ldb, ldu, rows_b, rows_f;
   const float2 *Xc, *Yc;
-  void *bb_hi, *bb_lo, *bf_hi, *bf_lo;  // operand elements
+  __half *b[2][2], *f[2][2];
   float2 *YT;
 };
 
-template <int OP>
-__global__ void tc_tables_kernel(TableArgs a) {
-  const long long nb = (long long)a.rows_b * a.Kb, nf = (long long)a.rows_f * a.Kf;
-  const long long ny = (long long)a.H * (a.Kb / 2);
+// One thread per two elements along K.
+static __global__ void tc_tables_kernel(TableArgs a) {
+  const long long nb = (long long)a.rows_b * (a.ldb / 2), nf = (long long)a.rows_f * (a.ldu / 2);
+  const long long ny = (long long)a.H * (a.Kp / 2);
   const long long stride = (long long)gridDim.x * blockDim.x;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nb + nf + ny; i += stride) {
-    if (i < nb) {
-      const int n = (int)(i / a.Kb), k = (int)(i % a.Kb);
-      const int ix = n >> 1, r = n & 1, m = k >> 1, s = k & 1;
-      float val = 0.f;
-      if (ix < a.W && m < a.M) {
-        const float2 x = a.Xc[(size_t)m * a.W + ix];
-        val = (r == s) ? x.x : (r == 0 ? -x.y : x.y);
+    const long long j = i < nb ? i : i < nb + nf ? i - nb : i - nb - nf;
+    const int half = i < nb ? a.ldb / 2 : i < nb + nf ? a.ldu / 2 : a.Kp / 2;
+    const int n = (int)(j / half), k = 2 * (int)(j % half);
+    float2 e[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      e[h] = make_float2(0.f, 0.f);
+      if (i < nb) {
+        if (n < a.W && k + h < a.M) e[h] = a.Xc[(size_t)(k + h) * a.W + n];
+      } else if (i < nb + nf) {
+        if (n < a.M && k + h < a.W) e[h] = a.Xc[(size_t)n * a.W + k + h];
+      } else if (k + h < a.M) {
+        e[h] = a.Yc[(size_t)(k + h) * a.H + n];
       }
-      const float2 h = split2<OP>(val);
-      store1<OP>(a.bb_hi, i, h.x);
-      store1<OP>(a.bb_lo, i, h.y);
-    } else if (i < nb + nf) {
-      const long long j = i - nb;
-      const int n = (int)(j / a.Kf), k = (int)(j % a.Kf);
-      const int m = n >> 1, r = n & 1, ix = k >> 1, s = k & 1;
-      float val = 0.f;
-      if (ix < a.W && m < a.M) {
-        const float2 x = a.Xc[(size_t)m * a.W + ix];
-        val = (r == s) ? x.x : (r == 0 ? x.y : -x.y);
-      }
-      const float2 h = split2<OP>(val);
-      store1<OP>(a.bf_hi, j, h.x);
-      store1<OP>(a.bf_lo, j, h.y);
-    } else {
-      const long long j = i - nb - nf;
-      const int iy = (int)(j / (a.Kb / 2)), m = (int)(j % (a.Kb / 2));
-      a.YT[j] = m < a.M ? a.Yc[(size_t)m * a.H + iy] : make_float2(0.f, 0.f);
     }
+    if (i < nb)
+      store_pair(a.b, (size_t)n * a.ldb + k, make_float2(e[0].x, e[1].x), make_float2(e[0].y, e[1].y));
+    else if (i < nb + nf)
+      store_pair(a.f, (size_t)n * a.ldu + k, make_float2(e[0].x, e[1].x), make_float2(e[0].y, e[1].y));
+    else
+      *reinterpret_cast<float4 *>(a.YT + (size_t)n * a.Kp + k) = make_float4(e[0].x, e[0].y, e[1].x, e[1].y);
   }
 }
 
 // The forward operand of given phases: u = e^{i phi} (unit_phasor), split; and one accumulator
 // buffer cleared for the launch after next.
-template <int OP>
-__global__ void tc_phase_kernel(int W, int H, int Kf, const float *phi, void *u_hi, void *u_lo,
-                                unsigned long long *acc_clear, int n_clear) {
+struct PhaseArgs {
+  int W, H, ldu;
+  const float *phi;
+  __half *u[2][2];
+  unsigned long long *acc_clear;
+  int n_clear;
+};
+static __global__ void tc_phase_kernel(PhaseArgs a) {
   grid_wait();
-  const long long N = (long long)W * H, stride = (long long)gridDim.x * blockDim.x;
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < N; j += stride) {
-    const int iy = (int)(j / W), ix = (int)(j % W);
-    float sn, cs;
-    unit_phasor(phi[j], sn, cs);
-    store_split<OP>(u_hi, u_lo, (size_t)iy * Kf + 2 * ix, cs, sn);
+  const int half = (a.W + 1) / 2;
+  const long long n = (long long)a.H * half, stride = (long long)gridDim.x * blockDim.x;
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n; j += stride) {
+    const int iy = n <= 0x7fffffffll ? (int)((unsigned)j / (unsigned)half) : (int)(j / half);
+    const int ix = 2 * (int)(j - (long long)iy * half);
+    const float *ph = a.phi + (size_t)iy * a.W + ix;
+    float2 sn, cs;
+    unit_phasor(ph[0], sn.x, cs.x);
+    sn.y = cs.y = 0.f;
+    if (ix + 1 < a.W) unit_phasor(ph[1], sn.y, cs.y);
+    store_pair(a.u, (size_t)iy * a.ldu + ix, cs, sn);
   }
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_clear; i += stride) acc_clear[i] = 0ull;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n_clear; i += stride) a.acc_clear[i] = 0ull;
   grid_release();
 }
 
 struct PrepArgs {
-  int H, M, Kb;
+  int H, M, Kp, ldb;                 // Kp: M padded (row stride of YT); ldb: row stride of P
   const unsigned long long *acc_in;  // [2][M] sums of the previous forward
   unsigned long long *acc_clear;     // [2][M] cleared here
   const float *w_in;
   float *w_out;                      // written by block 0
-  const float2 *YT;                  // [H][Kb/2]
-  void *p_hi, *p_lo;                 // [..][Kb] operand elements
+  const float2 *YT;                  // [H][Kp]
+  __half *p[2][2];                   // [..][ldb] by component and part
   float inv_fx_n;
   float *trace;                      // NULL, or e, u of the fields read (block 0)
 };
@@ -629,37 +760,44 @@ __device__ __forceinline__ ffp ffp_add(ffp a, ffp b) {  // TwoSum (Knuth) + reno
 }
 
 constexpr int kPrepThreads = 256;
-constexpr int kPrepPrefetch = 16;  // row-table elements a thread of tc_prep_kernel fetches before the wait
+constexpr int kPrepWeights = 4;   // weights a thread of tc_prep_kernel fetches before the wait
+constexpr int kPrepPrefetch = 8;  // pairs of row-table elements a thread of tc_prep_kernel fetches before the wait
 
 // Sec. 3 weight update and the back-projection operand of one iteration: every block reads the
-// field sums, forms V_m, <|V|> (float-float sum in one fixed order, so every block obtains the
-// same bits) and the coefficients c_m = w_m' V_m/|V_m| with w_m' = w_m <|V|>/|V_m| (|V_m| < 1e-30:
-// c_m = w_m, w kept) in shared memory, then writes its share of P[iy][2m..2m+1] = c_m Y_m(iy),
-// split.  Block 0 writes the new weights (and the trace); the blocks clear the next buffer.
-// The row table is constant during hot_gsw: a thread's first kPrepPrefetch elements of it are
-// fetched before the wait for the previous kernel (they come from HBM: the GEMMs' operands have
-// pushed the table out of L2).
-template <int OP>
-__global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(PrepArgs a) {
+// field sums, forms V_m and the coefficients c_m = w_m' V_m/|V_m| with w_m' = w_m <|V|>/|V_m|
+// (|V_m| < 1e-30: c_m = w_m, w kept) in shared memory, up to a common factor -- so <|V|>, a block-wide
+// sum, is not waited for unless a field vanishes -- then writes its share of P[iy][m] = c_m Y_m(iy),
+// split.  Block 0 then writes the new weights (and the trace), <|V|> from a float-float sum in one
+// fixed order; the blocks clear the next buffer.
+// The row table is constant during hot_gsw, and the weights are the previous iteration's, which ended
+// before the kernel ahead of this one could start: a thread's first elements of both are fetched before
+// the wait for that kernel (the table comes from HBM: the GEMMs' operands have pushed it out of L2;
+// the weights ahead of the wait save 0.2 us of 12 at 256^2, 1.5 of 100 at 1920 x 1152 with 1000 traps).
+static __global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(PrepArgs a) {
   extern __shared__ float2 cs[];  // [M]
   __shared__ ffp part[2][kPrepThreads / 32];
   __shared__ float ext[2][kPrepThreads / 32];
   __shared__ float cmx[kPrepThreads / 32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  // this block's rows of P: an even share of the H rows, all Kb/2 (padded) traps of each
-  const int half = a.Kb / 2;
+  // this block's rows of P: an even share of the H rows, all Kp (padded) traps of each, two at a time
+  const int half = a.Kp / 2;
+  const float4 *const YT = reinterpret_cast<const float4 *>(a.YT);
   const int r0 = (int)((long long)a.H * blockIdx.x / gridDim.x);
   const int r1 = (int)((long long)a.H * (blockIdx.x + 1) / gridDim.x);
   const int n = (r1 - r0) * half;
-  float2 ypre[kPrepPrefetch];
+  float4 ypre[kPrepPrefetch];
 #pragma unroll
   for (int j = 0; j < kPrepPrefetch; j++) {
     const int i = t + j * kPrepThreads;
-    ypre[j] = i < n ? __ldg(a.YT + (size_t)r0 * half + i) : make_float2(0.f, 0.f);
+    ypre[j] = i < n ? __ldg(YT + (size_t)r0 * half + i) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
+  float wpre[kPrepWeights];
+#pragma unroll
+  for (int j = 0; j < kPrepWeights; j++) wpre[j] = t + j * kPrepThreads < a.M ? __ldcg(a.w_in + t + j * kPrepThreads) : 0.f;
   grid_wait();
   ffp s = {0.f, 0.f}, si = {0.f, 0.f};
   float mx = -1.f, mn = 3.0e38f;
+#pragma unroll 4
   for (int m = t; m < a.M; m += kPrepThreads) {
     const float vr = (float)(long long)__ldcg(a.acc_in + m) * a.inv_fx_n;
     const float vi = (float)(long long)__ldcg(a.acc_in + a.M + m) * a.inv_fx_n;
@@ -683,11 +821,81 @@ __global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(PrepArgs a) {
     ext[0][warp] = mx;
     ext[1][warp] = mn;
   }
-  __syncthreads();
-  ffp q = part[0][0];
-  for (int i = 1; i < kPrepThreads / 32; i++) q = ffp_add(q, part[0][i]);
-  const float mean = (q.hi + q.lo) / (float)a.M;  // <|V|> (Sec. 3)
-  if (a.trace && blockIdx.x == 0 && t == 0) {  // e, u (Eq. 4) of the fields read
+  // the coefficients over <|V|> (arg S does not depend on a common factor)
+  float cmax = 0.f;  // largest magnitude: they are scaled by its inverse below
+  bool zero = false;
+  auto coefficient = [&](int m, float w) {
+    const float2 v = cs[m];
+    const float am = sqrtf(v.x * v.x + v.y * v.y), wn = w / am;
+    if (am >= 1e-30f) {
+      cs[m] = make_float2(wn * (v.x / am), wn * (v.y / am));
+      cmax = fmaxf(cmax, wn);
+    } else {
+      zero = true;
+    }
+  };
+#pragma unroll
+  for (int j = 0; j < kPrepWeights; j++)
+    if (t + j * kPrepThreads < a.M) coefficient(t + j * kPrepThreads, wpre[j]);
+  for (int m = t + kPrepWeights * kPrepThreads; m < a.M; m += kPrepThreads) coefficient(m, __ldcg(a.w_in + m));
+#pragma unroll
+  for (int o = 16; o; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
+  if (lane == 0) cmx[warp] = cmax;
+  const long long stride = (long long)gridDim.x * kPrepThreads;
+  for (long long i = blockIdx.x * (long long)kPrepThreads + t; i < 2LL * a.M; i += stride) a.acc_clear[i] = 0ull;
+  const bool any_zero = __syncthreads_or(zero);
+  // A factor common to all coefficients leaves arg S unchanged (Sec. 4; the weights' scale is
+  // free): P is formed from c_m / max |c| so that its magnitudes stay near 1 whatever the
+  // weights' scale (the FP16 operands lose precision below ~0.25).
+  float top = cmx[0];
+  for (int i = 1; i < kPrepThreads / 32; i++) top = fmaxf(top, cmx[i]);
+  auto mean_field = [&] {
+    ffp q = part[0][0];
+    for (int i = 1; i < kPrepThreads / 32; i++) q = ffp_add(q, part[0][i]);
+    return (q.hi + q.lo) / (float)a.M;
+  };
+  if (any_zero) {  // vanishing fields: c_m = w_m / <|V|> in this scale (w_m where every field vanishes)
+    const float mean = mean_field(), inv = mean > 0.f ? 1.f / mean : 1.f;
+    float zmax = 0.f;
+    for (int m = 0; m < a.M; m++) {  // (every thread: the largest of them)
+      const float vr = (float)(long long)__ldcg(a.acc_in + m) * a.inv_fx_n;
+      const float vi = (float)(long long)__ldcg(a.acc_in + a.M + m) * a.inv_fx_n;
+      if (sqrtf(vr * vr + vi * vi) >= 1e-30f) continue;
+      const float w = __ldcg(a.w_in + m) * inv;
+      zmax = fmaxf(zmax, w);
+      if (m % kPrepThreads == t) cs[m] = make_float2(w, 0.f);
+    }
+    top = fmaxf(top, zmax);
+    __syncthreads();
+  }
+  const float scale = top > 0.f ? 1.f / top : 1.f;
+  // pair i of the block's rows is P[r0 + i / half][m = 2 (i % half), + 1], pair i of the row table
+  auto put = [&](int i, float4 y) {
+    const int m = 2 * (i % half);
+    float2 c[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++)
+      c[h] = m + h < a.M ? make_float2(cs[m + h].x * scale, cs[m + h].y * scale) : make_float2(0.f, 0.f);
+    store_pair(a.p, (size_t)(r0 + i / half) * a.ldb + m,
+               make_float2(c[0].x * y.x - c[0].y * y.y, c[1].x * y.z - c[1].y * y.w),
+               make_float2(c[0].x * y.y + c[0].y * y.x, c[1].x * y.w + c[1].y * y.z));
+  };
+#pragma unroll
+  for (int j = 0; j < kPrepPrefetch; j++)
+    if (t + j * kPrepThreads < n) put(t + j * kPrepThreads, ypre[j]);
+  for (int i = t + kPrepPrefetch * kPrepThreads; i < n; i += kPrepThreads) put(i, __ldg(YT + (size_t)r0 * half + i));
+  grid_release();
+  if (blockIdx.x) return;
+  // Block 0: the weights w_m' = w_m <|V|>/|V_m| (Sec. 3), and e, u (Eq. 4) of the fields read
+  const float mean = mean_field();
+  for (int m = t; m < a.M; m += kPrepThreads) {
+    const float w = __ldcg(a.w_in + m);
+    const float vr = (float)(long long)__ldcg(a.acc_in + m) * a.inv_fx_n;
+    const float vi = (float)(long long)__ldcg(a.acc_in + a.M + m) * a.inv_fx_n;
+    const float am = sqrtf(vr * vr + vi * vi);
+    a.w_out[m] = am < 1e-30f ? w : w * mean / am;
+  }
+  if (a.trace && t == 0) {
     ffp e = part[1][0];
     float hi = ext[0][0], lo = ext[1][0];
     for (int i = 1; i < kPrepThreads / 32; i++) {
@@ -698,46 +906,6 @@ __global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(PrepArgs a) {
     a.trace[0] = e.hi + e.lo;
     a.trace[1] = (hi + lo > 0.f) ? 1.f - (hi - lo) / (hi + lo) : 0.f;
   }
-  float cmax = 0.f;  // largest |c_m| (= w_m'): the coefficients are scaled by its inverse below
-  for (int m = t; m < a.M; m += kPrepThreads) {
-    const float2 v = cs[m];
-    const float w = __ldcg(a.w_in + m);
-    const float am = sqrtf(v.x * v.x + v.y * v.y);
-    float2 c;
-    float wn = w;
-    if (am < 1e-30f) {
-      c = make_float2(w, 0.f);
-    } else {
-      wn = w * mean / am;
-      c = make_float2(wn * (v.x / am), wn * (v.y / am));
-    }
-    if (blockIdx.x == 0) a.w_out[m] = wn;
-    cs[m] = c;
-    cmax = fmaxf(cmax, wn);
-  }
-#pragma unroll
-  for (int o = 16; o; o >>= 1) cmax = fmaxf(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
-  if (lane == 0) cmx[warp] = cmax;
-  const long long stride = (long long)gridDim.x * kPrepThreads;
-  for (long long i = blockIdx.x * (long long)kPrepThreads + t; i < 2LL * a.M; i += stride) a.acc_clear[i] = 0ull;
-  __syncthreads();
-  // A factor common to all coefficients leaves arg S unchanged (Sec. 4; the weights' scale is
-  // free): P is formed from c_m / max |c| so that its magnitudes stay near 1 whatever the
-  // weights' scale (the FP16 operands lose precision below ~0.25).
-  float top = cmx[0];
-  for (int i = 1; i < kPrepThreads / 32; i++) top = fmaxf(top, cmx[i]);
-  const float scale = top > 0.f ? 1.f / top : 1.f;
-  // element i of the block's rows is P[r0 + i / half][m = i % half], at i of the row-major table
-  auto put = [&](int i, float2 y) {
-    const int m = i % half;
-    const float2 c = m < a.M ? make_float2(cs[m].x * scale, cs[m].y * scale) : make_float2(0.f, 0.f);
-    store_split<OP>(a.p_hi, a.p_lo, 2 * ((size_t)r0 * half + i), c.x * y.x - c.y * y.y, c.x * y.y + c.y * y.x);
-  };
-#pragma unroll
-  for (int j = 0; j < kPrepPrefetch; j++)
-    if (t + j * kPrepThreads < n) put(t + j * kPrepThreads, ypre[j]);
-  for (int i = t + kPrepPrefetch * kPrepThreads; i < n; i += kPrepThreads) put(i, __ldg(a.YT + (size_t)r0 * half + i));
-  grid_release();
 }
 
 // Operands of the plain GEMM entry point: src [rows][K] -> hi, lo [rows_pad][K_pad], zero padded.
