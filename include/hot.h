@@ -67,14 +67,14 @@ typedef enum {
                              fixed pseudo-random angle and its sums back, so that the unit's
                              systematic error does not add up over the pixels */
   HOT_PREC_SEPARABLE = 2, /* Eq. 2 factorised: e^{i Delta} = e^{i X_m(ix)} e^{i Y_m(iy)} from FP32
-                             complex tables (FP64 cos/sin once per entry); per pair one complex
+                             complex tables (exactly reduced phases); per pair one complex
                              multiply-add in each step, no transcendental function; the state is
                              the phases at every trap count (hot_get_phasors) */
   HOT_PREC_TENSOR = 3      /* EXPERIMENTAL, outside the direct method: the separable form on the
                              tensor cores; each step of a GSW iteration is a complex matrix product
                              (S = P X, T = U X^H) run as tcgen05 FP16 MMAs with every operand split
                              in two FP16 parts (three MMAs per product, FP32 accumulation); the GSW
-                             loop only (hot_gsw), other calls run the separable kernels; |V_m|
+                             loop only (hot_gsw), other calls run the separable mode's; |V_m|
                              error up to 5e-4 on strongly cancelling back-projections (above) */
 } hot_precision;
 
@@ -97,7 +97,7 @@ int hot_create(hot_ctx **out, int width, int height, double pitch_m, double wave
 /* Sets the M traps (Sec. 4 "trap structure"): xyz_m is a host array of M*3 doubles
  * (x_m, y_m, z_m) in metres, row per trap; w0 (host, M doubles > 0, or NULL for all 1) are
  * the initial GSW weights.  1 <= M <= HOT_MAX_TRAPS, coordinates finite.  Builds the
- * per-trap phase tables on the device (Eq. 2 reduced modulo 2 pi in FP64). */
+ * per-trap phase tables on the device (Eq. 2 reduced modulo 2 pi exactly). */
 int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0);
 
 /* Replaces the GSW weights (host, M doubles > 0).  HOT_ESTATE before hot_set_traps. */
@@ -108,11 +108,11 @@ int hot_set_weights(hot_ctx *c, const double *w);
 int hot_set_phase(hot_ctx *c, const float *phi, int on_device);
 
 /* Selects HOT_PREC_ACCURATE, HOT_PREC_FAST, HOT_PREC_SEPARABLE or HOT_PREC_TENSOR for the
- * following calls (switching between the direct and the separable kernels synchronises and
- * rebuilds the work schedule).  HOT_EINVAL for another value.  In HOT_PREC_TENSOR mode hot_gsw
+ * following calls (a switch that needs other tables or buffers synchronises and rebuilds the
+ * work schedule).  HOT_EINVAL for another value.  In HOT_PREC_TENSOR mode hot_gsw
  * runs three kernels per iteration (weight update and operand P, back-projection GEMM with the
  * phases in its epilogue, forward GEMM with the field sums in its epilogue); its operands
- * (about 4 (2W + 2M)(2M + 2W) + 8 H (W + M) + 8 H M bytes) are built on the first hot_gsw after the
+ * (about 16 M (W + H) + 8 W H bytes) are built on the first hot_gsw after the
  * traps are set (row-band steps, hot_sharded_*, run the same kernels).  HOT_PREC_TENSOR rejects the
  * persistent form (hot_use_persistent) and hot_autotune with HOT_EINVAL; its batches run each
  * member's own launch sequence (see hot_batch_create). */
@@ -332,7 +332,7 @@ int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chun
  * first) and cut into groups of at least `group_pairs` pairs per iteration (and at most 22
  * holograms: their parameters travel in the kernel launch); each group runs
  * its iterations with one kernel launch per iteration that covers all of its holograms (their
- * row segments are dealt out to one wave of blocks in equal shares of pairs), and the groups
+ * tiles are dealt out to one wave of blocks in equal shares of pairs), and the groups
  * run one after another, so that small holograms neither leave the GPU idle nor wait for the
  * large ones.  Each hologram keeps its own tables, phases, weights and accumulators (its
  * context's buffers); the iteration is the same as hot_gsw's (Sec. 3). */

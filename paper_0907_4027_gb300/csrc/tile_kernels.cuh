@@ -1,7 +1,7 @@
 // tile_kernels.cuh -- the register-tiled step kernel of the accurate, fast and separable modes.
 //
 // Eq. 2 is a sum of a column part and a row part, so a pair's exponential is the product of two
-// tabulated unit phasors, e^{i Delta_j^m} = X_m(ix) Y_m(iy) (FP64 cos/sin of the exactly reduced
+// tabulated unit phasors, e^{i Delta_j^m} = X_m(ix) Y_m(iy) (cos and sin of the exactly reduced
 // turns, rounded to FP32 once per trap set).  Both sums of an iteration are then complex
 // multiply-adds,
 //   S_j = sum_m (c_m X_m(ix)) Y_m(iy)                            (back-projection, Sec. 3-4)
