@@ -334,7 +334,8 @@ int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chun
  * its iterations with one kernel launch per iteration that covers all of its holograms (their
  * tiles are dealt out to one wave of blocks in equal shares of pairs), and the groups
  * run one after another, so that small holograms neither leave the GPU idle nor wait for the
- * large ones.  Each hologram keeps its own tables, phases, weights and accumulators (its
+ * large ones.  A group of one hologram runs the step and tiles of its own hot_gsw, unless a tiling
+ * was asked for.  Each hologram keeps its own tables, phases, weights and accumulators (its
  * context's buffers); the iteration is the same as hot_gsw's (Sec. 3). */
 typedef struct hot_batch hot_batch;
 

@@ -450,50 +450,65 @@ int tile_team(int M, long long row_pairs, int sms) {
   return best;
 }
 
-// The tile kernels' schedule: one wave of their blocks, the strips' row pairs dealt out to the
+// A hologram's tiles (hot::TileArgs): one wave of blocks, the strips' row pairs dealt out to the
 // teams in equal runs, cut into tiles of at most hot::kTilePairs pairs.
+struct TileCut {
+  int grid = 0, team = 1, pairs = 3, stride = 1;
+  std::vector<hot::SubTile> tiles;  // team i's are [i stride], ...; the first one's pad says how many
+};
+
+int cut_tiles(int W, int H, int M, int sms, TileCut &cut) {
+  const int P = (H + 1) / 2;
+  const long long U = (long long)((W + hot::kTileCols - 1) / hot::kTileCols) * P;
+  cut.team = tile_team(M, U, sms);
+  const int teams = hot::kWarps / cut.team;
+  std::vector<hot::SubTile> sub;
+  std::vector<int> first;
+  int per_sm = 0;
+  // two blocks per SM, or the one that fits beside very many traps' coefficients
+  for (int want = 2; want >= 1; want--) {
+    cut.grid = (int)std::min<long long>((long long)sms * want, (U + teams - 1) / teams);
+    cut_schedule(W, P, cut.grid * teams, hot::kTilePairs, sub, first, hot::kTileCols);
+    cut.pairs = 3;
+    for (const hot::SubTile &t : sub) cut.pairs = std::max(cut.pairs, t.rows);
+    HOT_CUDA(hot_tile::occupancy(M, cut.team, cut.pairs, &per_sm));
+    if (per_sm >= want) break;
+  }
+  if (per_sm < 1) return fail(HOT_ECUDA, "no tile kernel for %d traps", M);
+  const int n = cut.grid * teams;
+  cut.stride = 1;
+  for (int i = 0; i < n; i++) cut.stride = std::max(cut.stride, first[i + 1] - first[i]);
+  cut.tiles.assign((size_t)n * cut.stride, hot::SubTile{0, 0, 0, 0});
+  for (int i = 0; i < n; i++)
+    for (int j = first[i]; j < first[i + 1]; j++) {
+      hot::SubTile &t = cut.tiles[(size_t)i * cut.stride + j - first[i]] = sub[j];
+      t.y0 *= 2;
+      t.pad = first[i + 1] - j;
+    }
+  return HOT_OK;
+}
+
+// The tile kernels' schedule of a context.
 int build_tile_schedule(hot_ctx *c, int sms) {
   c->once = false;
   c->tgrid = 0;
   dfree(c->tsub);
   if (!tile_kernels(c)) return HOT_OK;
-  const int P = (c->H + 1) / 2;
-  const long long U = (long long)((c->W + hot::kTileCols - 1) / hot::kTileCols) * P;
-  const int team = tile_team(c->M, U, sms), teams = hot::kWarps / team;
-  std::vector<hot::SubTile> sub;
-  std::vector<int> first;
-  int G = 0, pairs = 0, per_sm = 0;
-  // two blocks per SM, or the one that fits beside very many traps' coefficients
-  for (int want = 2; want >= 1; want--) {
-    G = (int)std::min<long long>((long long)sms * want, (U + teams - 1) / teams);
-    cut_schedule(c->W, P, G * teams, hot::kTilePairs, sub, first, hot::kTileCols);
-    pairs = 3;
-    for (const hot::SubTile &t : sub) pairs = std::max(pairs, t.rows);
-    HOT_CUDA(hot_tile::occupancy(c->M, team, pairs, &per_sm));
-    if (per_sm >= want) break;
-  }
-  if (per_sm < 1) return fail(HOT_ECUDA, "no tile kernel for %d traps", c->M);
-  int stride = 1;
-  for (int i = 0; i < G * teams; i++) stride = std::max(stride, first[i + 1] - first[i]);
-  std::vector<hot::SubTile> tiles((size_t)G * teams * stride, hot::SubTile{0, 0, 0, 0});
-  for (int i = 0; i < G * teams; i++)
-    for (int j = first[i]; j < first[i + 1]; j++) {
-      hot::SubTile &t = tiles[(size_t)i * stride + j - first[i]] = sub[j];
-      t.y0 *= 2;
-      t.pad = first[i + 1] - j;
-    }
-  const int rc0 = dalloc(&c->tsub, tiles.size());
+  TileCut cut;
+  const int rc0 = cut_tiles(c->W, c->H, c->M, sms, cut);
   if (rc0 != HOT_OK) return rc0;
-  HOT_CUDA(cudaMemcpy(c->tsub, tiles.data(), sizeof(hot::SubTile) * tiles.size(), cudaMemcpyHostToDevice));
-  c->tstride = stride;
+  const int rc1 = dalloc(&c->tsub, cut.tiles.size());
+  if (rc1 != HOT_OK) return rc1;
+  HOT_CUDA(cudaMemcpy(c->tsub, cut.tiles.data(), sizeof(hot::SubTile) * cut.tiles.size(), cudaMemcpyHostToDevice));
+  c->tstride = cut.stride;
   c->once = !separable_kernels(c) && c->M <= hot::kOnceMaxM;
   if (c->once && !c->ubuf) {
     const int rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
     if (rc != HOT_OK) return rc;
   }
-  c->tgrid = G;
-  c->tteam = team;
-  c->tpairs = pairs;
+  c->tgrid = cut.grid;
+  c->tteam = cut.team;
+  c->tpairs = cut.pairs;
   return HOT_OK;
 }
 
@@ -1451,6 +1466,7 @@ struct hot_batch {
     std::vector<int> owner;                  // block that writes each hologram's weights
     std::vector<hot::TileArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
     int M = 1, pairs = 3;                    // shared-memory layout (hot::TileBatchArgs)
+    bool alone = false;                      // one hologram, on tiles and teams of its own
     hot::FinalizeArgs *fin[6] = {};          // finalize descriptors for iters % 6
   };
   std::vector<Group> groups;
@@ -1512,6 +1528,11 @@ double pairs_of(const hot_ctx *c) { return n_total(c) * (double)c->M; }
 // trap count, dealt out to one wave of G blocks in equal shares (a row pair goes to the block
 // that holds the midpoint of its weight interval); each block's run of pairs in a strip is cut
 // into equal tiles of <= rows / 2 pairs (the default 14: hot::kTilePairs).
+// A group of one hologram, as those of 2^26 pairs and more are, runs hot_gsw's step on its own cut
+// unless a tiling was asked for: the batched kernel's blocks are one team of 8 warps (a tile's traps
+// split eight ways whatever their number), which large holograms with smaller teams outrun
+// (8 holograms up to 1920 x 1152 with up to 2000 traps, 5 iterations: 16.55 -> 14.75 ms; 64 of them 965 ->
+// 853 ms, one by one 851).
 int build_group(hot_batch *b, hot_batch::Group &g) {
   const int count = (int)g.members.size();
   const int per_sm = b->bps > 0 ? std::min(b->bps, b->per_sm_max) : b->per_sm_max;
@@ -1525,6 +1546,13 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
     g.M = std::max(g.M, c->M);
   }
   const int pairs = b->rows >= hot::kRowsMax ? hot::kTilePairs : (b->rows + 1) / 2;
+  g.alone = count == 1 && pairs == hot::kTilePairs && per_sm == b->per_sm_max;
+  TileCut cut;
+  if (g.alone) {
+    const hot_ctx *c = b->ctx[g.members[0]];
+    const int rc = cut_tiles(c->W, c->H, c->M, b->sms, cut);
+    if (rc != HOT_OK) return rc;
+  }
   const int G = (int)std::min<long long>((long long)b->sms * per_sm, segments);
   std::vector<hot::SubTile> sub;
   std::vector<int> first(G + 1, 0), owner(count, -1);
@@ -1558,7 +1586,8 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
     }
   }
   while (cur_b < G) first[++cur_b] = (int)sub.size();
-  g.grid = G;
+  if (g.alone) sub = cut.tiles;
+  g.grid = g.alone ? cut.grid : G;
   g.n_sub = (int)sub.size();
   g.owner = owner;
   int rc = dalloc(&g.sub, sub.size());
@@ -1571,8 +1600,9 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
       t.s.sub = g.sub;
       t.s.first = g.first;
       t.s.trace = nullptr;
-      t.team = hot::kWarps;
-      t.pairs = g.pairs;
+      t.team = g.alone ? cut.team : hot::kWarps;
+      t.pairs = g.alone ? cut.pairs : g.pairs;
+      t.stride = cut.stride;
     }
   }
   for (int r6 = 0; rc == HOT_OK && r6 < 6; r6++) {  // finalize after `iters` iterations, iters % 6 == r6
@@ -1648,7 +1678,7 @@ template <bool BACK>
 int batch_launch(hot_batch *b, const hot_batch::Group &g, int k) {
   hot::TileBatchArgs a = {};
   const int count = (int)g.members.size();
-  for (int i = 0; i < count; i++) {
+  for (int i = 0; i < count && !g.alone; i++) {
     a.holo[i] = g.holo[k % 6][i];
     a.owner[i] = g.owner[i];
   }
@@ -1665,7 +1695,10 @@ int batch_launch(hot_batch *b, const hot_batch::Group &g, int k) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  hot_tile::launch_batch(BACK, cfg, a);
+  if (g.alone)
+    hot_tile::launch(BACK, true, false, cfg, g.holo[k % 6][0]);
+  else
+    hot_tile::launch_batch(BACK, cfg, a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_tile_batch_kernel: %s", cudaGetErrorString(e));
   return HOT_OK;
