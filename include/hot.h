@@ -332,11 +332,15 @@ int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chun
  * first) and cut into groups of at least `group_pairs` pairs per iteration (and at most 22
  * holograms: their parameters travel in the kernel launch); each group runs
  * its iterations with one kernel launch per iteration that covers all of its holograms (their
- * tiles are dealt out to one wave of blocks in equal shares of pairs), and the groups
+ * row segments are dealt out to one wave of blocks in equal shares of pairs), and the groups
  * run one after another, so that small holograms neither leave the GPU idle nor wait for the
- * large ones.  A group of one hologram runs the step and tiles of its own hot_gsw, unless a tiling
- * was asked for.  Each hologram keeps its own tables, phases, weights and accumulators (its
- * context's buffers); the iteration is the same as hot_gsw's (Sec. 3). */
+ * large ones.  Each hologram keeps its own tables, phases, weights and accumulators (its
+ * context's buffers); the iteration is the same as hot_gsw's (Sec. 3).
+ * The launches evaluate every pair directly in the accurate and fast modes (as hot_set_once(c, 0)
+ * does) and from FP64-built complex tables in the separable mode: a batch goes on from its own
+ * state call after call, and rounding that a sequence amplifies stays as it was.  With one group
+ * per hologram (hot_batch_set_tiling, group_pairs <= 1) and no tiling asked for, each member runs
+ * the step and tiles of its own hot_gsw instead, which is about twice as fast for large holograms. */
 typedef struct hot_batch hot_batch;
 
 /* Groups count >= 1 contexts (same device, traps set, same precision mode, not row bands)
@@ -354,7 +358,8 @@ int hot_batch_create(hot_batch **out, int count, hot_ctx *const *ctxs, void *cud
 
 /* Tiling of the batch's launches (as hot_set_tiling; 0 selects a default) and the minimum
  * work of a group in pixel-trap pairs per iteration (0: 2^26; 1: every hologram its own
- * group; a value above the total: one group, all holograms in lockstep).  Rebuilds the
+ * group, on the step of its own hot_gsw unless rows, blocks_per_sm or chunk ask for another tiling; a
+ * value above the total: one group, all holograms in lockstep).  Rebuilds the
  * schedule; synchronises the batch's stream. */
 int hot_batch_set_tiling(hot_batch *b, int rows, int blocks_per_sm, int chunk, double group_pairs);
 

@@ -40,6 +40,7 @@ constexpr int kYStride = (kRowsMax + 3) & ~3;  // floats per trap in the staged 
 static_assert(kTileW == 32 && kYStride == 16, "16-byte staging of 32 columns and 16 rows per trap");
 constexpr int kChunk = 128;     // traps whose tables are staged in shared memory at once
 constexpr float kTwoPi = 6.283185307179586f;
+constexpr int kModeAccurate = 0, kModeFast = 1, kModeSeparable = 2;  // variants of the batched kernel
 
 // Work decomposition: the image is cut into 32-pixel-wide column strips; each strip's rows
 // are dealt out as contiguous runs to a fixed number of resident blocks (one wave), so that
@@ -53,7 +54,7 @@ struct StepArgs {
   int W, H, M;
   int chunk;              // traps staged in shared memory at once (1..kChunk)
   int copies;             // copies of each fixed-point accumulator buffer (a power of two; more than
-                          // one with the tile kernels only): block b adds into copy b % copies,
+                          // one with the tile kernels and in separable batches): block b adds into copy b % copies,
                           // spreading the atomics over more addresses
   int ldy4;               // row stride of Y4 (below)
   const SubTile *sub;     // work schedule: sub-tiles
@@ -63,6 +64,10 @@ struct StepArgs {
   const float *Y4;        // NULL, or [4][M][ldy4]: copy s holds Y shifted by s rows (Y4[s][m][i + s] =
                           // Y[m][i], zero elsewhere), so that every sub-tile's rows start 16-byte aligned
                           // in one of the copies
+  const float2 *Xc;       // [M][W] e^{i 2pi X} (separable batches)
+  const float2 *Yc;       // [2][M][ldy4] e^{i 2pi Y} (separable batches), in two copies: copy s holds the
+                          // rows shifted by s (Yc[s][m][i + s] = e^{i 2pi Y_m(i)}, zero elsewhere), so
+                          // that every sub-tile's rows start 16-byte aligned in one of them
   float *phi;             // [H*W] pixel phases, radians
   // BACK: weight update and coefficients from the previous launch's forward field
   const unsigned long long *acc_in;  // [copies][2][M] fixed-point sums of the previous forward: Re, Im
@@ -494,12 +499,14 @@ struct LateWeight {
 };
 
 // Start of a GSW step: the previous forward's fields are read once, every load issued before
-// any is used.  Writes the coefficients of traps [0, mc) into C0 (polar) without the factor <|V|> of the weight update: a factor common to all coefficients
+// any is used.  Writes the coefficients of traps [0, mc) into C0 (polar, or complex when
+// COMPLEX) without the factor <|V|> of the weight update: a factor common to all coefficients
 // scales S_j and leaves arg S_j unchanged (the weights' global scale is free, reading R6), so
 // no block-wide reduction stands between the sums and the back-projection.  Keeps in lw the
 // thread's share of sum |V_m| and the prefetched weight of trap own + stride * gthread(),
 // which write_weights completes after the block's work.
 // trace: NULL, or where block 0 writes e and u (Eq. 4) of the fields it read (convergence trace).
+template <bool COMPLEX>
 __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *C0, int own, int stride,
                                              LateWeight &lw, float *trace = nullptr) {
   const int t = gthread();
@@ -508,7 +515,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
   lw.v = make_float2(0.f, 0.f);
   lw.w = 0.f;
   if (lw.m < a.M) {
-    lw.v = field_from_sums(a, lw.m);
+    lw.v = field_from_sums<COMPLEX>(a, lw.m);
     lw.w = __ldcg(a.w_in + lw.m);
   }
   const float w0 = t < mc ? __ldcg(a.w_in + t) : 0.f;
@@ -518,7 +525,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
   ff si = {0.f, 0.f};
   float mx = -1.f, mn = 3.0e38f;
   for (int m = t; m < a.M; m += kThreads) {
-    const float2 v = field_from_sums(a, m);
+    const float2 v = field_from_sums<COMPLEX>(a, m);
     if (m == t) v0 = v;
     s = ff_add(s, {sqrtf(abs2(v)), 0.f});
     if (tr) {
@@ -529,7 +536,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
     }
   }
   lw.part = s;
-  if (t < mc) C0[t] = update_from<false>(v0, w0, 1.f, a.angle_units, a.angle_eta);
+  if (t < mc) C0[t] = update_from<COMPLEX>(v0, w0, 1.f, a.angle_units, a.angle_eta);
   if (tr) {  // virtual block 0 only: e = sum I_m, u = 1 - (max - min)/(max + min) of the fields read
     __shared__ ff tpart[kWarps];
     __shared__ float ext[2][kWarps];  // (group 0 of block 0 alone uses these)
@@ -563,6 +570,7 @@ __device__ __forceinline__ void gsw_prologue(const StepArgs &a, int mc, float2 *
 // of |V_m| over the traps, Sec. 3) from the threads' shares in one fixed order (warp
 // shuffles, warps in order), so every such block obtains the same bits, and the block's
 // weight updates w_m <- w_m <|V|>/|V_m| (traps lw.m, lw.m + stride * kThreads, ...).
+template <bool MULTI = false>
 __device__ __forceinline__ void write_weights(const StepArgs &a, const LateWeight &lw, int stride) {
   if (lw.own >= a.M) return;
   __shared__ ff parts[kMaxGroups][kWarps];
@@ -580,7 +588,7 @@ __device__ __forceinline__ void write_weights(const StepArgs &a, const LateWeigh
   const float mean = (q.hi + q.lo) / (float)a.M;
   if (lw.m < a.M) a.w_out[lw.m] = update_from<false>(lw.v, lw.w, mean, 1.f).x;
   for (int m = lw.m + stride * kThreads; m < a.M; m += stride * kThreads)
-    a.w_out[m] = update_from<false>(field_from_sums(a, m), __ldcg(a.w_in + m), mean, 1.f).x;
+    a.w_out[m] = update_from<false>(field_from_sums<MULTI>(a, m), __ldcg(a.w_in + m), mean, 1.f).x;
 }
 
 struct FinalizeArgs {
@@ -832,7 +840,7 @@ __global__ void __launch_bounds__(kThreads * GROUPS, kMaxGroups / GROUPS) gsw_st
     for (int i = vb * kThreads + gthread(); i < 2 * a.M * a.copies; i += vg * kThreads) a.acc_clear[i] = 0ull;
   LateWeight lw;
   const bool gsw = BACK && !ADJ && !a.G;
-  if (gsw) gsw_prologue(a, mc, sm.C0, vb, vg, lw, a.trace);
+  if (gsw) gsw_prologue<false>(a, mc, sm.C0, vb, vg, lw, a.trace);
   for (int t = t_begin; t < t_end; t++)
     process_subtile<FAST, BACK, FWD, ADJ>(a, a.sub[t], 1.f, prestaged, sm, gsw ? sm.C0 : nullptr);
   if (gsw) write_weights(a, lw, vg);
@@ -1103,7 +1111,7 @@ __global__ void __launch_bounds__(kThreads, 4) gsw_persistent_kernel(const __gri
     const float mean = 1.f;  // coefficients without the common factor <|V|> (see gsw_prologue)
     LateWeight lw;
     const StepSmem sm(smem_raw);
-    if (k > 0) gsw_prologue(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, p.trace ? p.trace + 2 * (k - 1) : nullptr);
+    if (k > 0) gsw_prologue<false>(a, mc, sm.C0, blockIdx.x, gridDim.x, lw, p.trace ? p.trace + 2 * (k - 1) : nullptr);
     for (int t = t_begin; t < t_end; t++) {
       bool prestaged = resident && k > 0;
       if (k == 0)

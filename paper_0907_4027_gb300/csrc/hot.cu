@@ -12,6 +12,7 @@
 
 #include "../../include/hot.h"
 #include "gsw_kernels.cuh"
+#include "batch_kernels.cuh"
 #include "tc.h"
 #include "tile.h"
 
@@ -97,6 +98,7 @@ struct hot_ctx {
   float *Y4t = nullptr, *Y4r = nullptr;  // [4][M][ldy4] shifted row tables (hot::StepArgs::Y4)
   int ldy4 = 0;
   float2 *Xc = nullptr, *Yc = nullptr;                               // complex tables (tensor mode)
+  float2 *Xb = nullptr, *Yb = nullptr;  // [M][W], [2][M][ldy4]: complex tables (separable batches)
   float2 *Xq = nullptr;   // the tile kernels' tables (hot::TileArgs)
   float4 *Yq = nullptr;
   int Mp = 0, ldp = 0;
@@ -210,6 +212,8 @@ void free_traps(hot_ctx *c) {
   dfree(c->Y4r);
   dfree(c->Xc);
   dfree(c->Yc);
+  dfree(c->Xb);
+  dfree(c->Yb);
   dfree(c->Xq);
   dfree(c->Yq);
   dfree(c->acc);
@@ -626,6 +630,12 @@ int launch_build_tables(hot_ctx *c) {
                                                         c->Xr, c->Yr, c->Y4t, c->Y4r, c->ldy4);
     rc = check_launch(c, "build_tables_kernel");
   }
+  if (rc == HOT_OK && c->Yb) {
+    const long long total = (long long)c->M * (c->W + c->H);
+    const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
+    hot::batch_tables_kernel<<<blocks, 256, 0, c->st>>>(c->W, c->H, c->M, c->abc, c->Xb, c->Yb, c->ldy4);
+    rc = check_launch(c, "batch_tables_kernel");
+  }
   if (rc == HOT_OK && c->tc) {  // the tensor-core operands derive from the tables
     cudaError_t e = hot_tc::plan_refresh(c->tc, c->st);
     if (e != cudaSuccess) rc = fail(HOT_ECUDA, "rebuilding the tensor-core operands: %s", cudaGetErrorString(e));
@@ -634,36 +644,62 @@ int launch_build_tables(hot_ctx *c) {
   return rc;
 }
 
+// Row stride of the shifted row tables: rows y0 .. y0 + 15 of copy (4 - y0 % 4) % 4 (of copy y0 % 2 of
+// Yb) start 16-byte aligned.
+int shifted_rows(const hot_ctx *c) { return (c->H + 18 + 3) & ~3; }
+
+// Allocates the direct kernels' tables for M traps, once.  *added: set when there are new ones (to be built).
+int alloc_direct_tables(hot_ctx *c, int M, bool *added) {
+  if (c->Y4r) return HOT_OK;
+  c->ldy4 = shifted_rows(c);
+  const size_t n4 = 4 * (size_t)M * c->ldy4;
+  int rc = dalloc(&c->Xt, (size_t)M * c->W);
+  if (rc == HOT_OK) rc = dalloc(&c->Xr, (size_t)M * c->W);
+  if (rc == HOT_OK) rc = dalloc(&c->Yt, (size_t)M * c->H);
+  if (rc == HOT_OK) rc = dalloc(&c->Yr, (size_t)M * c->H);
+  if (rc == HOT_OK) rc = dalloc(&c->Y4t, n4);
+  if (rc == HOT_OK) rc = dalloc(&c->Y4r, n4);
+  if (rc == HOT_OK && (cudaMemsetAsync(c->Y4t, 0, sizeof(float) * n4, c->st) != cudaSuccess ||
+                       cudaMemsetAsync(c->Y4r, 0, sizeof(float) * n4, c->st) != cudaSuccess))
+    rc = fail(HOT_ECUDA, "clearing the shifted row tables failed");
+  if (rc != HOT_OK) {
+    dfree(c->Xt);
+    dfree(c->Xr);
+    dfree(c->Yt);
+    dfree(c->Yr);
+    dfree(c->Y4t);
+    dfree(c->Y4r);
+    return rc;
+  }
+  *added = true;
+  return HOT_OK;
+}
+
+// The same for the complex tables of a separable batch's member.
+int alloc_batch_tables(hot_ctx *c, bool *added) {
+  if (c->Yb) return HOT_OK;
+  c->ldy4 = shifted_rows(c);
+  const size_t n2 = 2 * (size_t)c->M * c->ldy4;
+  int rc = dalloc(&c->Xb, (size_t)c->M * c->W);
+  if (rc == HOT_OK) rc = dalloc(&c->Yb, n2);
+  if (rc == HOT_OK && cudaMemsetAsync(c->Yb, 0, sizeof(float2) * n2, c->st) != cudaSuccess)
+    rc = fail(HOT_ECUDA, "clearing the shifted complex row table failed");
+  if (rc != HOT_OK) {
+    dfree(c->Xb);
+    dfree(c->Yb);
+    return rc;
+  }
+  *added = true;
+  return HOT_OK;
+}
+
 // Allocates the tables that only the direct kernels or only the tensor mode read, once the context
 // is in such a mode.  *added: whether there are new ones (to be built).
 int alloc_mode_tables(hot_ctx *c, int M, bool *added) {
   int rc = HOT_OK;
   *added = false;
-  if (!tile_kernels(c) && !c->Y4r) {
-    rc = dalloc(&c->Xt, (size_t)M * c->W);
-    if (rc == HOT_OK) rc = dalloc(&c->Xr, (size_t)M * c->W);
-    if (rc == HOT_OK) rc = dalloc(&c->Yt, (size_t)M * c->H);
-    if (rc == HOT_OK) rc = dalloc(&c->Yr, (size_t)M * c->H);
-    // shifted row tables: rows y0 .. y0 + 15 of copy (4 - y0 % 4) % 4 start 16-byte aligned
-    c->ldy4 = (c->H + 18 + 3) & ~3;
-    const size_t n4 = 4 * (size_t)M * c->ldy4;
-    if (rc == HOT_OK) rc = dalloc(&c->Y4t, n4);
-    if (rc == HOT_OK) rc = dalloc(&c->Y4r, n4);
-    if (rc == HOT_OK && (cudaMemsetAsync(c->Y4t, 0, sizeof(float) * n4, c->st) != cudaSuccess ||
-                         cudaMemsetAsync(c->Y4r, 0, sizeof(float) * n4, c->st) != cudaSuccess))
-      rc = fail(HOT_ECUDA, "clearing the shifted row tables failed");
-    if (rc != HOT_OK) {
-      dfree(c->Xt);
-      dfree(c->Xr);
-      dfree(c->Yt);
-      dfree(c->Yr);
-      dfree(c->Y4t);
-      dfree(c->Y4r);
-      return rc;
-    }
-    *added = true;
-  }
-  if (c->precision == HOT_PREC_TENSOR && !c->Yc) {
+  if (!tile_kernels(c)) rc = alloc_direct_tables(c, M, added);
+  if (rc == HOT_OK && c->precision == HOT_PREC_TENSOR && !c->Yc) {
     rc = dalloc(&c->Xc, (size_t)M * c->W);
     if (rc == HOT_OK) rc = dalloc(&c->Yc, (size_t)M * c->H);
     if (rc != HOT_OK) {
@@ -672,7 +708,7 @@ int alloc_mode_tables(hot_ctx *c, int M, bool *added) {
     }
     *added = true;
   }
-  return HOT_OK;
+  return rc;
 }
 
 // After a change of the mode: its schedule (resched) and its tables.
@@ -1464,9 +1500,9 @@ struct hot_batch {
     hot::SubTile *sub = nullptr;
     int *first = nullptr;
     std::vector<int> owner;                  // block that writes each hologram's weights
-    std::vector<hot::TileArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
-    int M = 1, pairs = 3;                    // shared-memory layout (hot::TileBatchArgs)
-    bool alone = false;                      // one hologram, on tiles and teams of its own
+    std::vector<hot::StepArgs> holo[6];      // parameters for launch k (k % 6; k = 0 uses set 0)
+    bool alone = false;                      // one hologram on hot_gsw's own step ...
+    hot::TileArgs own[6];                    // ... whose parameters these are
     hot::FinalizeArgs *fin[6] = {};          // finalize descriptors for iters % 6
   };
   std::vector<Group> groups;
@@ -1488,13 +1524,44 @@ struct hot_batch {
 
 namespace {
 
-// Resident blocks per SM of the batch's kernel, with shared memory for its largest trap count.
+int batch_mode(const hot_batch *b) {
+  return b->precision == HOT_PREC_SEPARABLE ? hot::kModeSeparable
+                                            : b->precision == HOT_PREC_FAST ? hot::kModeFast : hot::kModeAccurate;
+}
+
+// Dynamic shared memory of the batch kernels: the separable one stages `chunk` complex traps.
+int batch_smem(const hot_batch *b) {
+  return b->precision == HOT_PREC_SEPARABLE ? hot::sep_smem_bytes(b->chunk) : hot::step_smem_bytes(0, true);
+}
+
+template <int MODE>
+int batch_set_smem() {
+  const int bytes = MODE == hot::kModeSeparable ? hot::sep_smem_bytes(hot::kChunk) : hot::step_smem_bytes(0, true);
+  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_batch_kernel<MODE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  HOT_CUDA(cudaFuncSetAttribute(hot::gsw_batch_kernel<MODE, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  return HOT_OK;
+}
+
+// Resident blocks per SM of the batch's fused kernel at its current staging chunk.
 int batch_occupancy(hot_batch *b) {
-  int M = 1;
-  for (const hot_ctx *c : b->ctx) M = std::max(M, c->M);
-  cudaError_t e = hot_tile::occupancy(M, hot::kWarps, hot::kTilePairs, &b->per_sm_max);
+  int per_sm = 0;
+  const int smem = batch_smem(b);
+  cudaError_t e;
+  switch (batch_mode(b)) {
+    case hot::kModeSeparable:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeSeparable, true>,
+                                                        hot::kThreads, smem);
+      break;
+    case hot::kModeFast:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeFast, true>,
+                                                        hot::kThreads, smem);
+      break;
+    default:
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hot::gsw_batch_kernel<hot::kModeAccurate, true>,
+                                                        hot::kThreads, smem);
+  }
   if (e != cudaSuccess) return fail(HOT_ECUDA, "batch occupancy query: %s", cudaGetErrorString(e));
-  if (b->per_sm_max < 1) b->per_sm_max = 1;
+  b->per_sm_max = per_sm < 1 ? 1 : per_sm;
   return HOT_OK;
 }
 
@@ -1522,17 +1589,48 @@ void batch_free(hot_batch *b) {
   b->chain_ev.clear();
 }
 
+// Copies of the accumulators of a batch's member: as acc_copies, but the batched kernel of the accurate
+// and fast modes keeps one.
+int batch_copies(const hot_batch *b, const hot_ctx *c) { return b->precision == HOT_PREC_SEPARABLE && c->M <= 512 ? 8 : 1; }
+
+// Batched-kernel parameters of context c for launch k of a sequence (buffers rotate as in hot_gsw).
+hot::StepArgs batch_args(const hot_batch *b, const hot_ctx *c, int k) {
+  hot::StepArgs a = {};
+  const bool fast = b->precision == HOT_PREC_FAST;
+  const size_t M2 = 2 * (size_t)c->M * batch_copies(b, c);
+  a.W = c->W;
+  a.H = c->H;
+  a.M = c->M;
+  a.chunk = b->chunk;
+  a.copies = batch_copies(b, c);
+  a.X = fast ? c->Xr : c->Xt;
+  a.Y = fast ? c->Yr : c->Yt;
+  a.Y4 = fast ? c->Y4r : c->Y4t;
+  a.ldy4 = c->ldy4;
+  a.Xc = c->Xb;
+  a.Yc = c->Yb;
+  a.phi = c->phi;
+  a.acc_in = c->acc + M2 * ((k + 2) % 3);
+  a.acc_out = c->acc + M2 * (k % 3);
+  a.acc_clear = c->acc + M2 * ((k + 1) % 3);
+  a.w_in = c->w + (size_t)c->M * ((k + 1) & 1);
+  a.w_out = c->w + (size_t)c->M * (k & 1);
+  a.fx_scale = ldexpf(1.0f, c->fx_shift);
+  a.inv_fx_n = (float)(1.0 / (n_total(c) * ldexp(1.0, c->fx_shift)));
+  a.angle_units = fast ? 1.0f : 0.15915494309189535f;
+  a.angle_eta = fast ? hot::kFastEta : 0.0f;
+  a.inv_n = (float)(1.0 / (n_total(c)));
+  return a;
+}
+
 double pairs_of(const hot_ctx *c) { return n_total(c) * (double)c->M; }
 
-// One group's work schedule: the strips' row pairs of its holograms in order, each weighted by its
-// trap count, dealt out to one wave of G blocks in equal shares (a row pair goes to the block
-// that holds the midpoint of its weight interval); each block's run of pairs in a strip is cut
-// into equal tiles of <= rows / 2 pairs (the default 14: hot::kTilePairs).
-// A group of one hologram, as those of 2^26 pairs and more are, runs hot_gsw's step on its own cut
-// unless a tiling was asked for: the batched kernel's blocks are one team of 8 warps (a tile's traps
-// split eight ways whatever their number), which large holograms with smaller teams outrun
-// (8 holograms up to 1920 x 1152 with up to 2000 traps, 5 iterations: 16.55 -> 14.75 ms; 64 of them 965 ->
-// 853 ms, one by one 851).
+// One group's work schedule: the row segments of its holograms in order, each weighted by its
+// trap count, dealt out to one wave of G blocks in equal shares (a segment goes to the block
+// that holds the midpoint of its weight interval); each block's run of rows in a strip is cut
+// into equal sub-tiles of <= rows rows.
+// A group of one hologram runs hot_gsw's own step on its own cut where one group per hologram was
+// asked for (group_pairs <= 1) with the default tiling, and hot_gsw runs the tile kernels.
 int build_group(hot_batch *b, hot_batch::Group &g) {
   const int count = (int)g.members.size();
   const int per_sm = b->bps > 0 ? std::min(b->bps, b->per_sm_max) : b->per_sm_max;
@@ -1540,13 +1638,12 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   long long segments = 0;
   for (int h : g.members) {
     const hot_ctx *c = b->ctx[h];
-    const long long seg = (long long)((c->W + hot::kTileCols - 1) / hot::kTileCols) * ((c->H + 1) / 2);
+    const long long seg = (long long)((c->W + hot::kTileW - 1) / hot::kTileW) * c->H;
     segments += seg;
     T += (long double)seg * c->M;
-    g.M = std::max(g.M, c->M);
   }
-  const int pairs = b->rows >= hot::kRowsMax ? hot::kTilePairs : (b->rows + 1) / 2;
-  g.alone = count == 1 && pairs == hot::kTilePairs && per_sm == b->per_sm_max;
+  g.alone = count == 1 && b->group_pairs <= 1.0 && b->rows == hot::kRowsMax && per_sm == b->per_sm_max &&
+            b->chunk == hot::kChunk && tile_kernels(b->ctx[g.members[0]]);
   TileCut cut;
   if (g.alone) {
     const hot_ctx *c = b->ctx[g.members[0]];
@@ -1560,7 +1657,7 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   int cur_b = 0;
   for (int i = 0; i < count; i++) {
     const hot_ctx *c = b->ctx[g.members[i]];
-    const int strips = (c->W + hot::kTileCols - 1) / hot::kTileCols, P = (c->H + 1) / 2;
+    const int strips = (c->W + hot::kTileW - 1) / hot::kTileW;
     for (int s = 0; s < strips; s++) {
       auto block_of = [&](int row) {
         const long double mid = w0 + ((long double)row + 0.5L) * c->M;
@@ -1568,21 +1665,20 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
         return bb < 0 ? 0 : (bb >= G ? G - 1 : bb);
       };
       int r = 0;
-      while (r < P) {  // the run of row pairs of this strip that goes to block bb, cut evenly
+      while (r < c->H) {  // the run of rows of this strip that goes to block bb, cut evenly
         const int bb = block_of(r);
         int r1 = r + 1;
-        while (r1 < P && block_of(r1) == bb) r1++;
+        while (r1 < c->H && block_of(r1) == bb) r1++;
         while (cur_b < bb) first[++cur_b] = (int)sub.size();
         if (owner[i] < 0) owner[i] = bb;
-        const int L = r1 - r, nsub = (L + pairs - 1) / pairs;
+        const int L = r1 - r, nsub = (L + b->rows - 1) / b->rows;
         for (int q = 0; q < nsub; q++) {
           const int q0 = r + (int)((long long)L * q / nsub), q1 = r + (int)((long long)L * (q + 1) / nsub);
-          sub.push_back({s * hot::kTileCols, 2 * q0, q1 - q0, i});
-          g.pairs = std::max(g.pairs, q1 - q0);
+          sub.push_back({s * hot::kTileW, q0, q1 - q0, i});
         }
         r = r1;
       }
-      w0 += (long double)P * c->M;
+      w0 += (long double)c->H * c->M;
     }
   }
   while (cur_b < G) first[++cur_b] = (int)sub.size();
@@ -1590,20 +1686,20 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   g.grid = g.alone ? cut.grid : G;
   g.n_sub = (int)sub.size();
   g.owner = owner;
-  int rc = dalloc(&g.sub, sub.size());
-  if (rc == HOT_OK) rc = dalloc(&g.first, first.size());
   for (int k = 0; k < 6; k++) {
     g.holo[k].resize(count);
-    for (int i = 0; i < count; i++) {
-      hot::TileArgs &t = g.holo[k][i];
-      t = make_tile_args(b->ctx[g.members[i]], k == 0 ? 6 : k, nullptr, nullptr, nullptr);
-      t.s.sub = g.sub;
-      t.s.first = g.first;
-      t.s.trace = nullptr;
-      t.team = g.alone ? cut.team : hot::kWarps;
-      t.pairs = g.alone ? cut.pairs : g.pairs;
-      t.stride = cut.stride;
-    }
+    for (int i = 0; i < count; i++) g.holo[k][i] = batch_args(b, b->ctx[g.members[i]], k == 0 ? 6 : k);
+  }
+  int rc = dalloc(&g.sub, sub.size());
+  if (rc == HOT_OK) rc = dalloc(&g.first, first.size());
+  for (int k = 0; g.alone && k < 6; k++) {
+    hot::TileArgs &t = g.own[k];
+    t = make_tile_args(b->ctx[g.members[0]], k == 0 ? 6 : k, nullptr, nullptr, nullptr);
+    t.s.sub = g.sub;
+    t.s.trace = nullptr;
+    t.team = cut.team;
+    t.pairs = cut.pairs;
+    t.stride = cut.stride;
   }
   for (int r6 = 0; rc == HOT_OK && r6 < 6; r6++) {  // finalize after `iters` iterations, iters % 6 == r6
     rc = dalloc(&g.fin[r6], (size_t)count);
@@ -1612,8 +1708,8 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
       const hot_ctx *c = b->ctx[g.members[i]];
       hot::FinalizeArgs &f = fs[i];
       f.M = c->M;
-      f.copies = acc_copies(c);
-      f.acc = c->acc + 2 * (size_t)c->M * acc_copies(c) * (r6 % 3);  // the last launch accumulated into acc[iters % 3]
+      f.copies = g.alone ? acc_copies(c) : batch_copies(b, c);
+      f.acc = c->acc + 2 * (size_t)c->M * f.copies * (r6 % 3);  // the last launch accumulated into acc[iters % 3]
       f.acc_all = c->acc;
       f.w_src = c->w + (size_t)c->M * (r6 & 1);       // and left the weights in w[iters & 1]
       f.w_dst = c->w;
@@ -1633,12 +1729,22 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
   return rc;
 }
 
+// The tables that the batched kernel reads, where the member does not have them yet.
+int batch_tables(const hot_batch *b, hot_ctx *c) {
+  bool added = false;
+  int rc = b->precision == HOT_PREC_SEPARABLE ? alloc_batch_tables(c, &added) : alloc_direct_tables(c, c->M, &added);
+  if (rc == HOT_OK && added) rc = launch_build_tables(c);
+  if (rc == HOT_OK && added) HOT_CUDA(cudaStreamSynchronize(c->st));
+  return rc;
+}
+
 // Orders the holograms by pairs per iteration (smallest first, stable), cuts them into
 // groups of >= group_pairs (a short last group joins the one before) and builds each group.
 int batch_schedule(hot_batch *b) {
   HOT_CUDA(cudaStreamSynchronize(b->st));
   batch_drop_graphs(b);
-  const int rc0 = batch_occupancy(b);
+  int rc0 = batch_occupancy(b);
+  for (size_t h = 0; h < b->ctx.size() && rc0 == HOT_OK; h++) rc0 = batch_tables(b, b->ctx[h]);
   if (rc0 != HOT_OK) return rc0;
   for (auto &g : b->groups) group_free(g);
   b->groups.clear();
@@ -1674,18 +1780,28 @@ int batch_schedule(hot_batch *b) {
   return HOT_OK;
 }
 
-template <bool BACK>
+template <int MODE, bool BACK>
 int batch_launch(hot_batch *b, const hot_batch::Group &g, int k) {
-  hot::TileBatchArgs a = {};
+  hot::BatchArgs a = {};
   const int count = (int)g.members.size();
-  for (int i = 0; i < count && !g.alone; i++) {
+  for (int i = 0; i < count; i++) {
     a.holo[i] = g.holo[k % 6][i];
     a.owner[i] = g.owner[i];
   }
+  a.sub = g.sub;
   a.first = g.first;
   a.count = count;
-  a.M = g.M;
-  a.pairs = g.pairs;
+  hot_ctx tmp;  // launch() needs a context only for the stream
+  tmp.st = b->st;
+  launch(&tmp, hot::gsw_batch_kernel<MODE, BACK>, g.grid, hot::kThreads, batch_smem(b), true, a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_batch_kernel: %s", cudaGetErrorString(e));
+  return HOT_OK;
+}
+
+// Launch k of a group of one hologram on hot_gsw's own step.
+template <bool BACK>
+int batch_launch_own(hot_batch *b, const hot_batch::Group &g, int k) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(g.grid);
   cfg.blockDim = dim3(hot::kThreads);
@@ -1695,13 +1811,21 @@ int batch_launch(hot_batch *b, const hot_batch::Group &g, int k) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (g.alone)
-    hot_tile::launch(BACK, true, false, cfg, g.holo[k % 6][0]);
-  else
-    hot_tile::launch_batch(BACK, cfg, a);
+  hot_tile::launch(BACK, true, false, cfg, g.own[k % 6]);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_tile_batch_kernel: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return fail(HOT_ECUDA, "launch of gsw_tile_kernel: %s", cudaGetErrorString(e));
   return HOT_OK;
+}
+
+// Launch k of a group: BACK an iteration, otherwise the forward field of the starting phases (k = 0).
+template <bool BACK>
+int batch_launch_mode(hot_batch *b, const hot_batch::Group &g, int k) {
+  if (g.alone) return batch_launch_own<BACK>(b, g, k);
+  switch (batch_mode(b)) {
+    case hot::kModeSeparable: return batch_launch<hot::kModeSeparable, BACK>(b, g, k);
+    case hot::kModeFast: return batch_launch<hot::kModeFast, BACK>(b, g, k);
+    default: return batch_launch<hot::kModeAccurate, BACK>(b, g, k);
+  }
 }
 
 constexpr int kTensorChains = 8;
@@ -1758,6 +1882,8 @@ int batch_enqueue_tensor(hot_batch *b, int iters) {
   return HOT_OK;
 }
 
+// A start stamp, then the groups in order: forward field of the starting phases (k = 0),
+// iterations 1..iters, and the per-hologram finalize with its completion stamp.
 int batch_enqueue(hot_batch *b, int iters) {
   if (b->precision == HOT_PREC_TENSOR) return batch_enqueue_tensor(b, iters);
   hot::stamp_kernel<<<1, 1, 0, b->st>>>(b->stamps + b->count);
@@ -1765,8 +1891,8 @@ int batch_enqueue(hot_batch *b, int iters) {
   if (e0 != cudaSuccess) return fail(HOT_ECUDA, "launch of stamp_kernel: %s", cudaGetErrorString(e0));
   for (size_t gi = 0; gi < b->groups.size(); gi++) {
     const hot_batch::Group &g = b->groups[gi];
-    int rc = batch_launch<false>(b, g, 0);
-    for (int k = 1; k <= iters && rc == HOT_OK; k++) rc = batch_launch<true>(b, g, k);
+    int rc = batch_launch_mode<false>(b, g, 0);
+    for (int k = 1; k <= iters && rc == HOT_OK; k++) rc = batch_launch_mode<true>(b, g, k);
     if (rc != HOT_OK) return rc;
     hot_ctx tmp;
     tmp.st = b->st;
@@ -2036,7 +2162,10 @@ int hot_batch_create(hot_batch **out, int count, hot_ctx *const *ctxs, void *cud
   b->precision = ctxs[0]->precision;
   b->dev = ctxs[0]->dev;
   const bool tensor = b->precision == HOT_PREC_TENSOR;
-  int rc = HOT_OK;
+  int rc = tensor                                 ? HOT_OK
+           : batch_mode(b) == hot::kModeSeparable ? batch_set_smem<hot::kModeSeparable>()
+           : batch_mode(b) == hot::kModeFast      ? batch_set_smem<hot::kModeFast>()
+                                                  : batch_set_smem<hot::kModeAccurate>();
   if (rc == HOT_OK && cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->dev) != cudaSuccess)
     rc = fail(HOT_ECUDA, "hot_batch_create: device query failed");
   if (rc == HOT_OK) rc = dalloc(&b->stamps, (size_t)count + 1);

@@ -24,15 +24,13 @@ cudaError_t set_smem() {
   raise(hot::gsw_tile_kernel<true, false, false>);
   raise(hot::gsw_tile_kernel<true, false, true>);
   raise(hot::gsw_tile_persistent_kernel);
-  raise(hot::gsw_tile_batch_kernel<true>);
-  raise(hot::gsw_tile_batch_kernel<false>);
   return e;
 }
 
 }  // namespace
 
 cudaError_t occupancy(int M, int team, int pairs, int *per_sm) {
-  int a = 0, b = 0, c = 0;
+  int a = 0, b = 0;
   const int smem = hot::tile_smem_bytes(M, team, pairs);
   *per_sm = 0;
   cudaError_t e = set_smem();
@@ -40,9 +38,7 @@ cudaError_t occupancy(int M, int team, int pairs, int *per_sm) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, hot::gsw_tile_kernel<true, true, false>, hot::kThreads, smem);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, hot::gsw_tile_persistent_kernel, hot::kThreads, smem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c, hot::gsw_tile_batch_kernel<true>, hot::kThreads, smem);
-  *per_sm = std::min(std::min(a, b), c);
+  *per_sm = std::min(a, b);
   return e;
 }
 
@@ -57,12 +53,6 @@ cudaError_t launch(bool back, bool fwd, bool adj, cudaLaunchConfig_t cfg, const 
 cudaError_t launch_persistent(cudaLaunchConfig_t cfg, const hot::TilePersistArgs &p) {
   cfg.dynamicSmemBytes = hot::tile_smem_bytes(p.step[0].s.M, p.step[0].team, p.step[0].pairs);
   return cudaLaunchKernelEx(&cfg, hot::gsw_tile_persistent_kernel, p);
-}
-
-cudaError_t launch_batch(bool back, cudaLaunchConfig_t cfg, const hot::TileBatchArgs &b) {
-  cfg.dynamicSmemBytes = hot::tile_smem_bytes(b.M, hot::kWarps, b.pairs);
-  return back ? cudaLaunchKernelEx(&cfg, hot::gsw_tile_batch_kernel<true>, b)
-              : cudaLaunchKernelEx(&cfg, hot::gsw_tile_batch_kernel<false>, b);
 }
 
 }  // namespace hot_tile

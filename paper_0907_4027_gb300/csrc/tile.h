@@ -7,7 +7,7 @@
 
 namespace hot_tile {
 
-// Blocks per SM that the step, the batched and the persistent kernel both keep resident (0: a block does not fit).
+// Blocks per SM that the step and the persistent kernel both keep resident (0: a block does not fit).
 cudaError_t occupancy(int M, int team, int pairs, int *per_sm);
 
 // One launch with the grid, block, stream and attributes of cfg (its dynamic shared memory is set
@@ -15,7 +15,5 @@ cudaError_t occupancy(int M, int team, int pairs, int *per_sm);
 // adjoint (back, adj); and the persistent form.
 cudaError_t launch(bool back, bool fwd, bool adj, cudaLaunchConfig_t cfg, const hot::TileArgs &a);
 cudaError_t launch_persistent(cudaLaunchConfig_t cfg, const hot::TilePersistArgs &p);
-// One launch of a batch's group (teams of 8 warps).
-cudaError_t launch_batch(bool back, cudaLaunchConfig_t cfg, const hot::TileBatchArgs &b);
 
 }  // namespace hot_tile

@@ -552,57 +552,6 @@ static __global__ void __launch_bounds__(kThreads, 2) gsw_tile_persistent_kernel
   }
 }
 
-// Batched launch: the tiles of up to kBatchMax holograms (SubTile::pad = hologram index) in one
-// grid, a block (one team of 8 warps) walking its run hologram by hologram: every block that meets
-// a hologram computes its coefficients itself; the weights of hologram h are written by block
-// owner[h].  The holograms' parameters travel in the launch itself.
-constexpr int kBatchMax = 22;
-
-struct TileBatchArgs {
-  TileArgs holo[kBatchMax];  // s.sub: the launch's tiles
-  int owner[kBatchMax];
-  const int *first;          // [gridDim.x + 1]
-  int count;
-  int M, pairs;              // largest trap count and row pairs (shared memory is laid out for them)
-};
-static_assert(sizeof(TileBatchArgs) <= 16384, "launch argument");
-
-template <bool BACK>
-__global__ void __launch_bounds__(kThreads, 2) gsw_tile_batch_kernel(const __grid_constant__ TileBatchArgs b) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const TileSmem sm(smem_raw, b.M, kWarps, b.pairs);
-  const SubTile *const sub = b.holo[0].s.sub;
-  const int t_end = b.first[blockIdx.x + 1];
-  int t = b.first[blockIdx.x];
-  allow_dependents();
-  bool waited = false;
-  do {
-    const int h = t < t_end ? sub[t].pad : 0;
-    int t1 = t;
-    while (t1 < t_end && sub[t1].pad == h) t1++;
-    const StepArgs &a = b.holo[h].s;
-    TileStream in(b.holo[h], sm, BACK ? 2 : 1, t, t1);
-    if (!waited) {
-      grid_dependency_wait();
-      for (int i = 0; i < b.count; i++) {  // the buffers the next launch accumulates into
-        unsigned long long *clr = b.holo[i].s.acc_clear;
-        const int n2 = 2 * b.holo[i].s.M * b.holo[i].s.copies;
-        for (int j = blockIdx.x * kThreads + threadIdx.x; j < n2; j += gridDim.x * kThreads) clr[j] = 0ull;
-      }
-      waited = true;
-    }
-    if (t == t1) break;
-    if (BACK) {
-      __syncthreads();  // the readers of the previous hologram's coefficients are done
-      tile_prologue(a, sm, b.owner[h] == (int)blockIdx.x ? 0 : a.M, 1, nullptr);
-      __syncthreads();
-    }
-    tile_run<BACK, true, false>(a, sm, in, t, t1, 0);
-    if (BACK && b.owner[h] == (int)blockIdx.x) tile_weights(a, sm, 0, 1);
-    t = t1;
-  } while (t < t_end);
-}
-
 // ---------------------------------------------------------------------------------------------
 // Tables of the column and row phasors (once per trap set).
 //
