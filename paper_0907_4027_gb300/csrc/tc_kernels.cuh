@@ -39,8 +39,8 @@
 //            the K range may be split over CTAs);
 //   plain:   C = A B^T (the GEMM alone, for tests).
 // Every wait on an mbarrier is bounded by %globaltimer; when one runs out the CTA sets the error
-// flag, stops issuing, waits (bounded) for the copies it has in flight, frees its tensor memory
-// and returns.
+// flag, stops issuing, waits (bounded by kDrainNs at least, whatever the caller's limit) for the copies
+// and the MMAs it has in flight, frees its tensor memory and returns.
 #pragma once
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -52,6 +52,7 @@ namespace tc {
 constexpr int kBM = 128;         // rows of a tile: the 128 lanes of tensor memory
 constexpr int kSliceBytes = 128; // one K slice per stage: one 128-byte swizzle row of every operand row
 constexpr int kMmaKBytes = 32;   // K of one MMA: 8 TF32 or 16 FP16 elements
+constexpr long long kDrainNs = 1000000000;  // what a CTA that gives up grants its copies and MMAs at least
 
 // Operand types.  TF32: FP32 storage, kind::tf32 (the MMA reads the top 19 bits).  FP16: halves,
 // kind::f16 at twice the TF32 rate; its 11-bit significand equals TF32's, so the split keeps the
@@ -651,9 +652,18 @@ __global__ void __launch_bounds__(Cfg<BN>::kThreads, 1) tc_gemm_kernel(const __g
   __syncthreads();
   if (threadIdx.x == 0 && failed) {
     atomicExch(a.err, 1);
-    // copies still in flight: wait (bounded) until they have landed before the CTA exits
-    for (int j = consumed_a; j < issued_a; j++) mbar_wait(&full_a[j % SA], (uint32_t)(j / SA) & 1u, a.limit_ns);
-    for (int i = consumed_b; i < issued_b; i++) mbar_wait(&full_b[i % SB], (uint32_t)(i / SB) & 1u, a.limit_ns);
+    // Copies that no MMA waited for, and the MMAs issued (steps 0 .. consumed_a - 1), may still be at work
+    // in this CTA's shared and tensor memory: wait (bounded) for the copies and for the last commits, which
+    // complete after the MMAs before them, and so for their arrivals too, before the CTA exits.
+    const long long limit = a.limit_ns > kDrainNs ? a.limit_ns : kDrainNs;
+    for (int j = consumed_a; j < issued_a; j++) mbar_wait(&full_a[j % SA], (uint32_t)(j / SA) & 1u, limit);
+    for (int i = consumed_b; i < issued_b; i++) mbar_wait(&full_b[i % SB], (uint32_t)(i / SB) & 1u, limit);
+    if (consumed_a > 0) {
+      const int j = consumed_a - 1, i = consumed_a / NA - 1;  // the last steps that committed each barrier
+      mbar_wait(&empty_a[j % SA], (uint32_t)(j / SA) & 1u, limit);
+      if (i >= 0) mbar_wait(&empty_b[i % SB], (uint32_t)(i / SB) & 1u, limit);
+      mbar_wait(&tfull[j % C::kBufs], (uint32_t)(j / C::kBufs) & 1u, limit);
+    }
   }
   tc_fence_before();
   __syncthreads();
