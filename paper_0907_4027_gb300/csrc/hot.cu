@@ -105,7 +105,7 @@ struct hot_ctx {
   float *w = nullptr;                                          // [2][M] weights (home: w[0])
   unsigned long long *acc = nullptr;                           // [3][copies][2][M] fixed-point field sums
   long long *Vsum = nullptr;                                   // [2][M] sums of the last forward
-  float *metrics = nullptr;                                    // [2]
+  float *metrics = nullptr;                                    // [2], and the words of sync behind them
   int fx_shift = 0;                                            // fixed-point scale 2^fx_shift
   unsigned char *u8 = nullptr;                                 // [N] staging for host output
   bool have_fields = false;
@@ -134,7 +134,7 @@ struct hot_ctx {
   float *trace = nullptr;  // [trace_cap][2]
   int trace_cap = 0, trace_iters = -1;
   double wait_limit_s = 2.0;
-  unsigned int *sync = nullptr;
+  unsigned int *sync = nullptr;  // (behind metrics: one copy reads both)
   std::vector<Graph> graphs;
   // HOT_PREC_TENSOR: operands and launch shapes of the tensor-core iteration (built on first use)
   hot_tc::Plan *tc = nullptr;
@@ -144,8 +144,9 @@ struct hot_ctx {
   // the stream's work and a round trip, as a synchronisation before the buffer's release does.
   unsigned char *pin = nullptr;
   cudaEvent_t ev_in = nullptr;
-  bool waits = false;  // a launch with bounded waits was queued since the last look at their error flag
 };
+
+constexpr size_t kStatusBytes = 20;  // two metrics, three words of sync
 
 // Layout of hot_ctx::io and of the pinned staging for M traps, in bytes.
 struct IoBytes {
@@ -819,7 +820,6 @@ int check_wait_error(hot_ctx *c, const char *who) {
   unsigned int st[3] = {0, 0, 0};  // [2]: error flag of the bounded waits
   HOT_CUDA(cudaMemcpyAsync(st, c->sync, sizeof st, cudaMemcpyDeviceToHost, c->st));
   HOT_CUDA(cudaStreamSynchronize(c->st));
-  c->waits = false;
   return st[2] ? wait_ran_out(c, who) : HOT_OK;
 }
 
@@ -834,21 +834,17 @@ const float *read_metrics(const hot_ctx *c) {
   return reinterpret_cast<const float *>(c->pin + b.back + b.read());
 }
 
-// Brings weights and field sums (fields) and the metrics (metrics) to the pinned staging with one
-// synchronisation, which also looks at the error flag if a launch with bounded waits was queued.
-int read_back(hot_ctx *c, const char *who, bool fields, bool metrics) {
+// Brings the metrics with the barrier's words behind them, and weights and field sums (fields), to the
+// pinned staging with one synchronisation; HOT_ETIMEOUT after a bounded wait ran out.  The error flag is
+// always looked at: which launches with bounded waits ran since the last look is not known here (replays
+// of a captured call, batches on a stream of their own).
+int read_back(hot_ctx *c, const char *who, bool fields) {
   const IoBytes b(c->M);
   unsigned char *const back = c->pin + b.back;
-  unsigned int *const flag = reinterpret_cast<unsigned int *>(back + b.read() + 8);
   if (fields) HOT_CUDA(cudaMemcpyAsync(back, c->io + b.w, b.read(), cudaMemcpyDeviceToHost, c->st));
-  if (metrics) HOT_CUDA(cudaMemcpyAsync(back + b.read(), c->metrics, 2 * sizeof(float), cudaMemcpyDeviceToHost, c->st));
-  if (c->waits) HOT_CUDA(cudaMemcpyAsync(flag, c->sync, 3 * sizeof(unsigned int), cudaMemcpyDeviceToHost, c->st));
+  HOT_CUDA(cudaMemcpyAsync(back + b.read(), c->metrics, kStatusBytes, cudaMemcpyDeviceToHost, c->st));
   HOT_CUDA(cudaStreamSynchronize(c->st));
-  if (c->waits) {
-    c->waits = false;
-    if (flag[2]) return wait_ran_out(c, who);
-  }
-  return HOT_OK;
+  return reinterpret_cast<const unsigned int *>(back + b.read())[4] ? wait_ran_out(c, who) : HOT_OK;
 }
 
 // Waits until the last copy out of the pinned staging is done, so that it can be filled again.  A
@@ -864,7 +860,7 @@ int staging_free(hot_ctx *c, const char *who) {
 // e and u to the caller's non-NULL outputs (synchronises); nothing when both are NULL.
 int return_metrics(hot_ctx *c, const char *who, double *eff_out, double *unif_out) {
   if (!eff_out && !unif_out) return HOT_OK;
-  const int rc = read_back(c, who, false, true);
+  const int rc = read_back(c, who, false);
   if (rc != HOT_OK) return rc;
   if (eff_out) *eff_out = read_metrics(c)[0];
   if (unif_out) *unif_out = read_metrics(c)[1];
@@ -966,8 +962,8 @@ int hot_create(hot_ctx **out, int width, int height, double pitch_m, double wave
   if (e != cudaSuccess) rc = fail(HOT_ECUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
   const size_t N = (size_t)width * height;
   if (rc == HOT_OK) rc = dalloc(&c->phi, N);
-  if (rc == HOT_OK) rc = dalloc(&c->metrics, 2);
-  if (rc == HOT_OK) rc = dalloc(&c->sync, 3);
+  if (rc == HOT_OK) rc = dalloc(&c->metrics, kStatusBytes / sizeof(float));
+  if (rc == HOT_OK) c->sync = reinterpret_cast<unsigned int *>(c->metrics + 2);
   if (rc == HOT_OK && cudaMemsetAsync(c->sync, 0, 3 * sizeof(unsigned int), c->st) != cudaSuccess)
     rc = fail(HOT_ECUDA, "hot_create: clearing the barrier state failed");
   if (rc == HOT_OK) {
@@ -998,7 +994,6 @@ void hot_destroy(hot_ctx *c) {
   dfree(c->ubuf);
   dfree(c->metrics);
   dfree(c->u8);
-  dfree(c->sync);
   dfree(c->trace);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   delete c;
@@ -1150,7 +1145,6 @@ int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
   // where the state keeps unit phasors, the last step left u_j of the phases it wrote in ubuf
   c->u_valid = iters > 0 ? c->once : had_u;
   c->have_fields = true;
-  if (c->persistent || c->precision == HOT_PREC_TENSOR) c->waits = true;
   return return_metrics(c, "hot_gsw", eff_out, unif_out);
 }
 
@@ -1188,7 +1182,7 @@ int hot_get_fields(hot_ctx *c, double *V, double *w) {
   if (!c) return fail(HOT_EINVAL, "hot_get_fields: NULL context");
   if (!c->M) return fail(HOT_ESTATE, "hot_get_fields: no traps set");
   if (V && !c->have_fields) return fail(HOT_ESTATE, "hot_get_fields: no forward evaluation since the last change");
-  const int rc = read_back(c, "hot_get_fields", V || w, false);
+  const int rc = read_back(c, "hot_get_fields", V || w);
   if (rc != HOT_OK) return rc;
   const long long *const vs = read_sums(c);
   const float *const wf = read_w(c);
@@ -1292,7 +1286,6 @@ int hot_sharded_begin(hot_ctx *c) {
   int rc = HOT_OK;
   if (c->precision == HOT_PREC_TENSOR) {
     rc = ensure_tc_plan(c);
-    c->waits = true;
     if (rc == HOT_OK) rc = launch_tc(c, false, 0);
   } else {
     rc = launch_step(c, false, true, false, 0);
@@ -1334,7 +1327,7 @@ int hot_sharded_end(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
 int hot_get_metrics(hot_ctx *c, double *eff_out, double *unif_out) {
   if (!c) return fail(HOT_EINVAL, "hot_get_metrics: NULL context");
   if (!c->M || !c->have_fields) return fail(HOT_ESTATE, "hot_get_metrics: no forward evaluation since the last change");
-  const int rc = read_back(c, "hot_get_metrics", false, true);
+  const int rc = read_back(c, "hot_get_metrics", false);
   if (rc != HOT_OK) return rc;
   if (eff_out) *eff_out = read_metrics(c)[0];
   if (unif_out) *unif_out = read_metrics(c)[1];
@@ -2213,7 +2206,6 @@ int hot_batch_gsw(hot_batch *b, int iters) {
       for (auto *c : b->ctx) {
         c->have_fields = true;
         c->u_valid = false;  // the batch kernels wrote the phases
-        if (b->precision == HOT_PREC_TENSOR) c->waits = true;
       }
       b->ran = true;
       return HOT_OK;
@@ -2244,7 +2236,6 @@ int hot_batch_gsw(hot_batch *b, int iters) {
   for (auto *c : b->ctx) {
     c->have_fields = true;
     c->u_valid = false;  // the batch kernels wrote the phases
-    if (b->precision == HOT_PREC_TENSOR) c->waits = true;
   }
   b->ran = true;
   return HOT_OK;
