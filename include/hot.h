@@ -23,6 +23,8 @@
  *   - Invalid sizes or pointers give HOT_EINVAL before any device work is queued.
  *   - Work is queued on the context's CUDA stream (given at creation; NULL is the legacy
  *     default stream).  Calls that return data to host memory synchronise that stream.
+ *     The others may return before their work is done, hot_set_traps, hot_set_weights and
+ *     hot_superposition among them; hot_batch_gsw orders its own stream behind its members'.
  *   - Host pointers are read or written before the call returns; device pointers
  *     (on_device = 1) must be valid on the context's device and are used in stream order.
  *   - The library owns every device buffer of a context; hot_destroy frees them.

@@ -1483,6 +1483,7 @@ struct hot_batch {
   int count = 0, precision = HOT_PREC_ACCURATE, dev = 0;
   std::vector<hot_ctx *> ctx;
   cudaStream_t st = nullptr, cap = nullptr;
+  cudaEvent_t ev = nullptr;  // the members' streams' work that a run starts after (batch_after_members)
   int sms = 0, per_sm_max = 1;
   // tiling (hot_batch_set_tiling) and group threshold in pixel-trap pairs per iteration
   int rows = hot::kRowsMax, bps = 0, chunk = hot::kChunk;
@@ -1576,6 +1577,8 @@ void batch_free(hot_batch *b) {
   dfree(b->stamps);
   if (b->cap) cudaStreamDestroy(b->cap);
   b->cap = nullptr;
+  if (b->ev) cudaEventDestroy(b->ev);
+  b->ev = nullptr;
   for (cudaStream_t s : b->chain_st) cudaStreamDestroy(s);
   for (cudaEvent_t e : b->chain_ev) cudaEventDestroy(e);
   b->chain_st.clear();
@@ -1897,6 +1900,37 @@ int batch_enqueue(hot_batch *b, int iters) {
   return HOT_OK;
 }
 
+// Orders the batch's stream behind what the members queued on other streams: traps, weights, phases
+// and superpositions are queued (their calls return before the work is done).  A member's stream
+// under capture is left to its owner; a batch's stream under capture can only wait on the host.
+int batch_after_members(hot_batch *b) {
+  std::vector<cudaStream_t> seen = {b->st};
+  cudaStreamCaptureStatus mine = cudaStreamCaptureStatusNone;
+  for (const hot_ctx *c : b->ctx) {
+    if (std::find(seen.begin(), seen.end(), c->st) != seen.end()) continue;
+    if (seen.size() == 1) HOT_CUDA(cudaStreamIsCapturing(b->st, &mine));
+    seen.push_back(c->st);
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaStreamCaptureStatus theirs = cudaStreamCaptureStatusNone;
+    if (mine == cudaStreamCaptureStatusNone) {
+      const cudaError_t e = cudaStreamIsCapturing(c->st, &theirs);
+      if (e == cudaErrorStreamCaptureImplicit) cudaGetLastError();  // the legacy stream, beside another's capture
+      else HOT_CUDA(e);
+      if (e != cudaSuccess || theirs != cudaStreamCaptureStatusNone) continue;
+      if (!b->ev) HOT_CUDA(cudaEventCreateWithFlags(&b->ev, cudaEventDisableTiming));
+      HOT_CUDA(cudaEventRecord(b->ev, c->st));
+      HOT_CUDA(cudaStreamWaitEvent(b->st, b->ev, 0));
+    } else if (c->st) {
+      HOT_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+      cudaError_t e = cudaStreamIsCapturing(c->st, &theirs);
+      if (e == cudaSuccess && theirs == cudaStreamCaptureStatusNone) e = cudaStreamSynchronize(c->st);
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e != cudaSuccess) return fail(HOT_ECUDA, "hot_batch_gsw: waiting for a member's stream: %s", cudaGetErrorString(e));
+    }
+  }
+  return HOT_OK;
+}
+
 int check_tiling(const char *who, int rows, int bps, int chunk) {
   if (rows < 0 || rows > hot::kRowsMax) return fail(HOT_EINVAL, "%s: rows = %d not in [1, %d] (0: default)", who, rows, hot::kRowsMax);
   if (bps < 0 || bps > 32) return fail(HOT_EINVAL, "%s: blocks_per_sm = %d not in [1, 32] (0: default)", who, bps);
@@ -2202,6 +2236,8 @@ int hot_batch_gsw(hot_batch *b, int iters) {
   if (iters < 0) return fail(HOT_EINVAL, "hot_batch_gsw: iters = %d < 0", iters);
   for (auto &g : b->graphs)
     if (g.iters == iters) {
+      const int rc = batch_after_members(b);
+      if (rc != HOT_OK) return rc;
       HOT_CUDA(cudaGraphLaunch(g.exec, b->st));
       for (auto *c : b->ctx) {
         c->have_fields = true;
@@ -2232,6 +2268,8 @@ int hot_batch_gsw(hot_batch *b, int iters) {
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return fail(HOT_ECUDA, "hot_batch_gsw: graph instantiation: %s", cudaGetErrorString(e));
   b->graphs.push_back({iters, exec});
+  rc = batch_after_members(b);
+  if (rc != HOT_OK) return rc;
   HOT_CUDA(cudaGraphLaunch(exec, b->st));
   for (auto *c : b->ctx) {
     c->have_fields = true;
@@ -2246,7 +2284,7 @@ int hot_batch_autotune(hot_batch *b, int iters, int *rows, int *blocks_per_sm, i
   if (b->precision == HOT_PREC_TENSOR) return fail(HOT_EINVAL, "hot_batch_autotune: a HOT_PREC_TENSOR batch has no tiling");
   if (iters < 1) return fail(HOT_EINVAL, "hot_batch_autotune: iters = %d < 1", iters);
   std::vector<Saved> saved(b->count);
-  int rc = HOT_OK;
+  int rc = batch_after_members(b);
   for (int h = 0; rc == HOT_OK && h < b->count; h++) rc = save_state(b->ctx[h], saved[h], b->st);
   if (rc != HOT_OK) return rc;
   auto restore = [&]() {
