@@ -38,10 +38,13 @@ int fail(int code, const char *fmt, ...) {
                   #call, cudaGetErrorString(e_), __FILE__, __LINE__);                   \
   } while (0)
 
+thread_local int g_refuse = 0;  // hot_test_refuse_alloc
+
 template <typename T>
 int dalloc(T **p, size_t count) {
   *p = nullptr;
   if (count == 0) return HOT_OK;
+  if (g_refuse && --g_refuse == 0) return fail(HOT_ENOMEM, "cudaMalloc(%zu B): refused", count * sizeof(T));
   cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), count * sizeof(T));
   if (e != cudaSuccess) {
     *p = nullptr;
@@ -49,6 +52,20 @@ int dalloc(T **p, size_t count) {
                 count * sizeof(T), cudaGetErrorString(e));
   }
   return HOT_OK;
+}
+
+template <typename T>
+void dfree(T *&p);
+
+// A device copy of v; nothing allocated on failure.
+template <typename T>
+int upload(T **p, const std::vector<T> &v) {
+  const int rc = dalloc(p, v.size());
+  if (rc != HOT_OK) return rc;
+  const cudaError_t e = cudaMemcpy(*p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) return HOT_OK;
+  dfree(*p);
+  return fail(HOT_ECUDA, "copying a schedule: %s", cudaGetErrorString(e));
 }
 
 template <typename T>
@@ -102,6 +119,7 @@ struct hot_ctx {
   float2 *Xq = nullptr;   // the tile kernels' tables (hot::TileArgs)
   float4 *Yq = nullptr;
   int Mp = 0, ldp = 0;
+  bool unbuilt = false;  // some of the tables were allocated since launch_build_tables last ran
   float *w = nullptr;                                          // [2][M] weights (home: w[0])
   unsigned long long *acc = nullptr;                           // [3][copies][2][M] fixed-point field sums
   long long *Vsum = nullptr;                                   // [2][M] sums of the last forward
@@ -493,35 +511,11 @@ int cut_tiles(int W, int H, int M, int sms, TileCut &cut) {
   return HOT_OK;
 }
 
-// The tile kernels' schedule of a context.
-int build_tile_schedule(hot_ctx *c, int sms) {
-  c->once = false;
-  c->tgrid = 0;
-  dfree(c->tsub);
-  if (!tile_kernels(c)) return HOT_OK;
-  TileCut cut;
-  const int rc0 = cut_tiles(c->W, c->H, c->M, sms, cut);
-  if (rc0 != HOT_OK) return rc0;
-  const int rc1 = dalloc(&c->tsub, cut.tiles.size());
-  if (rc1 != HOT_OK) return rc1;
-  HOT_CUDA(cudaMemcpy(c->tsub, cut.tiles.data(), sizeof(hot::SubTile) * cut.tiles.size(), cudaMemcpyHostToDevice));
-  c->tstride = cut.stride;
-  c->once = !separable_kernels(c) && c->M <= hot::kOnceMaxM;
-  if (c->once && !c->ubuf) {
-    const int rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
-    if (rc != HOT_OK) return rc;
-  }
-  c->tgrid = cut.grid;
-  c->tteam = cut.team;
-  c->tpairs = cut.pairs;
-  return HOT_OK;
-}
-
 // One wave of persistent blocks (SMs x resident blocks per SM: as many as fit, at most
 // tile_bps); the W/32 x H row segments are dealt out in equal contiguous runs, cut into
-// sub-tiles of <= tile_rows rows.  Also the tile kernels' schedule.
+// sub-tiles of <= tile_rows rows.  Also the tile kernels' schedule.  On failure the schedule stays as
+// it was.
 int build_schedule(hot_ctx *c) {
-  drop_graphs(c);  // graphs hold the old schedule
   int rc = set_step_smem(c->M);
   if (rc != HOT_OK) return rc;
   int sms = 0, per_sm = 0;
@@ -542,12 +536,11 @@ int build_schedule(hot_ctx *c) {
   }
   per_sm = std::min(per_sm, per_sm_p);
   if (per_sm < 1) per_sm = 1;
-  c->sched_bps_max = per_sm;
+  const int bps_max = per_sm;
   if (c->tile_bps > 0 && c->tile_bps < per_sm) per_sm = c->tile_bps;
-  c->sched_bps = per_sm;
   // Merged (hot_set_block_merge), with four schedule blocks per SM the direct modes' GSW step
   // runs one block per SM holding four of them (see gsw_step_kernel), if such a block fits.
-  c->groups = 1;
+  int groups = 1;
   if (c->tile_merge > 1 && !separable_kernels(c) && per_sm == hot::kMaxGroups) {
     int per_sm_g = 0;
     const int smem = c->tile_merge * hot::step_smem_bytes(c->M, true);
@@ -557,7 +550,7 @@ int build_schedule(hot_ctx *c) {
     else
       HOT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_g, hot::gsw_step_kernel<true, true, true, false, 2>,
                                                              hot::kThreads * 2, smem));
-    if (per_sm_g * c->tile_merge >= per_sm) c->groups = c->tile_merge;
+    if (per_sm_g * c->tile_merge >= per_sm) groups = c->tile_merge;
   }
   const int strips = (c->W + hot::kTileW - 1) / hot::kTileW;
   const long long U = (long long)strips * c->H;
@@ -568,19 +561,40 @@ int build_schedule(hot_ctx *c) {
   std::vector<hot::SubTile> sub;
   std::vector<int> first;
   cut_schedule(c->W, c->H, G, c->tile_rows, sub, first);
+  const bool tile = tile_kernels(c), once = tile && !separable_kernels(c) && c->M <= hot::kOnceMaxM;
+  TileCut cut;
+  if (tile) rc = cut_tiles(c->W, c->H, c->M, sms, cut);
   HOT_CUDA(cudaStreamSynchronize(c->st));
+  hot::SubTile *nsub = nullptr, *ntsub = nullptr;
+  int *nfirst = nullptr;
+  if (rc == HOT_OK) rc = upload(&nsub, sub);
+  if (rc == HOT_OK) rc = upload(&nfirst, first);
+  if (rc == HOT_OK && tile) rc = upload(&ntsub, cut.tiles);
+  if (rc == HOT_OK && once && !c->ubuf) rc = dalloc(&c->ubuf, (size_t)c->W * c->H);
+  if (rc != HOT_OK) {
+    dfree(nsub);
+    dfree(nfirst);
+    dfree(ntsub);
+    return rc;
+  }
+  drop_graphs(c);  // graphs hold the old schedule
   dfree(c->sub);
   dfree(c->first);
-  c->grid = 0;
-  c->n_sub = 0;
-  rc = dalloc(&c->sub, sub.size());
-  if (rc == HOT_OK) rc = dalloc(&c->first, first.size());
-  if (rc != HOT_OK) return rc;
-  HOT_CUDA(cudaMemcpy(c->sub, sub.data(), sizeof(hot::SubTile) * sub.size(), cudaMemcpyHostToDevice));
-  HOT_CUDA(cudaMemcpy(c->first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+  dfree(c->tsub);
+  c->sub = nsub;
+  c->first = nfirst;
+  c->tsub = ntsub;
+  c->sched_bps_max = bps_max;
+  c->sched_bps = per_sm;
+  c->groups = groups;
   c->grid = G;
   c->n_sub = (int)sub.size();
-  return build_tile_schedule(c, sms);
+  c->once = once;
+  c->tgrid = tile ? cut.grid : 0;
+  c->tteam = cut.team;
+  c->tpairs = cut.pairs;
+  c->tstride = cut.stride;
+  return HOT_OK;
 }
 
 // One step-kernel launch (launch k of the sequence): weight update + back-projection and/or
@@ -642,6 +656,7 @@ int launch_build_tables(hot_ctx *c) {
     if (e != cudaSuccess) rc = fail(HOT_ECUDA, "rebuilding the tensor-core operands: %s", cudaGetErrorString(e));
     c->launches++;
   }
+  if (rc == HOT_OK) c->unbuilt = false;
   return rc;
 }
 
@@ -649,8 +664,8 @@ int launch_build_tables(hot_ctx *c) {
 // Yb) start 16-byte aligned.
 int shifted_rows(const hot_ctx *c) { return (c->H + 18 + 3) & ~3; }
 
-// Allocates the direct kernels' tables for M traps, once.  *added: set when there are new ones (to be built).
-int alloc_direct_tables(hot_ctx *c, int M, bool *added) {
+// Allocates the direct kernels' tables for M traps, once (c->unbuilt: to be built).
+int alloc_direct_tables(hot_ctx *c, int M) {
   if (c->Y4r) return HOT_OK;
   c->ldy4 = shifted_rows(c);
   const size_t n4 = 4 * (size_t)M * c->ldy4;
@@ -672,12 +687,12 @@ int alloc_direct_tables(hot_ctx *c, int M, bool *added) {
     dfree(c->Y4r);
     return rc;
   }
-  *added = true;
+  c->unbuilt = true;
   return HOT_OK;
 }
 
 // The same for the complex tables of a separable batch's member.
-int alloc_batch_tables(hot_ctx *c, bool *added) {
+int alloc_batch_tables(hot_ctx *c) {
   if (c->Yb) return HOT_OK;
   c->ldy4 = shifted_rows(c);
   const size_t n2 = 2 * (size_t)c->M * c->ldy4;
@@ -690,16 +705,15 @@ int alloc_batch_tables(hot_ctx *c, bool *added) {
     dfree(c->Yb);
     return rc;
   }
-  *added = true;
+  c->unbuilt = true;
   return HOT_OK;
 }
 
 // Allocates the tables that only the direct kernels or only the tensor mode read, once the context
-// is in such a mode.  *added: whether there are new ones (to be built).
-int alloc_mode_tables(hot_ctx *c, int M, bool *added) {
+// is in such a mode.
+int alloc_mode_tables(hot_ctx *c, int M) {
   int rc = HOT_OK;
-  *added = false;
-  if (!tile_kernels(c)) rc = alloc_direct_tables(c, M, added);
+  if (!tile_kernels(c)) rc = alloc_direct_tables(c, M);
   if (rc == HOT_OK && c->precision == HOT_PREC_TENSOR && !c->Yc) {
     rc = dalloc(&c->Xc, (size_t)M * c->W);
     if (rc == HOT_OK) rc = dalloc(&c->Yc, (size_t)M * c->H);
@@ -707,18 +721,31 @@ int alloc_mode_tables(hot_ctx *c, int M, bool *added) {
       dfree(c->Xc);
       return rc;
     }
-    *added = true;
+    c->unbuilt = true;
   }
   return rc;
 }
 
-// After a change of the mode: its schedule (resched) and its tables.
-int enter_mode(hot_ctx *c, bool resched) {
-  if (!c->M) return HOT_OK;
-  bool added = false;
-  int rc = resched ? build_schedule(c) : HOT_OK;
-  if (rc == HOT_OK) rc = alloc_mode_tables(c, c->M, &added);
-  return rc == HOT_OK && added ? launch_build_tables(c) : rc;
+// Brings the context into a mode: its tables, its schedule (resched).  On failure the context stays in the
+// mode it was in; tables that it has by then are kept.
+int enter_mode(hot_ctx *c, int precision, bool once_req, bool resched) {
+  const int precision0 = c->precision;
+  const bool once_req0 = c->once_req;
+  c->precision = precision;
+  c->once_req = once_req;
+  int rc = HOT_OK;
+  if (c->M) {
+    rc = alloc_mode_tables(c, c->M);
+    if (rc == HOT_OK && c->unbuilt) rc = launch_build_tables(c);
+    if (rc == HOT_OK && resched) rc = build_schedule(c);
+  }
+  if (rc != HOT_OK) {
+    c->precision = precision0;
+    c->once_req = once_req0;
+    return rc;
+  }
+  c->u_valid = false;
+  return HOT_OK;
 }
 
 // The tensor-core plan of the context's traps (HOT_PREC_TENSOR), built on first use.
@@ -938,6 +965,10 @@ extern "C" {
 
 const char *hot_last_error(void) { return g_err; }
 
+// Test seam, not part of the interface: the calling thread's nth device allocation from now on is refused
+// with HOT_ENOMEM, once (0: none).
+void hot_test_refuse_alloc(int nth) { g_refuse = nth; }
+
 int hot_create(hot_ctx **out, int width, int height, double pitch_m, double wavelength_m,
                double focal_m, void *cuda_stream) {
   g_err[0] = 0;
@@ -1032,8 +1063,7 @@ int hot_set_traps(hot_ctx *c, int M, const double *xyz_m, const double *w0) {
       c->ev_in = nullptr;
       rc = fail(HOT_ECUDA, "hot_set_traps: cudaEventCreate failed");
     }
-    bool added;
-    if (rc == HOT_OK) rc = alloc_mode_tables(c, M, &added);
+    if (rc == HOT_OK) rc = alloc_mode_tables(c, M);
     // the tile kernels' tables, zero past the image: whole strips, whole trap pairs, row pairs read
     // kTilePairs at a time
     const size_t nx = (size_t)((c->W + hot::kTileCols - 1) / hot::kTileCols) * hot::kTileCols;
@@ -1109,9 +1139,7 @@ int hot_set_precision(hot_ctx *c, int precision) {
   const bool resched = was_sep != (precision == HOT_PREC_SEPARABLE || precision == HOT_PREC_TENSOR);
   const bool copies_change = (precision == HOT_PREC_TENSOR) != (c->precision == HOT_PREC_TENSOR);
   if (resched || copies_change) HOT_CUDA(cudaStreamSynchronize(c->st));
-  c->precision = precision;
-  c->u_valid = false;
-  return enter_mode(c, resched);  // (the kernels' occupancies differ)
+  return enter_mode(c, precision, c->once_req, resched);  // (the kernels' occupancies differ)
 }
 
 int hot_gsw(hot_ctx *c, int iters, double *eff_out, double *unif_out) {
@@ -1727,11 +1755,9 @@ int build_group(hot_batch *b, hot_batch::Group &g) {
 
 // The tables that the batched kernel reads, where the member does not have them yet.
 int batch_tables(const hot_batch *b, hot_ctx *c) {
-  bool added = false;
-  int rc = b->precision == HOT_PREC_SEPARABLE ? alloc_batch_tables(c, &added) : alloc_direct_tables(c, c->M, &added);
-  if (rc == HOT_OK && added) rc = launch_build_tables(c);
-  if (rc == HOT_OK && added) HOT_CUDA(cudaStreamSynchronize(c->st));
-  return rc;
+  const int rc = b->precision == HOT_PREC_SEPARABLE ? alloc_batch_tables(c) : alloc_direct_tables(c, c->M);
+  if (rc != HOT_OK || !c->unbuilt) return rc;
+  return launch_build_tables(c);  // (on the member's stream, behind which a run starts)
 }
 
 // Orders the holograms by pairs per iteration (smallest first, stable), cuts them into
@@ -2065,11 +2091,17 @@ int hot_set_tiling(hot_ctx *c, int rows, int blocks_per_sm, int chunk) {
   int rc = check_tiling("hot_set_tiling", rows, blocks_per_sm, chunk);
   if (rc != HOT_OK) return rc;
   HOT_CUDA(cudaStreamSynchronize(c->st));
+  const int rows0 = c->tile_rows, bps0 = c->tile_bps, chunk0 = c->tile_chunk;
   c->tile_rows = rows ? rows : hot::kRowsMax;
   c->tile_bps = blocks_per_sm;
   c->tile_chunk = chunk ? chunk : hot::kChunk;
-  drop_graphs(c);
-  return c->M ? build_schedule(c) : HOT_OK;
+  rc = c->M ? build_schedule(c) : HOT_OK;
+  if (rc != HOT_OK) {
+    c->tile_rows = rows0;
+    c->tile_bps = bps0;
+    c->tile_chunk = chunk0;
+  }
+  return rc;
 }
 
 int hot_get_tiling(const hot_ctx *c, int *rows, int *blocks_per_sm, int *chunk) {
@@ -2084,9 +2116,11 @@ int hot_set_block_merge(hot_ctx *c, int merge) {
   if (!c) return fail(HOT_EINVAL, "hot_set_block_merge: NULL context");
   if (merge != 1 && merge != 2 && merge != 4) return fail(HOT_EINVAL, "hot_set_block_merge: merge = %d is not 1, 2 or 4", merge);
   HOT_CUDA(cudaStreamSynchronize(c->st));
+  const int merge0 = c->tile_merge;
   c->tile_merge = merge;
-  drop_graphs(c);
-  return c->M ? build_schedule(c) : HOT_OK;
+  const int rc = c->M ? build_schedule(c) : HOT_OK;
+  if (rc != HOT_OK) c->tile_merge = merge0;
+  return rc;
 }
 
 int hot_get_block_merge(const hot_ctx *c, int *requested, int *in_effect) {
@@ -2100,10 +2134,7 @@ int hot_set_once(hot_ctx *c, int on) {
   if (!c) return fail(HOT_EINVAL, "hot_set_once: NULL context");
   if (on != 0 && on != 1) return fail(HOT_EINVAL, "hot_set_once: on = %d is not 0 or 1", on);
   HOT_CUDA(cudaStreamSynchronize(c->st));
-  c->once_req = on != 0;
-  c->u_valid = false;
-  drop_graphs(c);
-  return enter_mode(c, true);
+  return enter_mode(c, c->precision, on != 0, true);
 }
 
 int hot_get_once(const hot_ctx *c, int *requested, int *in_effect) {
@@ -2148,8 +2179,8 @@ int hot_autotune(hot_ctx *c, int iters, int *rows, int *blocks_per_sm, int *chun
     if (rc == HOT_OK && tile && tile_us < best_us) {
       rc = hot_set_once(c, 1);
       best_us = tile_us;
-    } else if (rc != HOT_OK) {
-      c->once_req = once_req;
+    } else if (rc != HOT_OK && c->once_req != once_req) {
+      hot_set_once(c, once_req ? 1 : 0);  // back to the kernels it had; the first error is reported
     }
   }
   c->profiling = profiling;
