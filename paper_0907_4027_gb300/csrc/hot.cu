@@ -1457,6 +1457,7 @@ int hot_use_persistent(hot_ctx *c, int enable) {
 int hot_set_wait_limit(hot_ctx *c, double seconds) {
   if (!c) return fail(HOT_EINVAL, "hot_set_wait_limit: NULL context");
   if (!(seconds >= 0.0) || seconds > 60.0) return fail(HOT_EINVAL, "hot_set_wait_limit: %g s not in [0, 60]", seconds);
+  if (seconds != c->wait_limit_s) drop_graphs(c);  // the tensor-core launches carry the limit
   c->wait_limit_s = seconds;
   return HOT_OK;
 }
@@ -1539,12 +1540,20 @@ struct hot_batch {
 
   struct Graph {
     int iters;
+    std::vector<double> limits;  // HOT_PREC_TENSOR: the members' wait limits, which the launches carry
     cudaGraphExec_t exec;
   };
   std::vector<Graph> graphs;
 };
 
 namespace {
+
+std::vector<double> batch_limits(const hot_batch *b) {
+  std::vector<double> v;
+  if (b->precision == HOT_PREC_TENSOR)
+    for (const hot_ctx *c : b->ctx) v.push_back(c->wait_limit_s);
+  return v;
+}
 
 int batch_mode(const hot_batch *b) {
   return b->precision == HOT_PREC_SEPARABLE ? hot::kModeSeparable
@@ -2265,8 +2274,9 @@ int hot_batch_get_tiling(const hot_batch *b, int *rows, int *blocks_per_sm, int 
 int hot_batch_gsw(hot_batch *b, int iters) {
   if (!b) return fail(HOT_EINVAL, "hot_batch_gsw: NULL batch");
   if (iters < 0) return fail(HOT_EINVAL, "hot_batch_gsw: iters = %d < 0", iters);
+  const std::vector<double> limits = batch_limits(b);
   for (auto &g : b->graphs)
-    if (g.iters == iters) {
+    if (g.iters == iters && g.limits == limits) {
       const int rc = batch_after_members(b);
       if (rc != HOT_OK) return rc;
       HOT_CUDA(cudaGraphLaunch(g.exec, b->st));
@@ -2298,7 +2308,7 @@ int hot_batch_gsw(hot_batch *b, int iters) {
   e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return fail(HOT_ECUDA, "hot_batch_gsw: graph instantiation: %s", cudaGetErrorString(e));
-  b->graphs.push_back({iters, exec});
+  b->graphs.push_back({iters, limits, exec});
   rc = batch_after_members(b);
   if (rc != HOT_OK) return rc;
   HOT_CUDA(cudaGraphLaunch(exec, b->st));

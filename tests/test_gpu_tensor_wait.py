@@ -90,3 +90,24 @@ def test_replayed_capture_timeout(hot, read):
         g.replay()
         with pytest.raises(hot.HotError, match="HOT_ETIMEOUT"):
             getattr(h, read)()
+
+
+@pytest.mark.parametrize("batch", [False, True])
+def test_a_new_limit_reaches_calls_that_were_captured_before(hot, batch):
+    """Among 50 runs of a graph's sequence with a limit of zero at least one wait runs out (each has some
+    thousand waits for copies from memory)."""
+    w = wl.random_case(1024, 1024, 1000, seed=3, precision="tensor")
+    with hot.Hologram.from_workload(w) as h, hot.Batch([h]) as b:
+        run = (lambda: b.gsw(2)) if batch else (lambda: h.gsw(2, metrics=False))
+        run()
+        h.sync()
+        h.set_wait_limit(0.0)
+        with pytest.raises(hot.HotError, match="HOT_ETIMEOUT"):
+            for _ in range(50):
+                run()
+                h.sync()
+        h.set_wait_limit(2.0)
+        h.set_phase(w.phi0)
+        h.set_weights(np.ones(w.M))
+        run()
+        h.sync()
