@@ -10,7 +10,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libhot.so")
 SOURCES = [os.path.join(CSRC, f) for f in ("hot.cu", "tc.cu", "tile.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("gsw_kernels.cuh", "batch_kernels.cuh", "tile_kernels.cuh", "tc_kernels.cuh", "tc.h", "tile.h")] + \
+DEPS = SOURCES + [os.path.join(CSRC, f) for f in ("gsw_kernels.cuh", "batch_kernels.cuh", "tile_kernels.cuh", "turns.cuh", "tc_kernels.cuh", "tc.h", "tile.h")] + \
     [os.path.join(ROOT, "include", "hot.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -23,6 +23,7 @@
 // shared memory (cp.async), so no barrier stands in the trap loops.
 #pragma once
 #include "gsw_kernels.cuh"
+#include "turns.cuh"
 
 namespace hot {
 
@@ -553,65 +554,7 @@ static __global__ void __launch_bounds__(kThreads, 2) gsw_tile_persistent_kernel
 }
 
 // ---------------------------------------------------------------------------------------------
-// Tables of the column and row phasors (once per trap set).
-//
-// A phase modulo one turn is a 64-bit fraction of a turn: a q and c q^2 (Eq. 2 per pixel index q) are
-// integer products that drop whole turns by themselves, exact to 2^-64 |q| turns.  cos and sin of it:
-// reduced to an eighth of a turn, Taylor series in the squared quarter turns, the leading
-// coefficients and products in float-float (Dekker, Knuth), rounded once: within 0.51 ulp.  No FP64
-// arithmetic: GB300 does ~2 FP64 operations per clock and SM, and FP64 sincospi made these tables
-// 20 us of a 657 us frame at 512^2 with 100 traps and 230 us at 1920 x 1152 with 1000.
-
-// |x| as a fixed-point number of fractions 2^-64, modulo 1 (truncated).
-__device__ __forceinline__ unsigned long long turns_fixed(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int sh = (int)((b >> 52) & 0x7ff) - 1011;  // x = m 2^(sh - 64)
-  const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
-  return sh >= 64 || sh <= -64 ? 0ull : sh >= 0 ? m << sh : m >> -sh;
-}
-
-struct TrapTurns {
-  unsigned long long a, c, cl;  // linear and quadratic turns per pixel index; cl: the next bits of |c|
-  bool neg;                     // c < 0
-  __device__ __forceinline__ TrapTurns(double lin, double quad) {
-    a = turns_fixed(lin);
-    if (lin < 0.0) a = 0ull - a;
-    c = turns_fixed(quad);
-    cl = turns_fixed(quad * 4294967296.0) << 32;  // (2^32: exact)
-    neg = quad < 0.0;
-  }
-  __device__ __forceinline__ unsigned long long phase(int q) const {
-    const unsigned long long q2 = (unsigned long long)((long long)q * q);
-    const unsigned long long t = c * q2 + __umul64hi(cl, q2);
-    return a * (unsigned long long)(long long)q + (neg ? 0ull - t : t);
-  }
-};
-
-// cos and sin of a phase in fractions 2^-64 of a turn.
-__device__ __forceinline__ float2 cis_turns(unsigned long long ph) {
-  const unsigned n = (unsigned)((ph + (1ull << 61)) >> 62);  // quarter turns
-  const long long r = (long long)(ph - ((unsigned long long)n << 62));
-  // the rest in quarter turns, [-1/2, 1/2]: f + g
-  const float f = (float)(int)(r >> 38) * 0x1p-24f, g = (float)(int)((r >> 14) & 0xffffff) * 0x1p-48f;
-  const float sh = __fmul_rn(f, f), sl = fmaf(f, f, -sh) + 2.f * f * g;
-  // sine: (f + g) (s0 + s (s1 + s p)), s_k = (-1)^k (pi/2)^(2k+1) / (2k+1)!
-  float t = sh * fmaf(sh, fmaf(sh, fmaf(sh, -3.59884325e-06f, 1.60441181e-04f), -4.68175393e-03f), 7.96926245e-02f);
-  float qh = __fadd_rn(-0.645964086f, t), ql = __fadd_rn(__fsub_rn(-0.645964086f, qh), t) - 1.14504903e-08f;
-  float ph_ = __fmul_rn(sh, qh), pl = fmaf(sh, qh, -ph_) + fmaf(sh, ql, sl * qh);
-  float vh = __fadd_rn(1.57079637f, ph_), vl = __fadd_rn(__fsub_rn(1.57079637f, vh), ph_) + (pl - 4.37113883e-08f);
-  const float sn = fmaf(f, vh, fmaf(f, vl, g * vh));
-  // cosine: 1 + s (c1 + s p), c_k = (-1)^k (pi/2)^(2k) / (2k)!
-  t = sh * fmaf(sh, fmaf(sh, fmaf(sh, -2.52020418e-05f, 9.19260259e-04f), -2.08634809e-02f), 0.2536695f);
-  qh = __fadd_rn(-1.23370051f, t);
-  ql = __fadd_rn(__fsub_rn(-1.23370051f, qh), t) - 3.62964485e-08f;
-  ph_ = __fmul_rn(sh, qh);
-  pl = fmaf(sh, qh, -ph_) + fmaf(sh, ql, sl * qh);
-  vh = __fadd_rn(1.f, ph_);
-  vl = __fadd_rn(__fsub_rn(1.f, vh), ph_) + pl;
-  const float co = vh + vl;
-  const float x = n & 1 ? sn : co, y = n & 1 ? co : sn;
-  return make_float2(n == 1 || n == 2 ? -x : x, n >= 2 ? -y : y);
-}
+// Tables of the column and row phasors (once per trap set), from the phases of turns.cuh.
 
 struct TileTables {
   int W, H, H_total, y_off;  // a row band: rows y_off .. of a hologram of H_total rows
@@ -627,16 +570,16 @@ static __global__ void __launch_bounds__(128) tile_tables_kernel(TileTables t) {
   const int m = blockIdx.y, j = blockIdx.x * 128 + threadIdx.x, P = (t.H + 1) / 2;
   if (j >= t.W + P) return;
   const bool col = j < t.W;
-  const TrapTurns k(t.abc[3 * m + (col ? 0 : 1)], t.abc[3 * m + 2]);
+  const TrapTurns k = trap_turns(t.abc[3 * m + (col ? 0 : 1)], t.abc[3 * m + 2]);
   if (col) {
-    const float2 e = cis_turns(k.phase(j - t.W / 2));
+    const float2 e = cis_turns(phase_at(k, j - t.W / 2));
     t.X[((size_t)(j / kTileCols) * t.Mp + m) * kTileCols + j % kTileCols] = e;
     if (t.Xc) t.Xc[(size_t)m * t.W + j] = e;
     return;
   }
   const int p = j - t.W, q = 2 * p + t.y_off - t.H_total / 2;
   const bool two = 2 * p + 1 < t.H;
-  const float2 e = cis_turns(k.phase(q)), f = two ? cis_turns(k.phase(q + 1)) : make_float2(0.f, 0.f);
+  const float2 e = cis_turns(phase_at(k, q)), f = two ? cis_turns(phase_at(k, q + 1)) : make_float2(0.f, 0.f);
   t.Y[(size_t)m * t.ldp + p] = make_float4(e.x, f.x, e.y, f.y);
   if (t.Yc) {
     t.Yc[(size_t)m * t.H + 2 * p] = e;
