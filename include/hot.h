@@ -272,14 +272,16 @@ int hot_sharded_end(hot_ctx *c, int iters, double *eff_out, double *unif_out);
 int hot_get_metrics(hot_ctx *c, double *eff_out, double *unif_out);
 
 /* ---- tiling and autotuning ----------------------------------------------------------------
- * The step kernels give every thread one pixel column of a sub-tile of `rows` rows
+ * The direct kernels (hot_set_once(c, 0)) and the batches' give every thread one pixel column of a
+ * sub-tile of `rows` rows
  * (1..14: pixels per thread), run `blocks_per_sm` resident blocks of 256 threads per SM
  * (1..4; the grid is one wave of SMs x blocks_per_sm persistent blocks) and stage the trap
  * tables in shared memory `chunk` traps at a time (1..128).  The results do not depend on the
- * tiling beyond FP32 rounding of the per-pixel sums.  Defaults: 14, as many as fit, 128. */
+ * tiling beyond FP32 rounding of the per-pixel sums.  Defaults: 14, as many as fit, 128.  A context's
+ * register-tiled and tensor-core kernels choose their own tiles. */
 
-/* Sets the tiling (0 selects a parameter's default) and rebuilds the work schedule.
- * Synchronises the context's stream.  HOT_EINVAL out of range. */
+/* Sets the tiling (0 selects a parameter's default) and rebuilds the work schedule; the tiling stays
+ * as it was where that fails.  Synchronises the context's stream.  HOT_EINVAL out of range. */
 int hot_set_tiling(hot_ctx *c, int rows, int blocks_per_sm, int chunk);
 
 /* The tiling in effect (blocks_per_sm as launched).  Any output pointer may be NULL. */
@@ -311,7 +313,9 @@ int hot_get_block_merge(const hot_ctx *c, int *requested, int *in_effect);
  * launch of a call, which keeps u_j; a call that continues from the phases of the previous one
  * starts from them (hot_get_phasors), so that resumed sequences, CUDA graphs and the persistent
  * form give the same bits.  With more traps u_j is e^{i phi_j} of the stored phases.
- * on: 1 or 0, else HOT_EINVAL.  Rebuilds the schedule; synchronises the context's stream.
+ * on: 1 or 0, else HOT_EINVAL.  Rebuilds the schedule and, the first time, builds the direct kernels'
+ * tables, which the context then keeps up with its traps; the kernels stay as they were where that fails
+ * (HOT_ENOMEM).  Synchronises the context's stream.
  * hot_get_once reports the setting and whether the unit phasors are in effect (M <= 128, mode
  * HOT_PREC_ACCURATE or HOT_PREC_FAST). */
 int hot_set_once(hot_ctx *c, int on);

@@ -11,7 +11,8 @@
 // buffers (read, written, cleared) and weights over two.  No FP64 runs per iteration.
 //
 // This file holds the direct step kernels (hot_set_once(c, 0)) and what every mode shares; the
-// register-tiled kernels of the accurate, fast and separable modes are in tile_kernels.cuh.
+// register-tiled kernels of the accurate, fast and separable modes are in tile_kernels.cuh, the batched
+// kernel in batch_kernels.cuh.
 // Per pair the direct kernels take exactly one complex exponential and accumulate it without a
 // complex multiply: the back-projection folds the phase of its coefficient into the argument,
 // S_j += w_m e^{i (Delta_j^m + arg V_m)}, and the forward field evaluates Eq. 1 as written,
@@ -886,7 +887,7 @@ static __global__ void __launch_bounds__(kLossThreads) intensity_loss_kernel(Los
   __shared__ double part[3][kLossThreads / 32];
   __shared__ int exps[kLossThreads / 32];
   __shared__ float ext[2][kLossThreads / 32];
-  __shared__ double total[3];  // sum I, sum log I, sum (I - mean)^2
+  __shared__ double total[2];  // sum I, sum log I
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int nw = min(kLossThreads / 32, (a.M + 31) / 32);  // warps that hold traps
   allow_dependents();

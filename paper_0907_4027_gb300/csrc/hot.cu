@@ -87,7 +87,6 @@ struct hot_ctx {
   int grid = 0, n_sub = 0;
   hot::SubTile *sub = nullptr;  // [n_sub]
   int *first = nullptr;         // [grid + 1]
-  int sched_smem_M = -1;        // M the schedule's occupancy was computed for
   // tiling (hot_set_tiling): rows per sub-tile (pixels per thread), resident blocks per SM
   // (0: as many as fit), traps per staged chunk
   int tile_rows = hot::kRowsMax, tile_bps = 0, tile_chunk = hot::kChunk;
@@ -455,8 +454,8 @@ void cut_schedule(int W, int H, int G, int rows, std::vector<hot::SubTile> &sub,
 // superpositions, phasors).  Measured us per iteration with 1 / 2 / 4 / 8 warps (the model's
 // choice in brackets): 256^2, M = 16 7.9 / 5.9 / 4.9 / [4.9]; 768^2, M = 8 8.3 / [8.5] / 9.4 / 12.3;
 // 801 x 603, M = 37 25 / 17.3 / [15.5] / 17.4; 768^2, M = 100 56 / 39 / [32] / 35; 512^2, M = 100
-// 40 / 24 / 17.4 / [15.9]; 1920 x 1152, M = 100 [103] / 98 / 101 / 107.  At most 128 traps are added
-// in a row (FP32 rounding of S_j).
+// 40 / 24 / 17.4 / [15.9]; 1920 x 1152, M = 100 [103] / 98 / 101 / 107.  Up to 1024
+// traps at most 128 are added in a row (FP32 rounding of S_j), above that an eighth of them.
 int tile_team(int M, long long row_pairs, int sms) {
   int best = hot::kWarps;
   double best_cost = 1e300;

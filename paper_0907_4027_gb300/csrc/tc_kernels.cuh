@@ -302,15 +302,6 @@ __device__ __forceinline__ void store1(void *base, size_t i, float v) {
   else
     static_cast<float *>(base)[i] = v;
 }
-// Elements i, i + 1 (i even).
-template <int OP>
-__device__ __forceinline__ void store2(void *base, size_t i, float a, float b) {
-  if (OP == kOpF16)
-    *reinterpret_cast<__half2 *>(static_cast<__half *>(base) + i) = __floats2half2_rn(a, b);
-  else
-    *reinterpret_cast<float2 *>(static_cast<float *>(base) + i) = make_float2(a, b);
-}
-
 // u = e^{i phi} of a phase in any range: reduced to [-pi, pi] (Cody-Waite with 2 pi split in
 // two floats; a no-op for the back-projection's own phases in (-pi, pi]), then the SFU's
 // sin/cos approximations (|error| ~ 4e-7 on that interval).  The forward operand of the phases
