@@ -785,8 +785,9 @@ def run_precision_report(args):
 
 def run_batch(args):
     """Batched form (batch64): 64 holograms, sizes from {512^2, 1024^2, 1920x1152}, M ~ U{8..2000},
-    30 GSW iterations per hologram in one CUDA graph, in the fast direct mode (shortest-first
-    groups, one launch per group and iteration, autotuned tiling) and in the tensor mode (each
+    30 GSW iterations per hologram in one CUDA graph, in the fast mode (shortest-first
+    groups, one launch per group and iteration, autotuned tiling; also a group per hologram, on the
+    step of each one's own hot_gsw) and in the tensor mode (each
     member's own launch sequence on 8 concurrent chains); --precision picks one mode.
     Holograms/s and per-hologram latency (device timer stamps from the start of the graph to each
     hologram's completion), beside the same holograms run one by one through hot_gsw in the same
@@ -819,20 +820,27 @@ def run_batch(args):
         t_tune = time.perf_counter() - t_tune
         tiling = batch.tiling()
         reps = max(1, min(args.steps, 5))
-        total, lats = [], []
-        for i in range(reps + 1):
-            reset()
-            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
-            ev[0].record(stream)
-            batch.gsw(K)
-            ev[1].record(stream)
-            torch.cuda.synchronize()
-            if i:  # i = 0: graph capture and warm-up
-                total.append(ev[0].elapsed_time(ev[1]))
-                lats.append(batch.latency())
-        batch_ms = float(np.median(total))
-        lat = np.concatenate(lats)
+
+        def timed_batch():
+            total, lats = [], []
+            for i in range(reps + 1):
+                reset()
+                ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+                ev[0].record(stream)
+                batch.gsw(K)
+                ev[1].record(stream)
+                torch.cuda.synchronize()
+                if i:  # i = 0: graph capture and warm-up
+                    total.append(ev[0].elapsed_time(ev[1]))
+                    lats.append(batch.latency())
+            return float(np.median(total)), np.concatenate(lats)
+
+        batch_ms, lat = timed_batch()
         eu_batch = batch.metrics()
+        own = None
+        if mode != "tensor":  # a group per hologram: each member's own hot_gsw step
+            batch.set_tiling(group_pairs=1.0)
+            own = timed_batch()
         batch.close()
         # the same holograms one by one (each its own hot_gsw graph, default tiling), in the given order
         for h in holos:
@@ -856,6 +864,9 @@ def run_batch(args):
                       "latency_ms_p99": float(np.percentile(lat, 99)),
                       "tiling": tiling,
                       "autotune": dict(tuned, seconds=t_tune, iters=2) if tuned else None},
+            **({"batch_group_per_hologram": {"holograms_per_s": len(ws) / (own[0] * 1e-3), "ms": own[0],
+                                             "latency_ms_p50": float(np.percentile(own[1], 50)),
+                                             "latency_ms_p99": float(np.percentile(own[1], 99))}} if own else {}),
             "sequential": {"holograms_per_s": len(ws) / (seq_lat[-1] * 1e-3), "ms": float(seq_lat[-1]),
                            "updates_per_s": pairs / (seq_lat[-1] * 1e-3),
                            "latency_ms_p50": float(np.percentile(seq_lat, 50)),
